@@ -106,6 +106,7 @@ void free_all(mm_ctx* ctx) {
         if (p) cudaFree(p);
     for (void* p : ctx->k)
         if (p) cudaFree(p);
+    plane_free(ctx);
     if (ctx->ctl_host) cudaFreeHost(ctx->ctl_host);
     free(ctx->newell_host);
     for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
@@ -142,7 +143,9 @@ int make_tables(mm_ctx* ctx) {
     return MM_OK;
 }
 
-int alloc(mm_ctx* ctx, void** p, size_t bytes) {
+}  // namespace
+
+int dev_alloc(mm_ctx* ctx, void** p, size_t bytes) {
     cudaError_t e = cudaMalloc(p, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -152,6 +155,8 @@ int alloc(mm_ctx* ctx, void** p, size_t bytes) {
     }
     return MM_OK;
 }
+
+namespace {
 
 int push_ctl(mm_ctx* ctx) {
     MM_CUDA_CHECK(ctx, cudaMemcpyAsync(ctx->ctl, ctx->ctl_host, sizeof(Control), cudaMemcpyHostToDevice, ctx->stream));
@@ -279,11 +284,8 @@ int mm_init_mesh(mm_ctx** out, int nx, int ny, int nz, double dx, double dy, dou
     const size_t v3 = 3 * (size_t)ctx->N * e;
     int rc = MM_OK;
     auto A = [&](void** p, size_t b) {
-        if (rc == MM_OK) rc = alloc(ctx, p, b);
+        if (rc == MM_OK) rc = dev_alloc(ctx, p, b);
     };
-    A(&ctx->kern, 6 * (size_t)ctx->Pz2 * ctx->Py2 * ctx->Hs * e);
-    A(&ctx->bufA, 3 * (size_t)nz * ny * ctx->Hs * 2 * e);
-    A(&ctx->bufB, 3 * (size_t)nz * ctx->Py * ctx->Hs * 2 * e);
     A(&ctx->Hd, v3);
     A(&ctx->Hs_field, v3);
     A(&ctx->ms[0], v3);
@@ -307,12 +309,16 @@ int mm_init_mesh(mm_ctx** out, int nx, int ny, int nz, double dx, double dy, dou
         if (ce != cudaSuccess) rc = fail(ctx, MM_ERR_CUDA, "cudaMemcpy: %s", cudaGetErrorString(ce));
     }
     if (rc == MM_OK) rc = make_tables(ctx);
-    if (rc == MM_OK) rc = blue_prepare(ctx);
     if (rc == MM_OK) {
         reset_ctl(ctx->ctl_host, 0.0, 1e-14, std::numeric_limits<double>::infinity(), 1e-5);
         rc = push_ctl(ctx);
     }
-    if (rc == MM_OK) rc = demag_setup(ctx);
+    // meshes with a side that is not a power of two need the octant of the
+    // 2n lengths only in the fft modes and for mm_kspace_product
+    auto p2 = [](int n) { return (n & (n - 1)) == 0; };
+    if (rc == MM_OK) rc = plane_plan(ctx);
+    if (rc == MM_OK && (!ctx->plane.on || (p2(nx) && p2(ny)))) rc = classic_prepare(ctx);
+    if (rc == MM_OK && ctx->plane.on) rc = plane_setup(ctx);
     if (rc == MM_OK) rc = sync(ctx);
     if (rc != MM_OK) {
         g_init_error = ctx->err;
@@ -437,7 +443,7 @@ int mm_llg_step_host(mm_ctx* ctx, void* m_host, double* t, double* dt, int metho
     if (!m_host) return fail(ctx, MM_ERR_INVALID_ARG, "m_host must not be NULL");
     const size_t bytes = 3 * (size_t)ctx->N * elem(ctx);
     int rc;
-    if (!ctx->m_stage && (rc = alloc(ctx, &ctx->m_stage, bytes))) return rc;
+    if (!ctx->m_stage && (rc = dev_alloc(ctx, &ctx->m_stage, bytes))) return rc;
     MM_CUDA_CHECK(ctx, cudaMemcpyAsync(ctx->m_stage, m_host, bytes, cudaMemcpyHostToDevice, ctx->stream));
     if ((rc = mm_llg_step(ctx, ctx->m_stage, t, dt, method, tol, err_out))) return rc;
     MM_CUDA_CHECK(ctx, cudaMemcpyAsync(m_host, ctx->m_stage, bytes, cudaMemcpyDeviceToHost, ctx->stream));

@@ -1923,7 +1923,9 @@ __global__ void k_split_ff(const double* __restrict__ in, ff* __restrict__ out, 
 
 // Prepares MM_FFT_FF on an FP64 context: float-float copies of the octant
 // and of the twiddle tables (kept until the context is destroyed).
+bool plane_ff_fits(const mm_ctx* ctx);
 int demag_prepare_ff(mm_ctx* ctx) {
+    if (plane_ff_fits(ctx)) return plane_prepare_ff(ctx);
     if (ctx->kern_ff && ctx->tw.ff) return MM_OK;
     const long nk = 6L * ctx->Pz2 * ctx->Py2 * ctx->Hs;
     const long nt = 2L * (ctx->tw.off_pz + ctx->Pz);          // doubles in the twiddle table
@@ -1938,6 +1940,8 @@ int demag_prepare_ff(mm_ctx* ctx) {
 }
 
 int demag_kspace_product(mm_ctx* ctx, void* spec) {
+    int rc = classic_prepare(ctx);
+    if (rc) return rc;
     const long n = (long)ctx->Pz * ctx->Py * ctx->Hx;
     const unsigned blocks = (unsigned)((n + 255) / 256);
     if (ctx->prec == MM_F64)
@@ -1953,7 +1957,7 @@ int demag_kspace_product(mm_ctx* ctx, void* spec) {
 namespace {
 // Bluestein data of one axis (host arithmetic in long double, exact phases)
 int blue_axis(mm_ctx* ctx, int P, Blue* bl) {
-    if (P <= kBlueMin || pow2(P)) return MM_OK;
+    if (P <= kBlueMin || pow2(P) || bl->P == P) return MM_OK;
     int M = 1;
     while (M < 2 * P - 1) M *= 2;
     const long double pi = 3.141592653589793238462643383279502884L;
@@ -1997,16 +2001,14 @@ int blue_axis(mm_ctx* ctx, int P, Blue* bl) {
             filt[2 * ((size_t)d * M + k) + 1] = (double)(ai / M);
         }
     }
-    bl->P = P;
-    bl->M = M;
     auto up = [&](void** dst, const std::vector<double>& src) -> int {
-        MM_CUDA_CHECK(ctx, cudaMalloc(dst, src.size() * sizeof(double)));
+        if (!*dst) MM_CUDA_CHECK(ctx, cudaMalloc(dst, src.size() * sizeof(double)));
         MM_CUDA_CHECK(ctx, cudaMemcpy(*dst, src.data(), src.size() * sizeof(double), cudaMemcpyHostToDevice));
         return MM_OK;
     };
     auto up32 = [&](void** dst, const std::vector<double>& src) -> int {
         std::vector<float> f(src.begin(), src.end());
-        MM_CUDA_CHECK(ctx, cudaMalloc(dst, f.size() * sizeof(float)));
+        if (!*dst) MM_CUDA_CHECK(ctx, cudaMalloc(dst, f.size() * sizeof(float)));
         MM_CUDA_CHECK(ctx, cudaMemcpy(*dst, f.data(), f.size() * sizeof(float), cudaMemcpyHostToDevice));
         return MM_OK;
     };
@@ -2015,6 +2017,8 @@ int blue_axis(mm_ctx* ctx, int P, Blue* bl) {
     if (ctx->prec == MM_F32 &&
         ((rc = up32(&bl->chirp32, chirp)) || (rc = up32(&bl->filt32, filt)) || (rc = up32(&bl->tw32, tw))))
         return rc;
+    bl->M = M;
+    bl->P = P;   // set last: marks the axis as prepared
     return MM_OK;
 }
 }  // namespace
@@ -2029,7 +2033,30 @@ int demag_setup(mm_ctx* ctx) {
     return ctx->prec == MM_F64 ? setup<double>(ctx) : setup<float>(ctx);
 }
 
+int classic_prepare(mm_ctx* ctx) {
+    if (ctx->classic_ready) return MM_OK;
+    const size_t e = ctx->prec == MM_F64 ? sizeof(double) : sizeof(float);
+    int rc;
+    if (!ctx->kern && (rc = dev_alloc(ctx, &ctx->kern, 6 * (size_t)ctx->Pz2 * ctx->Py2 * ctx->Hs * e))) return rc;
+    if (!ctx->bufA && (rc = dev_alloc(ctx, &ctx->bufA, 3 * (size_t)ctx->nz * ctx->ny * ctx->Hs * 2 * e))) return rc;
+    if (!ctx->bufB && (rc = dev_alloc(ctx, &ctx->bufB, 3 * (size_t)ctx->nz * ctx->Py * ctx->Hs * 2 * e))) return rc;
+    if ((rc = blue_prepare(ctx)) || (rc = demag_setup(ctx))) return rc;
+    ctx->classic_ready = true;
+    return MM_OK;
+}
+
+bool plane_ff_fits(const mm_ctx* ctx);   // mm_plane_ff.cu
+
+namespace {
+// whether the context's current mode runs in the plane layout (the
+// tensor-core and fused modes have passes of their own)
+bool plane_runs(const mm_ctx* ctx) {
+    return ctx->plane.on && (ctx->fft_mode == 0 || (ctx->fft_mode == MM_FFT_FF && plane_ff_fits(ctx)));
+}
+}  // namespace
+
 int demag_apply(mm_ctx* ctx, const void* m, void* H) {
+    if (plane_runs(ctx)) return plane_apply(ctx, m, H, false);
     if (ctx->prec == MM_F64) {
         if (ctx->fft_mode == MM_FFT_FF) return apply_ff(ctx, (const double*)m, (double*)H, false);
         return apply<double>(ctx, (const double*)m, (double*)H);
@@ -2038,6 +2065,7 @@ int demag_apply(mm_ctx* ctx, const void* m, void* H) {
 }
 
 int demag_apply_unit(mm_ctx* ctx, const void* g, void* H) {
+    if (plane_runs(ctx)) return plane_apply(ctx, g, H, true);
     if (ctx->prec == MM_F64) {
         if (ctx->fft_mode == MM_FFT_FF) return apply_ff(ctx, (const double*)g, (double*)H, true);
         return apply<double>(ctx, (const double*)g, (double*)H, true);

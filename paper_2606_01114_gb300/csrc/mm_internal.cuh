@@ -81,6 +81,25 @@ struct Blue {
     void* tw32 = nullptr;
 };
 
+// The plane-layout demag path (mm_plane.cu).  Lengths are padded to the next
+// of {4, 5, 6, 8} 2^k >= 2n, so they differ from ctx->Px, Py when a side is
+// not a power of two.
+struct PlanePlan {
+    int on = 0;          // the plain (fft_mode 0) and float-float passes run in the plane layout
+    int lines = 0;       // planes too large for one block: y, z, y as three kernels
+    int L = 0, P = 0;    // complex x length (P_x / 2), padded y length
+    int K = 0;           // planes: L + 1 kept x frequencies
+    int KQ = 0;          // octant row stride (P / 2 + 1 rounded up to 4)
+    long R = 0;          // plane stride of buf, complex (3 nz ny rounded up to 4)
+    long off_p = 0, off_y = 0, off_z = 0;   // twiddle tables of 2L, P and Pz behind that of L
+    void* buf = nullptr;     // complex [K][R]
+    void* buf2 = nullptr;    // complex [K][3 nz][P] (lines)
+    void* kern = nullptr;    // octant [K][6][Pz/2+1][KQ], path precision
+    void* kern_ff = nullptr; // its float-float copy (MM_FFT_FF)
+    void* tw = nullptr;      // complex tables, path precision
+    void* tw_ff = nullptr;
+};
+
 }  // namespace mm
 
 struct mm_ctx {
@@ -140,6 +159,9 @@ struct mm_ctx {
     int ymap_grid[2];         // persistent grids of the TMA-fed y forward [0] and inverse [1] passes
     int xtma_state;           // TMA-fed x inverse (nx = 512): 0 not tried, 1 ready, -1 not available
     int xtma_grid;            // its persistent grid
+
+    mm::PlanePlan plane;
+    bool classic_ready;       // kern, bufA, bufB and the transform tables of the [c][z][y][kx] passes exist
 
     long launches;
     std::string err;
@@ -211,6 +233,17 @@ int tc_prepare(mm_ctx* ctx);
 
 // ----- demag (mm_demag.cu)
 int demag_setup(mm_ctx* ctx);                          // K1: Newell tensor -> k-space octant
+// kern, bufA, bufB and tables of the [c][z][y][kx] passes: at once for
+// contexts that run them, on first use for the others (fft modes,
+// mm_kspace_product)
+int classic_prepare(mm_ctx* ctx);
+// plane layout (mm_plane.cu): chooses and allocates the plan, fills its octant
+int plane_plan(mm_ctx* ctx);
+int plane_setup(mm_ctx* ctx);
+void plane_free(mm_ctx* ctx);
+int plane_apply(mm_ctx* ctx, const void* m, void* H, bool unit);
+int plane_prepare_ff(mm_ctx* ctx);
+int dev_alloc(mm_ctx* ctx, void** p, size_t bytes);
 int demag_apply(mm_ctx* ctx, const void* m, void* H);  // K2..K6
 int demag_apply_unit(mm_ctx* ctx, const void* g, void* H);  // same with Ms = 1 (adjoint)
 int demag_prepare_ff(mm_ctx* ctx);                     // float-float tables for MM_FFT_FF
@@ -228,7 +261,8 @@ cudaStream_t fno_swap_stream(mm_fno* f, cudaStream_t s);
 
 // ----- Newell (mm_newell.cu)
 // Fills the FP64 real-space padded grid [Pz][Py][Px] of component c (0..5)
-// and, when octant_out != nullptr, the octant [nz][ny][nx] of that component.
+// (skipped when grid is NULL) and, when octant_out != nullptr, the octant
+// [nz][ny][nx] of that component.
 int newell_component(mm_ctx* ctx, int c, double* grid, double* octant_out, void* fgrid_scratch);
 
 // ----- LLG and fields (mm_llg.cu)

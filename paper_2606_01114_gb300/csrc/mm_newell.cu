@@ -265,6 +265,7 @@ __global__ void k_newell_assemble(int c, int nx, int ny, int nz, int Px, int Py,
     dd val = dd_div(acc, dd_mul(dd_mul_d(kPiDD, 4.0), V));
     double v = val.hi + val.lo;
     if (octant) octant[idx] = v;
+    if (!grid) return;
     for (int sz = -1; sz <= 1; sz += 2) {
         if (sz < 0 && K == 0) continue;
         for (int sy = -1; sy <= 1; sy += 2) {
@@ -296,7 +297,8 @@ int newell_component(mm_ctx* ctx, int c, double* grid, double* octant_out, void*
     k_newell_fgrid<<<(unsigned)((gtotal + 127) / 128), 128, 0, ctx->stream>>>(c, gx, gy, gz, ctx->dx, ctx->dy,
                                                                               ctx->dz, fg);
     MM_LAUNCH_CHECK(ctx);
-    MM_CUDA_CHECK(ctx, cudaMemsetAsync(grid, 0, sizeof(double) * (size_t)ctx->Px * ctx->Py * ctx->Pz, ctx->stream));
+    if (grid)
+        MM_CUDA_CHECK(ctx, cudaMemsetAsync(grid, 0, sizeof(double) * (size_t)ctx->Px * ctx->Py * ctx->Pz, ctx->stream));
     long total = ctx->N;
     k_newell_assemble<<<(unsigned)((total + 127) / 128), 128, 0, ctx->stream>>>(
         c, ctx->nx, ctx->ny, ctx->nz, ctx->Px, ctx->Py, ctx->Pz, ctx->dx, ctx->dy, ctx->dz, fg, grid, octant_out);

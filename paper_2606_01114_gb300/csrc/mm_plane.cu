@@ -1,0 +1,258 @@
+// The plane-layout demag path: plan, octant and sequencing (the kernels and
+// their layout: mm_plane.cuh).
+#include <cmath>
+#include <vector>
+
+#include "mm_ff.cuh"
+
+namespace mm {
+
+// per element type (mm_plane_f32.cu, mm_plane_f64.cu, mm_plane_ff.cu)
+int plane_apply_f32(mm_ctx* ctx, const float* m, const float* Ms, float ms, float* H);
+int plane_apply_f64(mm_ctx* ctx, const double* m, const double* Ms, double ms, double* H);
+int plane_apply_ff(mm_ctx* ctx, const double* m, const double* Ms, double ms, double* H);
+int plane_line_len(int P);
+
+namespace {
+
+bool pow2(int n) { return n > 0 && (n & (n - 1)) == 0; }
+
+// next of 16, 32 and {4, 5, 6} 2^k, k >= 3, that is >= n
+int next_len(int n) {
+    if (n <= 16) return 16;
+    if (n <= 32) return 32;
+    for (int p = 32;; p *= 2)
+        for (int q = 4; q <= 6; ++q)
+            if (q * p / 4 >= n) return q * p / 4;
+}
+
+// One axis of the octant's transform by its definition: the Newell tensor is
+// even or odd along each axis, so its DFT over the padded length P is
+//   even: N_0 + 2 sum_j N_j cos(2 pi j k / P),  odd: 2 sum_j N_j sin(2 pi j k / P)
+// (the factors -i of two odd axes make the -1 that the last axis applies).
+// in [O][n][I] -> out [O][m][I]; tab = cos or sin of 2 pi q / P, q < P.
+// Setup only: O(n) FP64 multiply-adds per output, any length.
+__global__ void k_octant_axis(const double* __restrict__ in, double* __restrict__ out, long O, int n, int I, int m,
+                              int P, int odd, const double* __restrict__ tab) {
+    const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= O * m * I) return;
+    const int i = (int)(idx % I);
+    const long r = idx / I;
+    const int k = (int)(r % m);
+    const double* p = in + (r / m) * n * (long)I + i;
+    double a0 = 0.0, a1 = 0.0;
+    int q = k;
+    for (int j = 1; j < n; ++j) {
+        const double w = tab[q];
+        if (j & 1) a0 += p[(long)j * I] * w;
+        else a1 += p[(long)j * I] * w;
+        q += k;
+        if (q >= P) q -= P;
+    }
+    out[idx] = (odd ? 0.0 : p[0]) + 2.0 * (a0 + a1);
+}
+
+// [kz][ky][kx] of one component -> its place in [K][6][Pz2][KQ]
+template <typename T>
+__global__ void k_octant_place(const double* __restrict__ in, T* __restrict__ kern, int comp, int K, int Pz2, int Py2,
+                               int KQ, double sign) {
+    const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (long)K * Pz2 * KQ) return;
+    const int ky = (int)(idx % KQ);
+    const int kz = (int)(idx / KQ % Pz2);
+    const long kx = idx / ((long)KQ * Pz2);
+    kern[((kx * 6 + comp) * Pz2 + kz) * KQ + ky] =
+        ky < Py2 ? (T)(sign * in[((long)kz * Py2 + ky) * K + kx]) : (T)0;
+}
+
+// octant of the [c][z][y][kx] passes, [6][Pz2][Py2][Hs] -> [K][6][Pz2][KQ]
+template <typename T>
+__global__ void k_octant_turn(const T* __restrict__ in, T* __restrict__ kern, int K, int Pz2, int Py2, int Hs, int KQ) {
+    const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (long)K * 6 * Pz2 * KQ) return;
+    const int ky = (int)(idx % KQ);
+    const long r = idx / KQ;
+    const int cz = (int)(r % (6 * Pz2));     // comp Pz2 + kz
+    const long kx = r / (6 * Pz2);
+    kern[idx] = ky < Py2 ? in[((long)cz * Py2 + ky) * Hs + kx] : (T)0;
+}
+
+__global__ void k_split(const double* __restrict__ in, ff* __restrict__ out, long n) {
+    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double d = in[i];
+    const float h = __double2float_rn(d);
+    out[i] = ff(h, __double2float_rn(d - (double)h));
+}
+
+unsigned blocks(long n) { return (unsigned)((n + 255) / 256); }
+size_t elem(const mm_ctx* ctx) { return ctx->prec == MM_F64 ? 8 : 4; }
+long kern_count(const mm_ctx* ctx) { return (long)ctx->plane.K * 6 * ctx->Pz2 * ctx->plane.KQ; }
+long tw_count(const mm_ctx* ctx) { return 2 * (ctx->plane.off_z + ctx->Pz); }
+
+void table(int L, std::vector<double>& out) {
+    const long double pi = 3.141592653589793238462643383279502884L;
+    for (int m = 0; m < L; ++m) {
+        const long double a = 2.0L * pi * (long double)m / (long double)L;
+        out.push_back((double)cosl(a));
+        out.push_back((double)-sinl(a));
+    }
+}
+
+}  // namespace
+
+// Which contexts run in the plane layout: every mesh with nx, ny > 1 and a
+// side that is not a power of two, and power-of-two meshes whose plane (3 nz
+// lines of the padded y length) fits one block's shared memory with a z
+// transform that fits a thread's registers (nz <= 8; FP64 and float-float 4).
+int plane_plan(mm_ctx* ctx) {
+    PlanePlan& p = ctx->plane;
+    p = PlanePlan();
+    if (ctx->nx < 2 || ctx->ny < 2) return MM_OK;
+    const size_t cs = 2 * elem(ctx);
+    p.L = next_len(ctx->nx);
+    p.P = next_len(2 * ctx->ny);
+    const bool regular = pow2(ctx->nx) && pow2(ctx->ny);
+    const bool fits = ctx->nz <= (ctx->prec == MM_F32 ? 8 : 4) &&
+                      3 * (size_t)ctx->nz * plane_line_len(p.P) * cs <= 227 * 1024;
+    if (regular && !fits) return MM_OK;
+    p.on = 1;
+    p.lines = !fits;
+    p.K = p.L + 1;
+    p.KQ = (p.P / 2 + 1 + 3) / 4 * 4;
+    p.R = (3L * ctx->nz * ctx->ny + 3) / 4 * 4;
+    p.off_p = p.L;
+    p.off_y = p.off_p + 2 * p.L;
+    p.off_z = p.off_y + p.P;
+    int rc;
+    if ((rc = dev_alloc(ctx, &p.buf, (size_t)p.K * p.R * cs))) return rc;
+    if (p.lines && (rc = dev_alloc(ctx, &p.buf2, (size_t)p.K * 3 * ctx->nz * p.P * cs))) return rc;
+    if ((rc = dev_alloc(ctx, &p.kern, (size_t)kern_count(ctx) * elem(ctx)))) return rc;
+    if ((rc = dev_alloc(ctx, &p.tw, (size_t)tw_count(ctx) * elem(ctx)))) return rc;
+    std::vector<double> t;
+    table(p.L, t);
+    table(2 * p.L, t);
+    table(p.P, t);
+    table(ctx->Pz, t);
+    if (ctx->prec == MM_F64) {
+        MM_CUDA_CHECK(ctx, cudaMemcpy(p.tw, t.data(), t.size() * sizeof(double), cudaMemcpyHostToDevice));
+    } else {
+        std::vector<float> f(t.begin(), t.end());
+        MM_CUDA_CHECK(ctx, cudaMemcpy(p.tw, f.data(), f.size() * sizeof(float), cudaMemcpyHostToDevice));
+    }
+    return MM_OK;
+}
+
+void plane_free(mm_ctx* ctx) {
+    PlanePlan& p = ctx->plane;
+    void* ptrs[] = {p.buf, p.buf2, p.kern, p.kern_ff, p.tw, p.tw_ff};
+    for (void* q : ptrs)
+        if (q) cudaFree(q);
+    p = PlanePlan();
+}
+
+// Fills the plan's octant.  Same padded lengths as the [c][z][y][kx] passes
+// (powers of two from 16 up): their octant, turned.  Otherwise the Newell
+// tensor transformed axis by axis from its definition; that also fills
+// ctx->newell_host.
+int plane_setup(mm_ctx* ctx) {
+    PlanePlan& p = ctx->plane;
+    const int Pz2 = ctx->Pz2, Py2 = p.P / 2 + 1;
+    if (ctx->classic_ready && p.L == ctx->nx && p.P == ctx->Py) {
+        const long n = kern_count(ctx);
+        if (ctx->prec == MM_F64)
+            k_octant_turn<double><<<blocks(n), 256, 0, ctx->stream>>>((const double*)ctx->kern, (double*)p.kern, p.K, Pz2,
+                                                                      Py2, ctx->Hs, p.KQ);
+        else
+            k_octant_turn<float><<<blocks(n), 256, 0, ctx->stream>>>((const float*)ctx->kern, (float*)p.kern, p.K, Pz2,
+                                                                     Py2, ctx->Hs, p.KQ);
+        MM_LAUNCH_CHECK(ctx);
+        return MM_OK;
+    }
+    const int len[3] = {2 * p.L, p.P, ctx->Pz}, n[3] = {ctx->nx, ctx->ny, ctx->nz}, m[3] = {p.K, Py2, Pz2};
+    std::vector<double> t;
+    long off[3];
+    for (int a = 0; a < 3; ++a) {
+        off[a] = (long)t.size();
+        std::vector<double> e;
+        table(len[a], e);
+        for (int s = 0; s < 2; ++s)
+            for (int q = 0; q < len[a]; ++q) t.push_back(s ? -e[2 * q + 1] : e[2 * q]);   // cos, then sin
+    }
+    const long fsize = (long)(ctx->nx + 1) * (ctx->ny + 1) * (ctx->nz + 1);
+    void *oct = nullptr, *fg = nullptr, *a1 = nullptr, *a2 = nullptr, *a3 = nullptr, *tab = nullptr;
+    auto cleanup = [&]() {
+        for (void* q : {oct, fg, a1, a2, a3, tab}) cudaFree(q);
+    };
+    int rc = MM_OK;
+    auto A = [&](void** q, size_t b) {
+        if (rc == MM_OK) rc = dev_alloc(ctx, q, b);
+    };
+    A(&oct, sizeof(double) * 6 * ctx->N);
+    A(&fg, sizeof(double2) * fsize);
+    A(&a1, sizeof(double) * (size_t)ctx->nz * ctx->ny * p.K);
+    A(&a2, sizeof(double) * (size_t)ctx->nz * Py2 * p.K);
+    A(&a3, sizeof(double) * (size_t)Pz2 * Py2 * p.K);
+    A(&tab, sizeof(double) * t.size());
+    if (rc == MM_OK && cudaMemcpy(tab, t.data(), sizeof(double) * t.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+        rc = fail(ctx, MM_ERR_CUDA, "octant table copy failed");
+    for (int c = 0; c < 6 && rc == MM_OK; ++c) {
+        double* oc = (double*)oct + c * ctx->N;
+        if ((rc = newell_component(ctx, c, nullptr, oc, fg))) break;
+        const int odd[3] = {c == 3 || c == 4, c == 3 || c == 5, c == 4 || c == 5};
+        const double* src[3] = {oc, (const double*)a1, (const double*)a2};
+        double* dst[3] = {(double*)a1, (double*)a2, (double*)a3};
+        const long O[3] = {(long)ctx->nz * ctx->ny, ctx->nz, 1}, I[3] = {1, p.K, (long)Py2 * p.K};
+        for (int a = 0; a < 3; ++a) {
+            const long total = O[a] * m[a] * I[a];
+            k_octant_axis<<<blocks(total), 256, 0, ctx->stream>>>(src[a], dst[a], O[a], n[a], (int)I[a], m[a], len[a],
+                                                                 odd[a], (const double*)tab + off[a] + (odd[a] ? len[a] : 0));
+        }
+        const long total = (long)p.K * Pz2 * p.KQ;
+        const double sign = c >= 3 ? -1.0 : 1.0;
+        if (ctx->prec == MM_F64)
+            k_octant_place<double><<<blocks(total), 256, 0, ctx->stream>>>((const double*)a3, (double*)p.kern, c, p.K,
+                                                                           Pz2, Py2, p.KQ, sign);
+        else
+            k_octant_place<float><<<blocks(total), 256, 0, ctx->stream>>>((const double*)a3, (float*)p.kern, c, p.K, Pz2,
+                                                                          Py2, p.KQ, sign);
+        ctx->launches += 4;
+        if (cudaGetLastError() != cudaSuccess) rc = fail(ctx, MM_ERR_CUDA, "octant kernel launch failed");
+    }
+    cudaError_t e = cudaSuccess;
+    if (rc == MM_OK)
+        e = cudaMemcpyAsync(ctx->newell_host, oct, sizeof(double) * 6 * ctx->N, cudaMemcpyDeviceToHost, ctx->stream);
+    const cudaError_t es = cudaStreamSynchronize(ctx->stream);
+    if (rc == MM_OK && (e != cudaSuccess || es != cudaSuccess))
+        rc = fail(ctx, MM_ERR_CUDA, "octant setup failed: %s", cudaGetErrorString(e != cudaSuccess ? e : es));
+    cleanup();
+    return rc;
+}
+
+// float-float copies of the octant and the tables (MM_FFT_FF)
+int plane_prepare_ff(mm_ctx* ctx) {
+    PlanePlan& p = ctx->plane;
+    if (p.kern_ff && p.tw_ff) return MM_OK;
+    const long nk = kern_count(ctx), nt = tw_count(ctx);
+    int rc;
+    if (!p.kern_ff && (rc = dev_alloc(ctx, &p.kern_ff, nk * sizeof(ff)))) return rc;
+    if (!p.tw_ff && (rc = dev_alloc(ctx, &p.tw_ff, nt * sizeof(ff)))) return rc;
+    k_split<<<blocks(nk), 256, 0, ctx->stream>>>((const double*)p.kern, (ff*)p.kern_ff, nk);
+    MM_LAUNCH_CHECK(ctx);
+    k_split<<<blocks(nt), 256, 0, ctx->stream>>>((const double*)p.tw, (ff*)p.tw_ff, nt);
+    MM_LAUNCH_CHECK(ctx);
+    MM_CUDA_CHECK(ctx, cudaStreamSynchronize(ctx->stream));
+    return MM_OK;
+}
+
+int plane_apply(mm_ctx* ctx, const void* m, void* H, bool unit) {
+    const void* Ms = ctx->has_Ms_cell && !unit ? ctx->Ms_cell : nullptr;
+    const double ms = unit ? 1.0 : ctx->Ms;
+    if (ctx->prec == MM_F32)
+        return plane_apply_f32(ctx, (const float*)m, (const float*)Ms, (float)ms, (float*)H);
+    if (ctx->fft_mode == MM_FFT_FF)
+        return plane_apply_ff(ctx, (const double*)m, (const double*)Ms, ms, (double*)H);
+    return plane_apply_f64(ctx, (const double*)m, (const double*)Ms, ms, (double*)H);
+}
+
+}  // namespace mm

@@ -1,0 +1,173 @@
+// Launchers of the plane-layout kernels: the length tables and one explicit
+// instantiation point per element type (mm_plane_f32*.cu,
+// mm_plane_f64*.cu).
+#pragma once
+
+#include "mm_plane.cuh"
+
+namespace mm {
+
+// f(integral_constant L1, integral_constant L2) for the four-step split of
+// length `len`; false when the length is not in the table.  Both factors are
+// even (the zero half of the input is n1 >= L1/2, the dropped half of the
+// output k2 >= L2/2).
+template <typename F> bool with_length(int len, F&& f) {
+#define MM_LEN(N, A, B) \
+    case N: f(std::integral_constant<int, A>{}, std::integral_constant<int, B>{}); return true
+    switch (len) {
+        MM_LEN(16, 4, 4);
+        MM_LEN(32, 8, 4);
+        MM_LEN(64, 8, 8);
+        MM_LEN(128, 16, 8);
+        MM_LEN(256, 16, 16);
+        MM_LEN(512, 32, 16);
+        MM_LEN(1024, 32, 32);
+        MM_LEN(40, 10, 4);
+        MM_LEN(48, 12, 4);
+        MM_LEN(80, 10, 8);
+        MM_LEN(96, 12, 8);
+        MM_LEN(160, 16, 10);
+        MM_LEN(192, 16, 12);
+        MM_LEN(320, 20, 16);
+        MM_LEN(384, 24, 16);
+        MM_LEN(640, 32, 20);
+        MM_LEN(768, 32, 24);
+        default: break;
+    }
+#undef MM_LEN
+    return false;
+}
+
+inline int plane_smem(mm_ctx* ctx, const void* fn, size_t bytes) {
+    if (bytes > 48 * 1024)
+        MM_CUDA_CHECK(ctx, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    return MM_OK;
+}
+
+// complex stride of a line of length P in the plane kernel's shared memory
+inline int plane_line(int P) {
+    int lp = 0;
+    with_length(P, [&](auto A, auto B) { lp = plane_pitch(decltype(A)::value, decltype(B)::value); });
+    return lp;
+}
+
+template <typename T, typename S>
+int launch_px_fwd(mm_ctx* ctx, const S* in, const S* Ms, T ms, long ms_rows, PC<T>* out, long rows, const PC<T>* tw) {
+    const PlanePlan& p = ctx->plane;
+    int rc = MM_OK;
+    KernelTimer kt(ctx, MM_K_XFWD);
+    if (!with_length(p.L, [&](auto A, auto B) {
+            constexpr int L1 = decltype(A)::value, L2 = decltype(B)::value, L = L1 * L2;
+            if constexpr (L <= 512) {
+                constexpr int BR = px_rows<T>(L);
+                k_px_fwd<T, S, L1, L2><<<(unsigned)((rows + BR - 1) / BR), px_threads(BR, L1, L2), 0, ctx->stream>>>(
+                    in, ctx->nx, Ms, ms, ms_rows, out, p.R, rows, tw, tw + p.off_p);
+            }
+        }))
+        rc = fail(ctx, MM_ERR_INVALID_ARG, "x length %d", p.L);
+    if (rc) return rc;
+    MM_LAUNCH_CHECK(ctx);
+    return MM_OK;
+}
+
+template <typename T, typename S>
+int launch_px_inv(mm_ctx* ctx, const PC<T>* in, S* out, long rows, T scale, const PC<T>* tw) {
+    const PlanePlan& p = ctx->plane;
+    int rc = MM_OK;
+    KernelTimer kt(ctx, MM_K_XINV);
+    if (!with_length(p.L, [&](auto A, auto B) {
+            constexpr int L1 = decltype(A)::value, L2 = decltype(B)::value, L = L1 * L2;
+            if constexpr (L <= 512) {
+                constexpr int BR = px_rows<T>(L);
+                k_px_inv<T, S, L1, L2><<<(unsigned)((rows + BR - 1) / BR), px_threads(BR, L1, L2), 0, ctx->stream>>>(
+                    in, p.R, out, ctx->nx, rows, scale, tw, tw + p.off_p);
+            }
+        }))
+        rc = fail(ctx, MM_ERR_INVALID_ARG, "x length %d", p.L);
+    if (rc) return rc;
+    MM_LAUNCH_CHECK(ctx);
+    return MM_OK;
+}
+
+template <typename T>
+int launch_plane(mm_ctx* ctx, PC<T>* buf, const T* kern, const PC<T>* tw) {
+    const PlanePlan& p = ctx->plane;
+    int rc = MM_OK;
+    KernelTimer kt(ctx, MM_K_ZCONV);
+    if (!with_length(p.P, [&](auto A, auto B) {
+            constexpr int L1 = decltype(A)::value, L2 = decltype(B)::value;
+            // the fused level 2 holds 3 L2 complex values: single precision, L2 <= 16
+            constexpr bool CANF = sizeof(T) == 4 && L2 <= 16;
+            const bool fused = CANF && ctx->nz == 1;
+            auto fn = fused ? k_plane<T, L1, L2, CANF> : k_plane<T, L1, L2, false>;
+            const size_t smem = (size_t)3 * ctx->nz * plane_pitch(L1, L2) * sizeof(PC<T>);
+            if ((rc = plane_smem(ctx, (const void*)fn, smem))) return;
+            const int tasks = 3 * ctx->nz * L1;
+            const int cap = sizeof(T) == 4 ? 512 : 256;
+            int nt = tasks;
+            if (nt > cap) nt = (tasks + (tasks + cap - 1) / cap - 1) / ((tasks + cap - 1) / cap);
+            nt = (nt + 31) / 32 * 32;
+            if (nt > cap) nt = cap;
+            fn<<<(unsigned)p.K, nt, smem, ctx->stream>>>(buf, kern, ctx->nz, ctx->ny, p.R, p.KQ, tw + p.off_y);
+        }))
+        rc = fail(ctx, MM_ERR_INVALID_ARG, "y length %d", p.P);
+    if (rc) return rc;
+    MM_LAUNCH_CHECK(ctx);
+    return MM_OK;
+}
+
+template <typename T, int DIR>
+int launch_py(mm_ctx* ctx, const PC<T>* in, PC<T>* out, const PC<T>* tw) {
+    const PlanePlan& p = ctx->plane;
+    int rc = MM_OK;
+    KernelTimer kt(ctx, DIR < 0 ? MM_K_YFWD : MM_K_YINV);
+    const int lines = 3 * ctx->nz;
+    const long nlines = (long)p.K * lines, wide = (long)lines * p.P;
+    if (!with_length(p.P, [&](auto A, auto B) {
+            constexpr int L1 = decltype(A)::value, L2 = decltype(B)::value;
+            auto fn = k_py<T, L1, L2, DIR>;
+            const size_t smem = (size_t)kPyLines * plane_pitch(L1, L2) * sizeof(PC<T>);
+            if ((rc = plane_smem(ctx, (const void*)fn, smem))) return;
+            fn<<<(unsigned)((nlines + kPyLines - 1) / kPyLines), (kPyLines * (L1 > L2 ? L1 : L2) + 31) / 32 * 32, smem,
+                 ctx->stream>>>(in, out, lines, nlines, ctx->ny, DIR < 0 ? p.R : wide, DIR < 0 ? wide : p.R, tw + p.off_y);
+        }))
+        rc = fail(ctx, MM_ERR_INVALID_ARG, "y length %d", p.P);
+    if (rc) return rc;
+    MM_LAUNCH_CHECK(ctx);
+    return MM_OK;
+}
+
+// columns per block of the z pass: 64-byte row segments where shared memory
+// allows (3 Pz B elements), 256 threads
+template <typename T, int L1, int L2, bool COLY>
+int launch_zline_t(mm_ctx* ctx, PC<T>* buf, const T* kern, const ZLine& g, int nrows, const PC<T>* tw) {
+    constexpr int PZ = L1 * L2, CS = (int)sizeof(PC<T>);
+    constexpr int B = PZ <= 64 ? 128 / CS : PZ <= 512 ? 64 / CS : 32 / CS;
+    constexpr int NT = 256;
+    constexpr int MINB = sizeof(T) == 4 && 3 * L2 <= 48 ? 2 : 1;
+    auto fn = k_zline<T, L1, L2, COLY, B, NT, MINB>;
+    const size_t smem = (size_t)3 * PZ * B * CS;
+    int rc = plane_smem(ctx, (const void*)fn, smem);
+    if (rc) return rc;
+    dim3 grid((unsigned)((g.ncol + B - 1) / B), (unsigned)nrows);
+    fn<<<grid, NT, smem, ctx->stream>>>(buf, kern, g, tw);
+    MM_LAUNCH_CHECK(ctx);
+    return MM_OK;
+}
+
+template <typename T, bool COLY>
+int launch_zline(mm_ctx* ctx, int Pz, PC<T>* buf, const T* kern, const ZLine& g, int nrows, const PC<T>* tw) {
+    KernelTimer kt(ctx, MM_K_ZCONV);
+    switch (Pz) {
+        case 16: return launch_zline_t<T, 4, 4, COLY>(ctx, buf, kern, g, nrows, tw);
+        case 32: return launch_zline_t<T, 8, 4, COLY>(ctx, buf, kern, g, nrows, tw);
+        case 64: return launch_zline_t<T, 8, 8, COLY>(ctx, buf, kern, g, nrows, tw);
+        case 128: return launch_zline_t<T, 16, 8, COLY>(ctx, buf, kern, g, nrows, tw);
+        case 256: return launch_zline_t<T, 32, 8, COLY>(ctx, buf, kern, g, nrows, tw);
+        case 512: return launch_zline_t<T, 32, 16, COLY>(ctx, buf, kern, g, nrows, tw);
+        case 1024: return launch_zline_t<T, 32, 32, COLY>(ctx, buf, kern, g, nrows, tw);
+        default: return fail(ctx, MM_ERR_INVALID_ARG, "z length %d", Pz);
+    }
+}
+
+}  // namespace mm

@@ -1,8 +1,8 @@
 // Register-resident DFTs of compile-time length (FP32 demag path).
 //
 // dif<N, DIR, HALF>(v) transforms the N complex values a thread holds in
-// registers by decimation in frequency (radix-2 split down to 8-, 4- or
-// 2-point kernels), leaving X[k] at register position dif_pos<N>(k) (a
+// registers by decimation in frequency (radix-2 split down to 8-, 5-, 4-, 3-
+// or 2-point kernels: N = 2^k times 1, 3 or 5), leaving X[k] at register position dif_pos<N>(k) (a
 // compile-time permutation, so reordering costs nothing).  HALF = true
 // declares the upper half of the input zero (the zero-padded half of a
 // line), which turns the first butterfly level into a copy and a twiddle.
@@ -35,9 +35,10 @@ constexpr double taylor_cos(double x) {
     }
     return s;
 }
-// cos and sin of 2 pi k / n, n a power of two
+// cos and sin of 2 pi k / n
 constexpr double cos2pi(int k, int n);
 constexpr double sin2pi(int k, int n) {
+    if (n % 4) return sin2pi(4 * k, 4 * n);
     k = ((k % n) + n) % n;
     if (2 * k > n) return -sin2pi(n - k, n);
     if (4 * k > n) return sin2pi(n / 2 - k, n);            // sin(pi - a) = sin a
@@ -45,6 +46,7 @@ constexpr double sin2pi(int k, int n) {
     return taylor_sin(2.0 * kPiTaylor * k / n);
 }
 constexpr double cos2pi(int k, int n) {
+    if (n % 4) return cos2pi(4 * k, 4 * n);
     k = ((k % n) + n) % n;
     if (2 * k > n) return cos2pi(n - k, n);
     if (4 * k > n) return -cos2pi(n / 2 - k, n);           // cos(pi - a) = -cos a
@@ -63,7 +65,7 @@ template <int I, int N, typename F> __host__ __device__ __forceinline__ void sta
 
 // position of X[k] after dif<N>
 template <int N> __host__ __device__ constexpr int dif_pos(int k) {
-    if constexpr (N <= 8) {
+    if constexpr (N % 2 == 1 || N == 2 || N == 4 || N == 8) {
         return k;
     } else {
         return (k & 1) ? N / 2 + dif_pos<N / 2>(k >> 1) : dif_pos<N / 2>(k >> 1);
@@ -142,6 +144,31 @@ template <int DIR, typename C> __host__ __device__ __forceinline__ void rdft8(C*
     v[3] = padd(e[3], w3o);
     v[7] = psub(e[3], w3o);
 }
+// 3- and 5-point DFTs from the sums and differences of conjugate pairs
+template <int DIR, typename C> __host__ __device__ __forceinline__ void rdft3(C* v) {
+    using T = decltype(C{}.x);
+    constexpr double sn = DIR * sin2pi(1, 3);
+    const C t = padd(v[1], v[2]), d = cscale(psub(v[1], v[2]), (T)sn);
+    const C a = cmk<C>(v[0].x - (T)0.5 * t.x, v[0].y - (T)0.5 * t.y);
+    v[0] = padd(v[0], t);
+    v[1] = cmk<C>(a.x - d.y, a.y + d.x);
+    v[2] = cmk<C>(a.x + d.y, a.y - d.x);
+}
+template <int DIR, typename C> __host__ __device__ __forceinline__ void rdft5(C* v) {
+    using T = decltype(C{}.x);
+    constexpr double dc1 = cos2pi(1, 5), dc2 = cos2pi(2, 5), ds1 = DIR * sin2pi(1, 5), ds2 = DIR * sin2pi(2, 5);
+    const T c1 = (T)dc1, c2 = (T)dc2, s1 = (T)ds1, s2 = (T)ds2;
+    const C t1 = padd(v[1], v[4]), t2 = padd(v[2], v[3]), t3 = psub(v[1], v[4]), t4 = psub(v[2], v[3]);
+    const C a = cmk<C>(v[0].x + c1 * t1.x + c2 * t2.x, v[0].y + c1 * t1.y + c2 * t2.y);
+    const C b = cmk<C>(v[0].x + c2 * t1.x + c1 * t2.x, v[0].y + c2 * t1.y + c1 * t2.y);
+    const C p = cmk<C>(s1 * t3.x + s2 * t4.x, s1 * t3.y + s2 * t4.y);
+    const C q = cmk<C>(s2 * t3.x - s1 * t4.x, s2 * t3.y - s1 * t4.y);
+    v[0] = cmk<C>(v[0].x + t1.x + t2.x, v[0].y + t1.y + t2.y);
+    v[1] = cmk<C>(a.x - p.y, a.y + p.x);
+    v[4] = cmk<C>(a.x + p.y, a.y - p.x);
+    v[2] = cmk<C>(b.x - q.y, b.y + q.x);
+    v[3] = cmk<C>(b.x + q.y, b.y - q.x);
+}
 // scalar 4- and 8-point DFTs of inputs whose upper half is zero: plain
 // arithmetic, so the compiler folds the zero operands away
 template <int DIR, typename C> __host__ __device__ __forceinline__ void rdft4_half(C* v) {
@@ -217,6 +244,10 @@ template <int N, int DIR, bool HALF, typename C> __host__ __device__ __forceinli
     } else if constexpr (N == 8) {
         if constexpr (HALF) rdft8_half<DIR>(v);
         else rdft8<DIR>(v);
+    } else if constexpr (N == 3) {
+        rdft3<DIR>(v);
+    } else if constexpr (N == 5) {
+        rdft5<DIR>(v);
     } else {
         dif_level<N, 0, DIR, HALF>(v);
         dif<N / 2, DIR, false>(v);

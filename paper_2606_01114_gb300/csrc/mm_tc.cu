@@ -556,7 +556,8 @@ extern "C" int mm_set_fft_mode(mm_ctx* ctx, int mode) {
         if (!f4_supported(ctx))
             return fail(ctx, MM_ERR_INVALID_ARG, "the fused y-z-y pass needs an MM_F32 context with ny = 512, nz = 16");
         MM_BIND(ctx);
-        int rc = f4_prepare(ctx);
+        int rc = classic_prepare(ctx);
+        if (!rc) rc = f4_prepare(ctx);
         if (rc) return rc;
         ctx->fft_mode = mode;
         return MM_OK;
@@ -575,7 +576,9 @@ extern "C" int mm_set_fft_mode(mm_ctx* ctx, int mode) {
     if (mode != 0 && ctx->prec != MM_F32) return fail(ctx, MM_ERR_INVALID_ARG, "tensor-core passes need an MM_F32 context");
     MM_BIND(ctx);
     if (mode != 0) {
-        int rc = tc_prepare(ctx);
+        int rc = classic_prepare(ctx);
+        if (rc) return rc;
+        rc = tc_prepare(ctx);
         if (rc) return fail(ctx, rc, "%s", mm_last_error(nullptr));
     }
     ctx->fft_mode = mode;
