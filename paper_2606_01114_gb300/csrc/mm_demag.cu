@@ -33,6 +33,10 @@
 #include "mm_tma.cuh"
 
 namespace mm {
+
+// mm_zline.cu: the FP32 z pass of long z lines (Pz >= 64)
+int zline_f32(mm_ctx* ctx, float2* buf, const float* kern, const float2* tw);
+
 namespace {
 
 template <typename T> using C_t = typename cx<T>::type;
@@ -1641,7 +1645,10 @@ int apply(mm_ctx* ctx, const T* m, T* H, bool unit = false) {
         if (rc) return rc;
     }
     // K4
-    if (sizeof(T) == 4 && ctx->Pz <= 32) {
+    if (sizeof(T) == 4 && ctx->Pz >= 64) {
+        rc = zline_f32(ctx, (float2*)Bf, (const float*)ctx->kern, (const float2*)table<T>(ctx, ctx->tw.off_z4));
+        if (rc) return rc;
+    } else if (sizeof(T) == 4) {
         KernelTimer kt(ctx, MM_K_ZCONV);
         rc = launch_zconv_reg(ctx, (float2*)Bf, (const float*)ctx->kern, 0, ctx->Hx);
         if (rc) return rc;

@@ -62,6 +62,7 @@ struct Tables {
     void* f32 = nullptr;   // float2 (only for MM_F32 contexts)
     void* ff = nullptr;    // float-float copy of f64 (MM_FFT_FF on an MM_F64 context)
     long off_lx = 0, off_px = 0, off_py = 0, off_pz = 0;
+    long off_z4 = 0;       // four-step tables of Pz (mm_zline.cu)
 };
 
 // Bluestein (chirp-z) data of one padded axis whose length P is not a power
@@ -91,7 +92,9 @@ struct PlanePlan {
     int K = 0;           // planes: L + 1 kept x frequencies
     int KQ = 0;          // octant row stride (P / 2 + 1 rounded up to 4)
     long R = 0;          // plane stride of buf, complex (3 nz ny rounded up to 4)
-    long off_p = 0, off_y = 0, off_z = 0;   // twiddle tables of 2L, P and Pz behind that of L
+    // twiddle tables exp(-2 pi i m / len), natural order: L at 0, then 2L, P,
+    // Pz; behind them the four-step tables ([k1][t], [t][k1]) of L, P and Pz
+    long off_p = 0, off_y = 0, off_z = 0, off_x4 = 0, off_y4 = 0, off_z4 = 0, tw_len = 0;
     void* buf = nullptr;     // complex [K][R]
     void* buf2 = nullptr;    // complex [K][3 nz][P] (lines)
     void* kern = nullptr;    // octant [K][6][Pz/2+1][KQ], path precision
@@ -243,6 +246,9 @@ int plane_setup(mm_ctx* ctx);
 void plane_free(mm_ctx* ctx);
 int plane_apply(mm_ctx* ctx, const void* m, void* H, bool unit);
 int plane_prepare_ff(mm_ctx* ctx);
+// appends the four-step tables w^(t k1), [k1][t] and then [t][k1], of an x or
+// y length (or a z length) of mm_plane_launch.cuh; nothing for other lengths
+void four_step_table(int len, bool z, std::vector<double>& out);
 int dev_alloc(mm_ctx* ctx, void** p, size_t bytes);
 int demag_apply(mm_ctx* ctx, const void* m, void* H);  // K2..K6
 int demag_apply_unit(mm_ctx* ctx, const void* g, void* H);  // same with Ms = 1 (adjoint)

@@ -88,7 +88,7 @@ __global__ void k_split(const double* __restrict__ in, ff* __restrict__ out, lon
 unsigned blocks(long n) { return (unsigned)((n + 255) / 256); }
 size_t elem(const mm_ctx* ctx) { return ctx->prec == MM_F64 ? 8 : 4; }
 long kern_count(const mm_ctx* ctx) { return (long)ctx->plane.K * 6 * ctx->Pz2 * ctx->plane.KQ; }
-long tw_count(const mm_ctx* ctx) { return 2 * (ctx->plane.off_z + ctx->Pz); }
+long tw_count(const mm_ctx* ctx) { return 2 * ctx->plane.tw_len; }
 
 void table(int L, std::vector<double>& out) {
     const long double pi = 3.141592653589793238462643383279502884L;
@@ -105,6 +105,12 @@ void table(int L, std::vector<double>& out) {
 // side that is not a power of two, and power-of-two meshes whose plane (3 nz
 // lines of the padded y length) fits one block's shared memory with a z
 // transform that fits a thread's registers (nz <= 8; FP64 and float-float 4).
+// Power-of-two meshes also need two blocks per SM (113 KB a plane) or no more
+// planes than SMs; at one block per SM over several waves the five streaming
+// passes are the faster: 512x512x8 FP32 169 against 185 us, 512x512x4 FP64
+// 1804 against 1826 us.  On the near side of the line: 512x512x4 FP32 85
+// against 96 us, 64x512x8 (65 planes) 40 against 43 us, 256x256x8 44 against
+// 56 us.
 int plane_plan(mm_ctx* ctx) {
     PlanePlan& p = ctx->plane;
     p = PlanePlan();
@@ -113,9 +119,9 @@ int plane_plan(mm_ctx* ctx) {
     p.L = next_len(ctx->nx);
     p.P = next_len(2 * ctx->ny);
     const bool regular = pow2(ctx->nx) && pow2(ctx->ny);
-    const bool fits = ctx->nz <= (ctx->prec == MM_F32 ? 8 : 4) &&
-                      3 * (size_t)ctx->nz * plane_line_len(p.P) * cs <= 227 * 1024;
-    if (regular && !fits) return MM_OK;
+    const size_t smem = 3 * (size_t)ctx->nz * plane_line_len(p.P) * cs;
+    const bool fits = ctx->nz <= (ctx->prec == MM_F32 ? 8 : 4) && smem <= 227 * 1024;
+    if (regular && (!fits || (smem > 113 * 1024 && p.L + 1 > 152))) return MM_OK;
     p.on = 1;
     p.lines = !fits;
     p.K = p.L + 1;
@@ -124,16 +130,23 @@ int plane_plan(mm_ctx* ctx) {
     p.off_p = p.L;
     p.off_y = p.off_p + 2 * p.L;
     p.off_z = p.off_y + p.P;
-    int rc;
-    if ((rc = dev_alloc(ctx, &p.buf, (size_t)p.K * p.R * cs))) return rc;
-    if (p.lines && (rc = dev_alloc(ctx, &p.buf2, (size_t)p.K * 3 * ctx->nz * p.P * cs))) return rc;
-    if ((rc = dev_alloc(ctx, &p.kern, (size_t)kern_count(ctx) * elem(ctx)))) return rc;
-    if ((rc = dev_alloc(ctx, &p.tw, (size_t)tw_count(ctx) * elem(ctx)))) return rc;
     std::vector<double> t;
     table(p.L, t);
     table(2 * p.L, t);
     table(p.P, t);
     table(ctx->Pz, t);
+    long* const off4[3] = {&p.off_x4, &p.off_y4, &p.off_z4};
+    const int len4[3] = {p.L, p.P, ctx->Pz};
+    for (int a = 0; a < 3; ++a) {
+        *off4[a] = (long)t.size() / 2;
+        four_step_table(len4[a], a == 2, t);
+    }
+    p.tw_len = (long)t.size() / 2;
+    int rc;
+    if ((rc = dev_alloc(ctx, &p.buf, (size_t)p.K * p.R * cs))) return rc;
+    if (p.lines && (rc = dev_alloc(ctx, &p.buf2, (size_t)p.K * 3 * ctx->nz * p.P * cs))) return rc;
+    if ((rc = dev_alloc(ctx, &p.kern, (size_t)kern_count(ctx) * elem(ctx)))) return rc;
+    if ((rc = dev_alloc(ctx, &p.tw, (size_t)tw_count(ctx) * elem(ctx)))) return rc;
     if (ctx->prec == MM_F64) {
         MM_CUDA_CHECK(ctx, cudaMemcpy(p.tw, t.data(), t.size() * sizeof(double), cudaMemcpyHostToDevice));
     } else {

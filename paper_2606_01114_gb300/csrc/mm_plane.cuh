@@ -22,7 +22,10 @@
 // level 2 (thread k1 < L1) DFT over n2, X[k1 + L1 k2].  Element (k1, t) sits
 // at k1 (L2 + 1) + t of its line: both levels read and write the same places
 // (no barrier between a level's loads and stores), and the odd pitch keeps
-// the row accesses of level 2 off each other's banks.
+// the row accesses of level 2 off each other's banks.  The twiddles w^(t k1)
+// come from tables laid out [k1][t] and, behind it, [t][k1]: every load of a
+// level sits at a compile-time offset from one pointer, and the lanes of a
+// warp (consecutive t, or consecutive k1) read consecutive values.
 #pragma once
 
 #include "mm_ff.cuh"
@@ -86,11 +89,12 @@ __global__ void __launch_bounds__(px_threads(px_rows<T>(L1 * L2), L1, L2))
             }
             v[n1] = cmk<C>(ta, tc);
         }
+        const C* tq = twL + t;
         dif<L1, -1, true>(v);
 #pragma unroll
         for (int k1 = 0; k1 < L1; ++k1) {
             C y = v[dif_pos<L1>(k1)];
-            if (k1 > 0) y = cmul(y, twL[t * k1]);
+            if (k1 > 0) y = cmul(y, tq[k1 * L2]);
             Sm[b * LP + k1 * (L2 + 1) + t] = y;
         }
     }
@@ -154,11 +158,12 @@ __global__ void __launch_bounds__(px_threads(px_rows<T>(L1 * L2), L1, L2))
         C v[L1];
 #pragma unroll
         for (int n1 = 0; n1 < L1; ++n1) v[n1] = s[n1 * (L2 + 1)];
+        const C* tq = twL + t;
         dif<L1, +1, false>(v);
 #pragma unroll
         for (int k1 = 0; k1 < L1; ++k1) {
             C y = v[dif_pos<L1>(k1)];
-            if (k1 > 0) y = cmul(y, cconj(twL[t * k1]));
+            if (k1 > 0) y = cmul(y, cconj(tq[k1 * L2]));
             s[k1 * (L2 + 1)] = y;
         }
     }
@@ -275,10 +280,11 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 512 : 256)
         }
         dif<L1, -1, true>(v);
         C* s = Sm + line * LP + t;
+        const C* tq = tw + t;
 #pragma unroll
         for (int k1 = 0; k1 < L1; ++k1) {
             C y = v[dif_pos<L1>(k1)];
-            if (k1 > 0) y = cmul(y, tw[t * k1]);
+            if (k1 > 0) y = cmul(y, tq[k1 * L2]);
             s[k1 * (L2 + 1)] = y;
         }
     }
@@ -286,6 +292,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 512 : 256)
     if constexpr (FUSED) {
         for (int k1 = tid; k1 < L1; k1 += nt) {
             C* s = Sm + k1 * (L2 + 1);
+            const C* tq = tw + P + k1;
             C u[3][L2];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
@@ -317,7 +324,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 512 : 256)
 #pragma unroll
                 for (int t = 0; t < L2; ++t) {
                     C y = w[dif_pos<L2>(t)];
-                    if (t > 0) y = cmul(y, cconj(tw[t * k1]));
+                    if (t > 0) y = cmul(y, cconj(tq[t * L1]));
                     s[c * LP + t] = y;
                 }
             }
@@ -350,6 +357,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 512 : 256)
         for (int i = tid; i < lines * L1; i += nt) {
             const int k1 = i % L1;
             C* s = Sm + (i / L1) * LP + k1 * (L2 + 1);
+            const C* tq = tw + P + k1;
             C u[L2];
 #pragma unroll
             for (int k2 = 0; k2 < L2; ++k2) u[k2] = s[k2];
@@ -357,7 +365,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 512 : 256)
 #pragma unroll
             for (int t = 0; t < L2; ++t) {
                 C y = u[dif_pos<L2>(t)];
-                if (t > 0) y = cmul(y, cconj(tw[t * k1]));
+                if (t > 0) y = cmul(y, cconj(tq[t * L1]));
                 s[t] = y;
             }
         }
@@ -408,11 +416,12 @@ __global__ void __launch_bounds__((kPyLines * (L1 > L2 ? L1 : L2) + 31) / 32 * 3
             }
             dif<L1, DIR, (DIR < 0)>(v);
             C* s = Sm + b * LP + t;
+            const C* tq = tw + t;
 #pragma unroll
             for (int k1 = 0; k1 < L1; ++k1) {
                 C y = v[dif_pos<L1>(k1)];
                 if (k1 > 0) {
-                    C w = tw[t * k1];
+                    C w = tq[k1 * L2];
                     if (DIR > 0) w = cconj(w);
                     y = cmul(y, w);
                 }
@@ -454,13 +463,25 @@ struct ZLine {
     int nz, ncol, P;      // P: length of the mirrored axis (y)
 };
 
+// The tile's octant values are copied into shared memory by asynchronous
+// copies that land while level 1 runs: read from global memory they sat on
+// the critical path of the middle level (6 L2 dependent loads per thread).
+template <typename T> __device__ __forceinline__ void cp_async_value(T* smem, const T* gmem) {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(a), "l"(gmem), "n"(sizeof(T)) : "memory");
+}
+template <typename T, int L1, int L2, int B> constexpr size_t zline_smem() {
+    return (size_t)3 * L1 * (L2 + 1) * B * sizeof(PC<T>) + (size_t)6 * (L1 * L2 / 2 + 1) * B * sizeof(T);
+}
+
 template <typename T, int L1, int L2, bool COLY, int B, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
     k_zline(PC<T>* __restrict__ buf, const T* __restrict__ kern, ZLine g, const PC<T>* __restrict__ tw) {
     using C = PC<T>;
-    constexpr int PZ = L1 * L2;
+    constexpr int PZ = L1 * L2, PZ2 = PZ / 2 + 1, LQ = L2 + 1, CP = L1 * LQ * B;   // component pitch
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* Sm = reinterpret_cast<C*>(smem_raw);        // [3][L1][L2][B]
+    C* Sm = reinterpret_cast<C*>(smem_raw);                 // [3][L1][L2 + 1][B]
+    T* Kn = reinterpret_cast<T*>(Sm + 3 * CP);              // [6][PZ2][B]
     const int tid = threadIdx.x;
     const int col0 = blockIdx.x * B;
     int row = blockIdx.y;
@@ -475,10 +496,17 @@ __global__ void __launch_bounds__(NT, MINB)
     }
     C* base = buf + (long)row * g.row_s + col0;
     const T* kbase = kern + (long)krow * g.k_row;
+    for (int i = tid; i < 6 * PZ2 * B; i += NT) {
+        const int b = i % B, ck = i / B, kz = ck % PZ2, c = ck / PZ2;
+        const int col = col0 + b < g.ncol ? col0 + b : g.ncol - 1;
+        const int kcol = COLY && 2 * col > g.P ? g.P - col : col;
+        cp_async_value(Kn + i, kbase + c * g.kc_s + kz * g.kz_s + kcol);
+    }
 #pragma unroll 1
     for (int i = tid; i < 3 * L2 * B; i += NT) {
         const int b = i % B, ct = i / B, t = ct % L2, c = ct / L2;
-        C* s = Sm + ((c * L1) * L2 + t) * B + b;
+        C* s = Sm + c * CP + t * B + b;
+        const C* tq = tw + t;
         const C* p = base + c * g.c_s + b;
         const bool act = col0 + b < g.ncol;
         C v[L1];
@@ -488,32 +516,32 @@ __global__ void __launch_bounds__(NT, MINB)
 #pragma unroll
         for (int k1 = 0; k1 < L1; ++k1) {
             C y = v[dif_pos<L1>(k1)];
-            if (k1 > 0) y = cmul(y, tw[t * k1]);
-            s[k1 * L2 * B] = y;
+            if (k1 > 0) y = cmul(y, tq[k1 * L2]);
+            s[k1 * LQ * B] = y;
         }
     }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
 #pragma unroll 1
     for (int i = tid; i < L1 * B; i += NT) {
         const int b = i % B, k1 = i / B;
-        const int col = col0 + b < g.ncol ? col0 + b : g.ncol - 1;
-        const bool yodd = COLY ? 2 * col > g.P : rodd;
-        const T* kb = kbase + (COLY ? (yodd ? g.P - col : col) : col);
-        C* s = Sm + (k1 * L2) * B + b;
+        const bool yodd = COLY ? 2 * (col0 + b) > g.P : rodd;
+        C* s = Sm + k1 * LQ * B + b;
+        const C* tq = tw + PZ + k1;
         C u[3][L2];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
 #pragma unroll
-            for (int n2 = 0; n2 < L2; ++n2) u[c][n2] = s[(c * L1 * L2 + n2) * B];
+            for (int n2 = 0; n2 < L2; ++n2) u[c][n2] = s[c * CP + n2 * B];
             dif<L2, -1, false>(u[c]);
         }
 #pragma unroll
         for (int k2 = 0; k2 < L2; ++k2) {
             const int kz = k1 + L1 * k2;
             const bool zodd = 2 * kz > PZ;
-            const T* kk = kb + (zodd ? PZ - kz : kz) * g.kz_s;
-            const T xx = kk[0], yy = kk[g.kc_s], zz = kk[2 * g.kc_s];
-            T xy = kk[3 * g.kc_s], xz = kk[4 * g.kc_s], yz = kk[5 * g.kc_s];
+            const T* kk = Kn + (zodd ? PZ - kz : kz) * B + b;
+            const T xx = kk[0], yy = kk[PZ2 * B], zz = kk[2 * PZ2 * B];
+            T xy = kk[3 * PZ2 * B], xz = kk[4 * PZ2 * B], yz = kk[5 * PZ2 * B];
             if (yodd) xy = -xy;
             if (zodd) xz = -xz;
             if (yodd != zodd) yz = -yz;
@@ -529,8 +557,8 @@ __global__ void __launch_bounds__(NT, MINB)
 #pragma unroll
             for (int t = 0; t < L2; ++t) {
                 C y = w[dif_pos<L2>(t)];
-                if (t > 0) y = cmul(y, cconj(tw[t * k1]));
-                s[(c * L1 * L2 + t) * B] = y;
+                if (t > 0) y = cmul(y, cconj(tq[t * L1]));
+                s[c * CP + t * B] = y;
             }
         }
     }
@@ -538,10 +566,10 @@ __global__ void __launch_bounds__(NT, MINB)
 #pragma unroll 1
     for (int i = tid; i < 3 * L2 * B; i += NT) {
         const int b = i % B, ct = i / B, t = ct % L2, c = ct / L2;
-        const C* s = Sm + ((c * L1) * L2 + t) * B + b;
+        const C* s = Sm + c * CP + t * B + b;
         C v[L1];
 #pragma unroll
-        for (int k1 = 0; k1 < L1; ++k1) v[k1] = s[k1 * L2 * B];
+        for (int k1 = 0; k1 < L1; ++k1) v[k1] = s[k1 * LQ * B];
         dif<L1, +1, false>(v);
         C* p = base + c * g.c_s + b;
         if (col0 + b < g.ncol) {

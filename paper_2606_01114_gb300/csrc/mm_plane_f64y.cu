@@ -14,7 +14,7 @@ int plane_yzy_f64(mm_ctx* ctx) {
     if (rc) return rc;
     const ZLine g{3L * ctx->nz * p.P, (long)ctx->nz * p.P, p.P, 6L * ctx->Pz2 * p.KQ, (long)ctx->Pz2 * p.KQ, p.KQ,
                   ctx->nz, p.P, p.P};
-    if ((rc = launch_zline<double, true>(ctx, ctx->Pz, wide, kern, g, p.K, tw + p.off_z))) return rc;
+    if ((rc = launch_zline<double, true>(ctx, ctx->Pz, wide, kern, g, p.K, tw + p.off_z4))) return rc;
     return launch_py<double, +1>(ctx, wide, buf, tw);
 }
 

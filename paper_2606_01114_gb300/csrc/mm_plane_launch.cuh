@@ -61,7 +61,7 @@ int launch_px_fwd(mm_ctx* ctx, const S* in, const S* Ms, T ms, long ms_rows, PC<
             if constexpr (L <= 512) {
                 constexpr int BR = px_rows<T>(L);
                 k_px_fwd<T, S, L1, L2><<<(unsigned)((rows + BR - 1) / BR), px_threads(BR, L1, L2), 0, ctx->stream>>>(
-                    in, ctx->nx, Ms, ms, ms_rows, out, p.R, rows, tw, tw + p.off_p);
+                    in, ctx->nx, Ms, ms, ms_rows, out, p.R, rows, tw + p.off_x4, tw + p.off_p);
             }
         }))
         rc = fail(ctx, MM_ERR_INVALID_ARG, "x length %d", p.L);
@@ -80,7 +80,7 @@ int launch_px_inv(mm_ctx* ctx, const PC<T>* in, S* out, long rows, T scale, cons
             if constexpr (L <= 512) {
                 constexpr int BR = px_rows<T>(L);
                 k_px_inv<T, S, L1, L2><<<(unsigned)((rows + BR - 1) / BR), px_threads(BR, L1, L2), 0, ctx->stream>>>(
-                    in, p.R, out, ctx->nx, rows, scale, tw, tw + p.off_p);
+                    in, p.R, out, ctx->nx, rows, scale, tw + p.off_x4, tw + p.off_p);
             }
         }))
         rc = fail(ctx, MM_ERR_INVALID_ARG, "x length %d", p.L);
@@ -108,7 +108,7 @@ int launch_plane(mm_ctx* ctx, PC<T>* buf, const T* kern, const PC<T>* tw) {
             if (nt > cap) nt = (tasks + (tasks + cap - 1) / cap - 1) / ((tasks + cap - 1) / cap);
             nt = (nt + 31) / 32 * 32;
             if (nt > cap) nt = cap;
-            fn<<<(unsigned)p.K, nt, smem, ctx->stream>>>(buf, kern, ctx->nz, ctx->ny, p.R, p.KQ, tw + p.off_y);
+            fn<<<(unsigned)p.K, nt, smem, ctx->stream>>>(buf, kern, ctx->nz, ctx->ny, p.R, p.KQ, tw + p.off_y4);
         }))
         rc = fail(ctx, MM_ERR_INVALID_ARG, "y length %d", p.P);
     if (rc) return rc;
@@ -129,7 +129,8 @@ int launch_py(mm_ctx* ctx, const PC<T>* in, PC<T>* out, const PC<T>* tw) {
             const size_t smem = (size_t)kPyLines * plane_pitch(L1, L2) * sizeof(PC<T>);
             if ((rc = plane_smem(ctx, (const void*)fn, smem))) return;
             fn<<<(unsigned)((nlines + kPyLines - 1) / kPyLines), (kPyLines * (L1 > L2 ? L1 : L2) + 31) / 32 * 32, smem,
-                 ctx->stream>>>(in, out, lines, nlines, ctx->ny, DIR < 0 ? p.R : wide, DIR < 0 ? wide : p.R, tw + p.off_y);
+                 ctx->stream>>>(in, out, lines, nlines, ctx->ny, DIR < 0 ? p.R : wide, DIR < 0 ? wide : p.R,
+                                                      tw + p.off_y4);
         }))
         rc = fail(ctx, MM_ERR_INVALID_ARG, "y length %d", p.P);
     if (rc) return rc;
@@ -137,16 +138,37 @@ int launch_py(mm_ctx* ctx, const PC<T>* in, PC<T>* out, const PC<T>* tw) {
     return MM_OK;
 }
 
-// columns per block of the z pass: 64-byte row segments where shared memory
-// allows (3 Pz B elements), 256 threads
+// the split of a z length: the middle level holds 3 L2 complex values
+template <typename F> bool with_z_length(int len, F&& f) {
+#define MM_LEN(N, A, B) \
+    case N: f(std::integral_constant<int, A>{}, std::integral_constant<int, B>{}); return true
+    switch (len) {
+        MM_LEN(16, 4, 4);
+        MM_LEN(32, 8, 4);
+        MM_LEN(64, 8, 8);
+        MM_LEN(128, 16, 8);
+        MM_LEN(256, 32, 8);
+        MM_LEN(512, 32, 16);
+        MM_LEN(1024, 32, 32);
+        default: return false;
+    }
+#undef MM_LEN
+}
+
+// B columns per block: 128-byte row segments for short lines, 64 bytes up to
+// Pz = 512 (256^3, Pz = 512: 32-byte segments 1980-2230 us, 64-byte 950 us).
+// NT threads: level 1 has 3 L2 B tasks, the middle level L1 B.  256^3: 384
+// threads 952 us, 256 threads 1050 us (208 registers) or 1450 us (128, two
+// blocks per SM, spills), 128 threads 1243 us; 256 x 256 x 32 (Pz = 64,
+// whole field): 128 threads 194 us, 256 threads 234 us.
 template <typename T, int L1, int L2, bool COLY>
 int launch_zline_t(mm_ctx* ctx, PC<T>* buf, const T* kern, const ZLine& g, int nrows, const PC<T>* tw) {
     constexpr int PZ = L1 * L2, CS = (int)sizeof(PC<T>);
     constexpr int B = PZ <= 64 ? 128 / CS : PZ <= 512 ? 64 / CS : 32 / CS;
-    constexpr int NT = 256;
-    constexpr int MINB = sizeof(T) == 4 && 3 * L2 <= 48 ? 2 : 1;
+    constexpr int NT = sizeof(T) == 8 ? (PZ == 512 ? 192 : 128) : PZ == 64 ? 128 : PZ == 256 ? 256 : PZ >= 512 ? 384 : 192;
+    constexpr int MINB = sizeof(T) == 8 ? 1 : PZ <= 32 ? 4 : PZ == 64 ? 4 : PZ == 128 ? 3 : PZ == 256 ? 2 : 1;
     auto fn = k_zline<T, L1, L2, COLY, B, NT, MINB>;
-    const size_t smem = (size_t)3 * PZ * B * CS;
+    const size_t smem = zline_smem<T, L1, L2, B>();
     int rc = plane_smem(ctx, (const void*)fn, smem);
     if (rc) return rc;
     dim3 grid((unsigned)((g.ncol + B - 1) / B), (unsigned)nrows);
@@ -158,16 +180,12 @@ int launch_zline_t(mm_ctx* ctx, PC<T>* buf, const T* kern, const ZLine& g, int n
 template <typename T, bool COLY>
 int launch_zline(mm_ctx* ctx, int Pz, PC<T>* buf, const T* kern, const ZLine& g, int nrows, const PC<T>* tw) {
     KernelTimer kt(ctx, MM_K_ZCONV);
-    switch (Pz) {
-        case 16: return launch_zline_t<T, 4, 4, COLY>(ctx, buf, kern, g, nrows, tw);
-        case 32: return launch_zline_t<T, 8, 4, COLY>(ctx, buf, kern, g, nrows, tw);
-        case 64: return launch_zline_t<T, 8, 8, COLY>(ctx, buf, kern, g, nrows, tw);
-        case 128: return launch_zline_t<T, 16, 8, COLY>(ctx, buf, kern, g, nrows, tw);
-        case 256: return launch_zline_t<T, 32, 8, COLY>(ctx, buf, kern, g, nrows, tw);
-        case 512: return launch_zline_t<T, 32, 16, COLY>(ctx, buf, kern, g, nrows, tw);
-        case 1024: return launch_zline_t<T, 32, 32, COLY>(ctx, buf, kern, g, nrows, tw);
-        default: return fail(ctx, MM_ERR_INVALID_ARG, "z length %d", Pz);
-    }
+    int rc = MM_OK;
+    if (!with_z_length(Pz, [&](auto A, auto B) {
+            rc = launch_zline_t<T, decltype(A)::value, decltype(B)::value, COLY>(ctx, buf, kern, g, nrows, tw);
+        }))
+        return fail(ctx, MM_ERR_INVALID_ARG, "z length %d", Pz);
+    return rc;
 }
 
 }  // namespace mm

@@ -51,10 +51,13 @@ PLANE = [(2, 2, 1), (2, 3, 2), (17, 8, 4), (16, 9, 1), (33, 17, 2), (40, 21, 1),
          (257, 97, 1), (321, 161, 2), (385, 193, 1), (7, 320, 1), (5, 321, 2), (3, 384, 1), (9, 511, 1), (511, 3, 1)]
 # y, z and y as three kernels: nz above the plane kernel's, every z length
 LINES = [(11, 7, 8), (5, 9, 16), (18, 20, 32), (6, 5, 64), (3, 7, 128), (7, 3, 256), (3, 3, 512), (6, 300, 16)]
+# power-of-two meshes with long z lines: the z pass of the [c][z][y][kx]
+# layout, every z length, a column tile that is not full, nx = 1 and ny = 1
+ZCOLS = [(8, 4, 32), (64, 2, 32), (16, 8, 64), (4, 8, 128), (8, 4, 256), (2, 2, 512), (1, 4, 64), (64, 1, 32)]
 
 
 @pytest.mark.parametrize("prec", ["f64", "f32"])
-@pytest.mark.parametrize("n", PLANE + LINES, ids=lambda n: "x".join(map(str, n)))
+@pytest.mark.parametrize("n", PLANE + LINES + ZCOLS, ids=lambda n: "x".join(map(str, n)))
 def test_demag_on_padded_lengths_matches_oracle(n, prec):
     p = micromag.Problem(n, D)
     m = wl.random_unit(n, seed=sum(n))
