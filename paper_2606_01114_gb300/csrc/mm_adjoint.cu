@@ -85,6 +85,7 @@ __global__ void k_vjp_norm(Params<T> p, const T* __restrict__ m0, const T* __res
                            const T* __restrict__ k2, const T* __restrict__ x3, const T* __restrict__ hd3, T dt,
                            T* __restrict__ lam, T* __restrict__ lk0, T* __restrict__ lk1, T* __restrict__ lk2,
                            T* __restrict__ lk3) {
+    dep_wait();
     long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= p.N) return;
     int x, y, z;
@@ -120,6 +121,7 @@ __global__ void k_vjp_norm(Params<T> p, const T* __restrict__ m0, const T* __res
 template <typename T>
 __global__ void k_vjp_rhs_a(Params<T> p, const T* __restrict__ X, const T* __restrict__ hd, const T* __restrict__ w,
                             T* __restrict__ G, T* __restrict__ P) {
+    dep_wait();
     long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= p.N) return;
     int x, y, z;
@@ -151,6 +153,7 @@ template <typename T>
 __global__ void k_vjp_rhs_b(Params<T> p, const T* __restrict__ X, const T* __restrict__ G, const T* __restrict__ P,
                             const T* __restrict__ D, T* __restrict__ lam, T* __restrict__ lk_prev, T coef,
                             T* __restrict__ gMs) {
+    dep_wait();
     long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= p.N) return;
     int x, y, z;
@@ -183,6 +186,7 @@ __global__ void k_vjp_rhs_b(Params<T> p, const T* __restrict__ X, const T* __res
 template <typename T>
 __global__ void k_demag_vjp(Params<T> p, const T* __restrict__ m, const T* __restrict__ D, T* __restrict__ gm,
                             T* __restrict__ gMs) {
+    dep_wait();
     long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= p.N) return;
     const T Msi = ms_at(p, i);
@@ -194,6 +198,7 @@ __global__ void k_demag_vjp(Params<T> p, const T* __restrict__ m, const T* __res
 template <typename T>
 __global__ void k_exchange_vjp(Params<T> p, const T* __restrict__ m, const T* __restrict__ g, T* __restrict__ gm,
                                T* __restrict__ gMs) {
+    dep_wait();
     long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= p.N) return;
     int x, y, z;
@@ -295,7 +300,7 @@ int step_vjp(mm_ctx* ctx, const T* m0, double dt, T* lam, T* gMs, const StepTape
     Params<T> p = make_params<T>(ctx);
     {
         KernelTimer kt(ctx, MM_K_STAGE);
-        k_vjp_norm<T><<<nblk(ctx->N), kT, 0, ctx->stream>>>(p, m0, kk[0], kk[1], kk[2], X[3], Hst[3], (T)dt, lam,
+        dep(k_vjp_norm<T>, nblk(ctx->N), kT, 0, ctx->stream)(p, m0, kk[0], kk[1], kk[2], X[3], Hst[3], (T)dt, lam,
                                                             lk[0], lk[1], lk[2], lk[3]);
         MM_LAUNCH_CHECK(ctx);
     }
@@ -304,13 +309,13 @@ int step_vjp(mm_ctx* ctx, const T* m0, double dt, T* lam, T* gMs, const StepTape
     for (int s = 3; s >= 0; --s) {
         {
             KernelTimer kt(ctx, MM_K_STAGE);
-            k_vjp_rhs_a<T><<<nblk(ctx->N), kT, 0, ctx->stream>>>(p, X[s], Hst[s], lk[s], G, P);
+            dep(k_vjp_rhs_a<T>, nblk(ctx->N), kT, 0, ctx->stream)(p, X[s], Hst[s], lk[s], G, P);
             MM_LAUNCH_CHECK(ctx);
         }
         if ((rc = demag_apply_unit(ctx, G, D))) return rc;
         {
             KernelTimer kt(ctx, MM_K_STAGE);
-            k_vjp_rhs_b<T><<<nblk(ctx->N), kT, 0, ctx->stream>>>(p, X[s], G, P, D, lam, s > 0 ? lk[s - 1] : nullptr,
+            dep(k_vjp_rhs_b<T>, nblk(ctx->N), kT, 0, ctx->stream)(p, X[s], G, P, D, lam, s > 0 ? lk[s - 1] : nullptr,
                                                                  (T)coef[s], gMs);
             MM_LAUNCH_CHECK(ctx);
         }
@@ -326,7 +331,7 @@ int demag_vjp_t(mm_ctx* ctx, const T* g, const T* m, T* gm, T* gMs) {
     if ((rc = demag_apply_unit(ctx, g, D))) return rc;
     Params<T> p = make_params<T>(ctx);
     KernelTimer kt(ctx, MM_K_REDUCE);
-    k_demag_vjp<T><<<nblk(ctx->N), kT, 0, ctx->stream>>>(p, m, D, gm, gMs);
+    dep(k_demag_vjp<T>, nblk(ctx->N), kT, 0, ctx->stream)(p, m, D, gm, gMs);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
@@ -335,7 +340,7 @@ template <typename T>
 int exchange_vjp_t(mm_ctx* ctx, const T* g, const T* m, T* gm, T* gMs) {
     Params<T> p = make_params<T>(ctx);
     KernelTimer kt(ctx, MM_K_REDUCE);
-    k_exchange_vjp<T><<<nblk(ctx->N), kT, 0, ctx->stream>>>(p, m, g, gm, gMs);
+    dep(k_exchange_vjp<T>, nblk(ctx->N), kT, 0, ctx->stream)(p, m, g, gm, gMs);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }

@@ -69,6 +69,7 @@ template <typename T, typename S = T, bool HIN = false>
 __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512) k_xfwd(const S* __restrict__ in, long in_ld, int nin, const S* __restrict__ Ms, T ms,
                        long ms_rows, C_t<T>* __restrict__ out, int Hs, int lgL, long rows, int lgB,
                        const C_t<T>* __restrict__ twL, const C_t<T>* __restrict__ twP) {
+    dep_wait();
     using C = C_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* s = reinterpret_cast<C*>(smem_raw);
@@ -125,6 +126,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512) k_xfwd(const S* _
 template <typename T, typename S = T>
 __global__ void k_x1fwd(const S* __restrict__ in, const S* __restrict__ Ms, T ms, long ms_rows,
                         C_t<T>* __restrict__ out, int Hs, long rows) {
+    dep_wait();
     long r = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= rows) return;
     T w = Ms ? ld_r<T>(Ms[r % ms_rows]) : ms;
@@ -136,6 +138,7 @@ __global__ void k_x1fwd(const S* __restrict__ in, const S* __restrict__ Ms, T ms
 template <typename T, typename S = T>
 __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512) k_xinv(const C_t<T>* __restrict__ in, int Hs, S* __restrict__ out, int nx, int lgL, long rows,
                        int lgB, T scale, const C_t<T>* __restrict__ twL, const C_t<T>* __restrict__ twP) {
+    dep_wait();
     using C = C_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* s = reinterpret_cast<C*>(smem_raw);
@@ -183,6 +186,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512) k_xinv(const C_t<
 
 template <typename T, typename S = T>
 __global__ void k_x1inv(const C_t<T>* __restrict__ in, int Hs, S* __restrict__ out, long rows, T scale) {
+    dep_wait();
     long r = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= rows) return;
     out[r] = to_d(in[r * Hs].x * scale);
@@ -197,6 +201,7 @@ __global__ void k_x1inv(const C_t<T>* __restrict__ in, int Hs, S* __restrict__ o
 template <typename T, int DIR, bool HIN = false, bool HOUT = false>
 __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512) k_cols(const C_t<T>* in, C_t<T>* out, int lgL, int nin, int nout, int Hx, int lgB, ColGeom cg,
                        const C_t<T>* __restrict__ tw) {
+    dep_wait();
     using C = C_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* s = reinterpret_cast<C*>(smem_raw);
@@ -298,6 +303,7 @@ template <typename T>
 __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512)
     k_zconv(C_t<T>* buf, const T* __restrict__ kern, int nz, int lgPz, int Py, int Hs, int Hx, int Py2, int Pz2,
             int lgB, const C_t<T>* __restrict__ twz) {
+    dep_wait();
     using C = C_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* s = reinterpret_cast<C*>(smem_raw);
@@ -609,6 +615,7 @@ __device__ __forceinline__ void zconv_product(float2 (&v)[PZ], const float2* S, 
 template <int PZ>
 __global__ void __launch_bounds__(3 * kZB, PZ >= 32 ? 7 : 8)
     k_zconv_reg(float2* buf, const float* __restrict__ kern, int Py, int Hs, int c0, int Hx, int Py2) {
+    dep_wait();
     constexpr int NZ = PZ > 1 ? PZ / 2 : 1;
     constexpr int PZ2 = PZ / 2 + 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -678,6 +685,7 @@ template <int L1, int L2>
 __global__ void __launch_bounds__(128, (L1 * L2 >= 512) ? 6 : 8)
     k_xinv_reg(const float2* __restrict__ in, int Hs, float* __restrict__ out, long rows, float scale,
                const float2* __restrict__ twL, const float2* __restrict__ twP) {
+    dep_wait();
     constexpr int L = L1 * L2, B = 4, NX = L;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* S = reinterpret_cast<float2*>(smem_raw);      // [B][L]
@@ -752,6 +760,7 @@ template <int L1, int L2>
 __global__ void __launch_bounds__(128, 6)
     k_xinv_pk(const float2* __restrict__ in, int Hs, float* __restrict__ out, long rows, float scale,
               const float2* __restrict__ twL, const float2* __restrict__ twP) {
+    dep_wait();
     constexpr int L = L1 * L2, B = 4, NX = L;
     static_assert(B * L2 == 128, "level 1 takes every thread");
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -823,6 +832,7 @@ __global__ void __launch_bounds__(128, 7)
     k_xfwd_reg(const float* __restrict__ in, const float* __restrict__ Ms, float ms, long ms_rows,
                 float2* __restrict__ out, int Hs, long rows, const float2* __restrict__ twL,
                 const float2* __restrict__ twP) {
+    dep_wait();
     constexpr int L = L1 * L2, B = 4, NX = L;
     static_assert(32 % L1 == 0 || L1 % 32 == 0, "rows must not straddle warps unevenly");
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -951,6 +961,7 @@ constexpr long kTmaWaitLimit = 1L << 24;   // polls of a TMA-fed pass's mbarrier
 __global__ void __launch_bounds__(128, 6)
     k_xinv_tma(const float2* __restrict__ in, float* __restrict__ out, long rows, int ntiles, float scale,
                const float2* __restrict__ twL, const float2* __restrict__ twP, int* __restrict__ status) {
+    dep_wait();
     constexpr int L1 = 16, L2 = 32, L = L1 * L2, B = kXB, NX = L, S = 2, HS = kXHs;
     constexpr int STAGE = B * HS;                  // float2 per stage (>= B L)
     static_assert(B * HS >= B * L && (B * HS * 8) % 128 == 0, "stage holds the input tile and the transpose");
@@ -1058,6 +1069,7 @@ __global__ void __launch_bounds__(128, 6)
 template <int L1, int L2, int DIR, bool PIN, bool POUT>
 __global__ void __launch_bounds__(256)
     k_cols_reg(const float2* in, float2* out, int c0, int Hx, int lgB, ColGeom cg, const float2* __restrict__ tw) {
+    dep_wait();
     constexpr int L = L1 * L2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* S = reinterpret_cast<float2*>(smem_raw);      // [L1][L2][B]
@@ -1125,6 +1137,7 @@ template <int L1, int L2, int DIR, bool PIN, bool POUT>
 __global__ void __launch_bounds__(kYB * (L1 > L2 ? L1 : L2), L1 * L2 >= 1024 ? 1 : 2)
     k_cols_tma(const __grid_constant__ CUtensorMap tin, float2* __restrict__ out, int Hx, int ntx, int ntiles,
                long rs_out, long out_plane, const float2* __restrict__ tw, int* __restrict__ status) {
+    dep_wait();
     constexpr int L = L1 * L2, B = kYB, S = kYStages;
     constexpr int NIN = PIN ? L / 2 : L;
     constexpr int BOX = NIN < 256 ? NIN : 256;
@@ -1289,14 +1302,14 @@ int launch_xfwd_reg(mm_ctx* ctx, const float* in, const float* Ms, float ms, lon
         // level 1 split by output parity over all 128 threads: 39.0 -> 33.4 us on the 512 x 512 x 16 film
         int rc = set_smem(ctx, (const void*)k_xfwd_reg<L1, L2, true>, smem);
         if (rc) return rc;
-        k_xfwd_reg<L1, L2, true><<<(unsigned)((rows + B - 1) / B), B * L1, smem, ctx->stream>>>(
+        dep(k_xfwd_reg<L1, L2, true>, (unsigned)((rows + B - 1) / B), B * L1, smem, ctx->stream)(
             in, Ms, ms, ms_rows, out, ctx->Hs, rows, twL, twP);
         MM_LAUNCH_CHECK(ctx);
         return MM_OK;
     }
     int rc = set_smem(ctx, (const void*)k_xfwd_reg<L1, L2>, smem);
     if (rc) return rc;
-    k_xfwd_reg<L1, L2><<<(unsigned)((rows + B - 1) / B), B * L1, smem, ctx->stream>>>(in, Ms, ms, ms_rows, out,
+    dep(k_xfwd_reg<L1, L2>, (unsigned)((rows + B - 1) / B), B * L1, smem, ctx->stream)(in, Ms, ms, ms_rows, out,
                                                                                    ctx->Hs, rows, twL, twP);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
@@ -1328,14 +1341,14 @@ int launch_xinv_reg(mm_ctx* ctx, const float2* in, float* out, long rows, float 
         // 16 x 32 with the packing folded into the level-1 loads: 53.3 -> 35.5 us on the 512 x 512 x 16 film
         int rc = set_smem(ctx, (const void*)k_xinv_pk<16, 32>, smem);
         if (rc) return rc;
-        k_xinv_pk<16, 32><<<(unsigned)((rows + B - 1) / B), 128, smem, ctx->stream>>>(in, ctx->Hs, out, rows, scale,
+        dep(k_xinv_pk<16, 32>, (unsigned)((rows + B - 1) / B), 128, smem, ctx->stream)(in, ctx->Hs, out, rows, scale,
                                                                                      twL, twP);
         MM_LAUNCH_CHECK(ctx);
         return MM_OK;
     }
     int rc = set_smem(ctx, (const void*)k_xinv_reg<L1, L2>, smem);
     if (rc) return rc;
-    k_xinv_reg<L1, L2><<<(unsigned)((rows + B - 1) / B), B * L1, smem, ctx->stream>>>(in, ctx->Hs, out, rows, scale,
+    dep(k_xinv_reg<L1, L2>, (unsigned)((rows + B - 1) / B), B * L1, smem, ctx->stream)(in, ctx->Hs, out, rows, scale,
                                                                                    twL, twP);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
@@ -1399,7 +1412,7 @@ int run_xfwd(mm_ctx* ctx, const T* in, long in_ld, int nin, const T* Ms, T ms, l
     }
     KernelTimer kt(ctx, MM_K_XFWD);
     if (Px == 1) {
-        k_x1fwd<T><<<(unsigned)((rows + 255) / 256), 256, 0, ctx->stream>>>(in, Ms, ms, ms_rows, out, ctx->Hs, rows);
+        dep(k_x1fwd<T>, (unsigned)((rows + 255) / 256), 256, 0, ctx->stream)(in, Ms, ms, ms_rows, out, ctx->Hs, rows);
         MM_LAUNCH_CHECK(ctx);
         return MM_OK;
     }
@@ -1416,7 +1429,7 @@ int run_xfwd(mm_ctx* ctx, const T* in, long in_ld, int nin, const T* Ms, T ms, l
     auto fn = nin <= L ? k_xfwd<T, T, true> : k_xfwd<T, T, false>;
     int rc = set_smem(ctx, (const void*)fn, smem);
     if (rc) return rc;
-    fn<<<(unsigned)((rows + B - 1) / B), block_threads(B * L / 8), smem, ctx->stream>>>(
+    dep(fn, (unsigned)((rows + B - 1) / B), block_threads(B * L / 8), smem, ctx->stream)(
         in, in_ld, nin, Ms, ms, ms_rows, out, ctx->Hs, ilog2(L), rows, ilog2(B), twL, twP);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
@@ -1434,7 +1447,7 @@ int launch_cols_reg(mm_ctx* ctx, const float2* in, float2* out, int nplanes, Col
     int rc = set_smem(ctx, (const void*)fn, smem);
     if (rc) return rc;
     dim3 grid((unsigned)((c1 - c0 + B - 1) / B), (unsigned)nplanes);
-    fn<<<grid, B * (L1 > L2 ? L1 : L2), smem, ctx->stream>>>(in, out, c0, c1, 3, g, tw);
+    dep(fn, grid, B * (L1 > L2 ? L1 : L2), smem, ctx->stream)(in, out, c0, c1, 3, g, tw);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
@@ -1526,11 +1539,11 @@ int try_cols_tma(mm_ctx* ctx, const float2* in, float2* out, int L, int nplanes,
     int* status = &ctx->ctl->status;
     if (L == 1024) {
         auto fn = cols_tma_fn<32, 32, DIR>();
-        fn<<<grid, kYB * 32, cols_tma_smem<32, 32>(), ctx->stream>>>(map, out, ctx->Hx, ntx, ntiles, g.rs_out,
+        dep(fn, grid, kYB * 32, cols_tma_smem<32, 32>(), ctx->stream)(map, out, ctx->Hx, ntx, ntiles, g.rs_out,
                                                                      g.out_inner, tw, status);
     } else {
         auto fn = cols_tma_fn<32, 16, DIR>();
-        fn<<<grid, kYB * 32, cols_tma_smem<32, 16>(), ctx->stream>>>(map, out, ctx->Hx, ntx, ntiles, g.rs_out,
+        dep(fn, grid, kYB * 32, cols_tma_smem<32, 16>(), ctx->stream)(map, out, ctx->Hx, ntx, ntiles, g.rs_out,
                                                                      g.out_inner, tw, status);
     }
     *done = true;
@@ -1582,7 +1595,7 @@ int run_cols(mm_ctx* ctx, const C_t<T>* in, C_t<T>* out, int L, int nin, int nou
     int rc = set_smem(ctx, (const void*)fn, smem);
     if (rc) return rc;
     dim3 grid((unsigned)((ctx->Hx + B - 1) / B), (unsigned)nplanes);
-    fn<<<grid, block_threads(B * L / 8), smem, ctx->stream>>>(in, out, ilog2(L), nin, nout, ctx->Hx,
+    dep(fn, grid, block_threads(B * L / 8), smem, ctx->stream)(in, out, ilog2(L), nin, nout, ctx->Hx,
                                                                           ilog2(B), g, tw);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
@@ -1596,7 +1609,7 @@ int launch_zconv_reg_t(mm_ctx* ctx, float2* buf, const float* kern, int c0, int 
     int rc = set_smem(ctx, (const void*)k_zconv_reg<PZ>, smem);
     if (rc) return rc;
     dim3 grid((unsigned)((c1 - c0 + kZB - 1) / kZB), (unsigned)ctx->Py);
-    k_zconv_reg<PZ><<<grid, 3 * kZB, smem, ctx->stream>>>(buf, kern, ctx->Py, ctx->Hs, c0, c1, ctx->Py2);
+    dep(k_zconv_reg<PZ>, grid, 3 * kZB, smem, ctx->stream)(buf, kern, ctx->Py, ctx->Hs, c0, c1, ctx->Py2);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
@@ -1660,7 +1673,7 @@ int apply(mm_ctx* ctx, const T* m, T* H, bool unit = false) {
         rc = set_smem(ctx, (const void*)k_zconv<T>, smem);
         if (rc) return rc;
         dim3 grid((unsigned)((ctx->Hx + B - 1) / B), (unsigned)(ctx->Py / 2 + 1));
-        k_zconv<T><<<grid, block_threads(3 * B * Pz / 8), smem, ctx->stream>>>(
+        dep(k_zconv<T>, grid, block_threads(3 * B * Pz / 8), smem, ctx->stream)(
             Bf, (const T*)ctx->kern, ctx->nz, ilog2(Pz), ctx->Py, ctx->Hs, ctx->Hx, ctx->Py2, ctx->Pz2, ilog2(B),
             table<T>(ctx, ctx->tw.off_pz));
         MM_LAUNCH_CHECK(ctx);
@@ -1701,7 +1714,7 @@ int xinv_pass(mm_ctx* ctx, const C_t<T>* xin, T* H, long rows) {
         return MM_OK;
     }
     if (ctx->Px == 1) {
-        k_x1inv<T><<<(unsigned)((rows + 255) / 256), 256, 0, ctx->stream>>>(xin, ctx->Hs, H, rows, scale);
+        dep(k_x1inv<T>, (unsigned)((rows + 255) / 256), 256, 0, ctx->stream)(xin, ctx->Hs, H, rows, scale);
         MM_LAUNCH_CHECK(ctx);
     } else {
         const int L = ctx->Lx;
@@ -1711,7 +1724,7 @@ int xinv_pass(mm_ctx* ctx, const C_t<T>* xin, T* H, long rows) {
                 if (ctx->xtma_state == 1) {
                     const int ntiles = (int)((rows + kXB - 1) / kXB);
                     const int grid = ctx->xtma_grid < ntiles ? ctx->xtma_grid : ntiles;
-                    k_xinv_tma<<<grid, 128, kXinvTmaSmem, ctx->stream>>>(
+                    dep(k_xinv_tma, grid, 128, kXinvTmaSmem, ctx->stream)(
                         (const float2*)xin, (float*)H, rows, ntiles, (float)scale,
                         (const float2*)table<T>(ctx, ctx->tw.off_lx), (const float2*)table<T>(ctx, ctx->tw.off_px),
                         &ctx->ctl->status);
@@ -1731,7 +1744,7 @@ int xinv_pass(mm_ctx* ctx, const C_t<T>* xin, T* H, long rows) {
         size_t smem = (size_t)L * B * sizeof(C);
         rc = set_smem(ctx, (const void*)k_xinv<T>, smem);
         if (rc) return rc;
-        k_xinv<T><<<(unsigned)((rows + B - 1) / B), block_threads(B * L / 8), smem, ctx->stream>>>(
+        dep(k_xinv<T>, (unsigned)((rows + B - 1) / B), block_threads(B * L / 8), smem, ctx->stream)(
             xin, ctx->Hs, H, ctx->nx, ilog2(L), rows, ilog2(B), scale, table<T>(ctx, ctx->tw.off_lx),
             table<T>(ctx, ctx->tw.off_px));
         MM_LAUNCH_CHECK(ctx);
@@ -1825,7 +1838,7 @@ int apply_ff(mm_ctx* ctx, const double* m, double* H, bool unit) {
     {   // K2
         KernelTimer kt(ctx, MM_K_XFWD);
         if (ctx->Px == 1) {
-            k_x1fwd<ff, double><<<(unsigned)((rows + 255) / 256), 256, 0, ctx->stream>>>(m, Ms, ms, ms_rows, xout,
+            dep(k_x1fwd<ff, double>, (unsigned)((rows + 255) / 256), 256, 0, ctx->stream)(m, Ms, ms, ms_rows, xout,
                                                                                       ctx->Hs, rows);
         } else {
             const int L = ctx->Px / 2;
@@ -1833,7 +1846,7 @@ int apply_ff(mm_ctx* ctx, const double* m, double* H, bool unit) {
             const size_t smem = (size_t)L * B * sizeof(C);
             // nin = nx = L: the upper half of each packed line is zero padding
             if ((rc = set_smem(ctx, (const void*)k_xfwd<ff, double, true>, smem))) return rc;
-            k_xfwd<ff, double, true><<<(unsigned)((rows + B - 1) / B), block_threads(B * L / 8), smem, ctx->stream>>>(
+            dep(k_xfwd<ff, double, true>, (unsigned)((rows + B - 1) / B), block_threads(B * L / 8), smem, ctx->stream)(
                 m, ctx->nx, ctx->nx, Ms, ms, ms_rows, xout, ctx->Hs, ilog2(L), rows, ilog2(B), tw + ctx->tw.off_lx,
                 tw + ctx->tw.off_px);
         }
@@ -1852,7 +1865,7 @@ int apply_ff(mm_ctx* ctx, const double* m, double* H, bool unit) {
         const size_t smem = (size_t)3 * Pz * B * sizeof(C) + (size_t)6 * ctx->Pz2 * B * sizeof(ff);
         if ((rc = set_smem(ctx, (const void*)k_zconv<ff>, smem))) return rc;
         dim3 grid((unsigned)((ctx->Hx + B - 1) / B), (unsigned)(ctx->Py / 2 + 1));
-        k_zconv<ff><<<grid, block_threads(3 * B * Pz / 8), smem, ctx->stream>>>(
+        dep(k_zconv<ff>, grid, block_threads(3 * B * Pz / 8), smem, ctx->stream)(
             Bf, (const ff*)ctx->kern_ff, ctx->nz, ilog2(Pz), ctx->Py, ctx->Hs, ctx->Hx, ctx->Py2, ctx->Pz2, ilog2(B),
             tw + ctx->tw.off_pz);
         MM_LAUNCH_CHECK(ctx);
@@ -1868,13 +1881,13 @@ int apply_ff(mm_ctx* ctx, const double* m, double* H, bool unit) {
         const ff scale = ff(1.0 / ((double)ctx->Lx * ctx->Py * ctx->Pz));
         KernelTimer kt(ctx, MM_K_XINV);
         if (ctx->Px == 1) {
-            k_x1inv<ff, double><<<(unsigned)((rows + 255) / 256), 256, 0, ctx->stream>>>(xin, ctx->Hs, H, rows, scale);
+            dep(k_x1inv<ff, double>, (unsigned)((rows + 255) / 256), 256, 0, ctx->stream)(xin, ctx->Hs, H, rows, scale);
         } else {
             const int L = ctx->Lx;
             const int B = x_rows_per_block(L);
             const size_t smem = (size_t)L * B * sizeof(C);
             if ((rc = set_smem(ctx, (const void*)k_xinv<ff, double>, smem))) return rc;
-            k_xinv<ff, double><<<(unsigned)((rows + B - 1) / B), block_threads(B * L / 8), smem, ctx->stream>>>(
+            dep(k_xinv<ff, double>, (unsigned)((rows + B - 1) / B), block_threads(B * L / 8), smem, ctx->stream)(
                 xin, ctx->Hs, H, ctx->nx, ilog2(L), rows, ilog2(B), scale, tw + ctx->tw.off_lx, tw + ctx->tw.off_px);
         }
         MM_LAUNCH_CHECK(ctx);

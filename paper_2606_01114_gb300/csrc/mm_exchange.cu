@@ -38,6 +38,7 @@ template <int MODE>
 __global__ void __launch_bounds__(256) k_field4(Params<float> p, float wx, float wy, float wz,
                                                 const float* __restrict__ m, const float* __restrict__ Hd,
                                                 float* __restrict__ H) {
+    dep_wait();
     const long i = 4 * ((long)blockIdx.x * blockDim.x + threadIdx.x);
     const long N = p.N;
     if (i >= N) return;
@@ -94,10 +95,10 @@ int field4(mm_ctx* ctx, const void* m, const void* Hd, void* H, bool effective, 
     const long quads = ctx->N / 4;
     const unsigned blocks = (unsigned)((quads + 255) / 256);
     if (effective)
-        k_field4<1><<<blocks, 256, 0, ctx->stream>>>(p, p.A * p.cx * inv, p.A * p.cy * inv, p.A * p.cz * inv,
+        dep(k_field4<1>, blocks, 256, 0, ctx->stream)(p, p.A * p.cx * inv, p.A * p.cy * inv, p.A * p.cz * inv,
                                                      (const float*)m, (const float*)Hd, (float*)H);
     else
-        k_field4<0><<<blocks, 256, 0, ctx->stream>>>(p, p.A * p.cx * inv, p.A * p.cy * inv, p.A * p.cz * inv,
+        dep(k_field4<0>, blocks, 256, 0, ctx->stream)(p, p.A * p.cx * inv, p.A * p.cy * inv, p.A * p.cz * inv,
                                                      (const float*)m, nullptr, (float*)H);
     *done = true;
     MM_LAUNCH_CHECK(ctx);

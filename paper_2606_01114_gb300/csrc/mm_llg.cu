@@ -125,6 +125,7 @@ __device__ __forceinline__ double block_reduce_t(T v, bool is_max) {
 // mode 0: exchange only; mode 1: Hd + exchange + anisotropy + Zeeman
 template <typename T, int MODE>
 __global__ void k_field(Params<T> p, const T* __restrict__ m, const T* __restrict__ Hd, T* __restrict__ H) {
+    dep_wait();
     long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= p.N) return;
     int x, y, z;
@@ -153,6 +154,7 @@ __global__ void k_field(Params<T> p, const T* __restrict__ m, const T* __restric
 template <typename T, int METHOD, int S>
 __global__ void k_stage(Params<T> p, const T* __restrict__ m_in, const T* __restrict__ Hd, const T* m0,
                         T* const* __restrict__ kbuf, T* m_out, Control* ctl) {
+    dep_wait();
     constexpr int NS = rk_stages(METHOD);
     constexpr bool LAST = (S == NS - 1);
     if (ctl->status != 0 || ctl->done) return;
@@ -274,6 +276,7 @@ template <int METHOD, int S>
 __global__ void __launch_bounds__(256) k_stage4(Params<float> p, float wx, float wy, float wz,
                                                 const float* __restrict__ m_in, const float* __restrict__ Hd,
                                                 const float* m0, KPtrs kb, float* m_out, Control* ctl) {
+    dep_wait();
     constexpr int NS = rk_stages(METHOD);
     constexpr bool LAST = (S == NS - 1);
     if (ctl->status != 0 || ctl->done) return;
@@ -435,6 +438,7 @@ template <int METHOD, int S>
 __global__ void __launch_bounds__(256)
     k_stage_ff(FFStageCoef c, int nx, int ny, int nz, long N, const double* __restrict__ m_in,
                const double* __restrict__ Hd, const double* m0, KPtrsD kb, double* m_out, Control* ctl) {
+    dep_wait();
     constexpr int NS = rk_stages(METHOD);
     constexpr bool LAST = (S == NS - 1);
     if (ctl->status != 0 || ctl->done) return;
@@ -547,6 +551,7 @@ __global__ void __launch_bounds__(256)
 
 // RKF45 step control on the device.
 __global__ void k_controller(Control* ctl, int method) {
+    dep_wait();
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     if (ctl->status != 0 || ctl->done) {
         ctl->accepted = 0;
@@ -592,6 +597,7 @@ __global__ void k_controller(Control* ctl, int method) {
 
 template <typename T>
 __global__ void k_commit(long n3, const T* __restrict__ src, T* __restrict__ dst, const Control* ctl) {
+    dep_wait();
     if (!ctl->accepted) return;
     long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n3) dst[i] = src[i];
@@ -601,6 +607,7 @@ __global__ void k_commit(long n3, const T* __restrict__ src, T* __restrict__ dst
 template <typename T>
 __global__ void k_energy(Params<T> p, const T* __restrict__ m, const T* __restrict__ Hd, double V, double mu0,
                          double Ku, Control* ctl) {
+    dep_wait();
     long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     double ed = 0, ex = 0, ea = 0, ez = 0, em = 0;
     if (i < p.N) {
@@ -636,6 +643,7 @@ __global__ void k_energy(Params<T> p, const T* __restrict__ m, const T* __restri
 
 template <typename T>
 __global__ void k_torque(Params<T> p, const T* __restrict__ m, const T* __restrict__ Hd, Control* ctl) {
+    dep_wait();
     long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     double tq = 0.0;
     if (i < p.N) {
@@ -661,6 +669,7 @@ __global__ void k_torque(Params<T> p, const T* __restrict__ m, const T* __restri
 
 template <typename T>
 __global__ void k_finite(long n3, const T* __restrict__ m, Control* ctl) {
+    dep_wait();
     long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n3 && !isfinite((double)m[i])) atomicCAS(&ctl->status, 0, (int)MM_ERR_NONFINITE);
 }
@@ -681,6 +690,7 @@ constexpr double kBBTau0 = 1e-4, kBBTauMax = 1.0;
 template <typename T>
 __global__ void k_bb_grad(Params<T> p, const T* __restrict__ m, const T* __restrict__ Hd, T* __restrict__ g,
                           const T* __restrict__ g_prev, const T* __restrict__ m_prev, int have_prev, Control* ctl) {
+    dep_wait();
     if (ctl->status != 0 || ctl->done) return;
     long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     T tq2 = 0, ss = 0, sy = 0, yy = 0;   // squared torque and the BB sums, in the path's type
@@ -734,6 +744,7 @@ __global__ void k_bb_grad(Params<T> p, const T* __restrict__ m, const T* __restr
 
 // stop test and step length; ctl->dt carries tau to the update
 __global__ void k_bb_tau(Control* ctl, double torque_tol, long max_iter) {
+    dep_wait();
     if (threadIdx.x != 0 || blockIdx.x != 0 || ctl->status != 0 || ctl->done) return;
     const double tq = __longlong_as_double((long long)ctl->torque_bits);
     const long k = (long)ctl->steps;
@@ -755,6 +766,7 @@ __global__ void k_bb_tau(Control* ctl, double torque_tol, long max_iter) {
 template <typename T>
 __global__ void k_bb_update(Params<T> p, T* __restrict__ m, const T* __restrict__ g, T* __restrict__ m_prev,
                             const Control* ctl) {
+    dep_wait();
     if (ctl->status != 0 || ctl->done) return;
     long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= p.N) return;
@@ -791,7 +803,7 @@ int launch_stage(mm_ctx* ctx, const Params<T>& p, const void* m_in, const void* 
             c.hz = ff((double)p.hz);
             c.pref = ff((double)p.pref);
             c.alpha = ff((double)p.alpha);
-            k_stage_ff<METHOD, S><<<blocks_for(p.N), kThreads, 0, ctx->stream>>>(
+            dep(k_stage_ff<METHOD, S>, blocks_for(p.N), kThreads, 0, ctx->stream)(
                 c, p.nx, p.ny, p.nz, p.N, (const double*)m_in, (const double*)ctx->Hd, (const double*)m0, kb,
                 (double*)m_out, ctx->ctl);
             MM_LAUNCH_CHECK(ctx);
@@ -803,14 +815,14 @@ int launch_stage(mm_ctx* ctx, const Params<T>& p, const void* m_in, const void* 
             KPtrs kb;
             for (int s = 0; s < 6; ++s) kb.k[s] = (float*)ctx->k[s];
             const float inv = 1.f / p.Ms;
-            k_stage4<METHOD, S><<<blocks_for(p.N / 4), kThreads, 0, ctx->stream>>>(
+            dep(k_stage4<METHOD, S>, blocks_for(p.N / 4), kThreads, 0, ctx->stream)(
                 p, p.A * p.cx * inv, p.A * p.cy * inv, p.A * p.cz * inv, (const float*)m_in, (const float*)ctx->Hd,
                 (const float*)m0, kb, (float*)m_out, ctx->ctl);
             MM_LAUNCH_CHECK(ctx);
             return MM_OK;
         }
     }
-    k_stage<T, METHOD, S><<<blocks_for(p.N), kThreads, 0, ctx->stream>>>(p, (const T*)m_in, (const T*)ctx->Hd,
+    dep(k_stage<T, METHOD, S>, blocks_for(p.N), kThreads, 0, ctx->stream)(p, (const T*)m_in, (const T*)ctx->Hd,
                                                                           (const T*)m0, kdev, (T*)m_out, ctx->ctl);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
@@ -839,7 +851,7 @@ template <typename T>
 int exchange_t(mm_ctx* ctx, const void* m, void* H) {
     KernelTimer kt(ctx, MM_K_REDUCE);
     Params<T> p = make_params<T>(ctx);
-    k_field<T, 0><<<blocks_for(p.N), kThreads, 0, ctx->stream>>>(p, (const T*)m, nullptr, (T*)H);
+    dep(k_field<T, 0>, blocks_for(p.N), kThreads, 0, ctx->stream)(p, (const T*)m, nullptr, (T*)H);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
@@ -847,7 +859,7 @@ template <typename T>
 int effective_t(mm_ctx* ctx, const void* m, const void* Hd, void* H) {
     KernelTimer kt(ctx, MM_K_REDUCE);
     Params<T> p = make_params<T>(ctx);
-    k_field<T, 1><<<blocks_for(p.N), kThreads, 0, ctx->stream>>>(p, (const T*)m, (const T*)Hd, (T*)H);
+    dep(k_field<T, 1>, blocks_for(p.N), kThreads, 0, ctx->stream)(p, (const T*)m, (const T*)Hd, (T*)H);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
@@ -856,7 +868,7 @@ int energy_t(mm_ctx* ctx, const void* m, const void* Hd) {
     KernelTimer kt(ctx, MM_K_REDUCE);
     Params<T> p = make_params<T>(ctx);
     double V = ctx->dx * ctx->dy * ctx->dz;
-    k_energy<T><<<blocks_for(p.N), kThreads, 0, ctx->stream>>>(p, (const T*)m, (const T*)Hd, V, kMu0, ctx->Ku, ctx->ctl);
+    dep(k_energy<T>, blocks_for(p.N), kThreads, 0, ctx->stream)(p, (const T*)m, (const T*)Hd, V, kMu0, ctx->Ku, ctx->ctl);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
@@ -864,7 +876,7 @@ template <typename T>
 int torque_t(mm_ctx* ctx, const void* m, const void* Hd) {
     KernelTimer kt(ctx, MM_K_REDUCE);
     Params<T> p = make_params<T>(ctx);
-    k_torque<T><<<blocks_for(p.N), kThreads, 0, ctx->stream>>>(p, (const T*)m, (const T*)Hd, ctx->ctl);
+    dep(k_torque<T>, blocks_for(p.N), kThreads, 0, ctx->stream)(p, (const T*)m, (const T*)Hd, ctx->ctl);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
@@ -896,7 +908,7 @@ int rk_stage(mm_ctx* ctx, int method, int s, const void* m_in, const void* m0, v
 
 int rk_controller(mm_ctx* ctx, int method) {
     KernelTimer kt(ctx, MM_K_CONTROL);
-    k_controller<<<1, 32, 0, ctx->stream>>>(ctx->ctl, method);
+    dep(k_controller, 1, 32, 0, ctx->stream)(ctx->ctl, method);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
@@ -905,9 +917,9 @@ int rk_commit(mm_ctx* ctx, void* m0) {
     KernelTimer kt(ctx, MM_K_CONTROL);
     long n3 = 3 * ctx->N;
     if (ctx->prec == MM_F64)
-        k_commit<double><<<blocks_for(n3), kThreads, 0, ctx->stream>>>(n3, (const double*)ctx->mnext, (double*)m0, ctx->ctl);
+        dep(k_commit<double>, blocks_for(n3), kThreads, 0, ctx->stream)(n3, (const double*)ctx->mnext, (double*)m0, ctx->ctl);
     else
-        k_commit<float><<<blocks_for(n3), kThreads, 0, ctx->stream>>>(n3, (const float*)ctx->mnext, (float*)m0, ctx->ctl);
+        dep(k_commit<float>, blocks_for(n3), kThreads, 0, ctx->stream)(n3, (const float*)ctx->mnext, (float*)m0, ctx->ctl);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
@@ -917,11 +929,11 @@ int bb_iteration_t(mm_ctx* ctx, void* m, void* g, const void* g_prev, void* m_pr
                    long max_iter) {
     KernelTimer kt(ctx, MM_K_REDUCE);
     const Params<T> p = make_params<T>(ctx);
-    k_bb_grad<T><<<blocks_for(p.N), kThreads, 0, ctx->stream>>>(p, (const T*)m, (const T*)ctx->Hd, (T*)g,
+    dep(k_bb_grad<T>, blocks_for(p.N), kThreads, 0, ctx->stream)(p, (const T*)m, (const T*)ctx->Hd, (T*)g,
                                                                 (const T*)g_prev, (const T*)m_prev, have_prev ? 1 : 0,
                                                                 ctx->ctl);
-    k_bb_tau<<<1, 32, 0, ctx->stream>>>(ctx->ctl, tol, max_iter);
-    k_bb_update<T><<<blocks_for(p.N), kThreads, 0, ctx->stream>>>(p, (T*)m, (const T*)g, (T*)m_prev, ctx->ctl);
+    dep(k_bb_tau, 1, 32, 0, ctx->stream)(ctx->ctl, tol, max_iter);
+    dep(k_bb_update<T>, blocks_for(p.N), kThreads, 0, ctx->stream)(p, (T*)m, (const T*)g, (T*)m_prev, ctx->ctl);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
@@ -936,9 +948,9 @@ int check_finite_launch(mm_ctx* ctx, const void* m) {
     KernelTimer kt(ctx, MM_K_REDUCE);
     long n3 = 3 * ctx->N;
     if (ctx->prec == MM_F64)
-        k_finite<double><<<blocks_for(n3), kThreads, 0, ctx->stream>>>(n3, (const double*)m, ctx->ctl);
+        dep(k_finite<double>, blocks_for(n3), kThreads, 0, ctx->stream)(n3, (const double*)m, ctx->ctl);
     else
-        k_finite<float><<<blocks_for(n3), kThreads, 0, ctx->stream>>>(n3, (const float*)m, ctx->ctl);
+        dep(k_finite<float>, blocks_for(n3), kThreads, 0, ctx->stream)(n3, (const float*)m, ctx->ctl);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }

@@ -57,6 +57,7 @@ template <typename T, typename S, int L1, int L2>
 __global__ void __launch_bounds__(px_threads(px_rows<T>(L1 * L2), L1, L2))
     k_px_fwd(const S* __restrict__ in, int nx, const S* __restrict__ Ms, T ms, long ms_rows, PC<T>* __restrict__ out,
              long R, long rows, const PC<T>* __restrict__ twL, const PC<T>* __restrict__ twP) {
+    dep_wait();
     using C = PC<T>;
     constexpr int L = L1 * L2, B = px_rows<T>(L), LP = plane_pitch(L1, L2) + (sizeof(T) == 4 ? 4 : 2);
     __shared__ C Sm[B * LP];
@@ -68,14 +69,22 @@ __global__ void __launch_bounds__(px_threads(px_rows<T>(L1 * L2), L1, L2))
         const bool act = r < rows;
         const S* row = in + (act ? r : 0) * nx;
         const S* mrow = Ms ? Ms + ((act ? r : 0) % ms_rows) * nx : nullptr;
+        // pairs in one access where every row starts on a pair boundary
+        const bool even = nx % 2 == 0 && reinterpret_cast<uintptr_t>(in) % (2 * sizeof(S)) == 0;
         C v[L1];
 #pragma unroll
         for (int n1 = 0; n1 < L1 / 2; ++n1) {
             const int x = 2 * (t + L2 * n1);
             S a = 0, c = 0;
             if (act && x < nx) {
-                a = row[x];
-                if (x + 1 < nx) c = row[x + 1];
+                if (even) {
+                    const PC<S> q = *reinterpret_cast<const PC<S>*>(row + x);
+                    a = q.x;
+                    c = q.y;
+                } else {
+                    a = row[x];
+                    if (x + 1 < nx) c = row[x + 1];
+                }
             }
             T ta = pl_ld<T>(a), tc = pl_ld<T>(c);
             if (mrow) {
@@ -131,6 +140,7 @@ template <typename T, typename S, int L1, int L2>
 __global__ void __launch_bounds__(px_threads(px_rows<T>(L1 * L2), L1, L2))
     k_px_inv(const PC<T>* __restrict__ in, long R, S* __restrict__ out, int nx, long rows, T scale,
              const PC<T>* __restrict__ twL, const PC<T>* __restrict__ twP) {
+    dep_wait();
     using C = PC<T>;
     constexpr int L = L1 * L2, B = px_rows<T>(L), LP = plane_pitch(L1, L2) + (sizeof(T) == 4 ? 4 : 2);
     __shared__ C Sm[B * LP];
@@ -178,7 +188,7 @@ __global__ void __launch_bounds__(px_threads(px_rows<T>(L1 * L2), L1, L2))
         const long r = r0 + b;
         if (r < rows) {
             S* row = out + r * nx;
-            const bool even = nx % 2 == 0;
+            const bool even = nx % 2 == 0 && reinterpret_cast<uintptr_t>(out) % (2 * sizeof(S)) == 0;
 #pragma unroll
             for (int k2 = 0; k2 < L2 / 2; ++k2) {
                 const C z = u[dif_pos<L2>(k2)];
@@ -260,6 +270,7 @@ template <typename T, int L1, int L2, bool FUSED>
 __global__ void __launch_bounds__(sizeof(T) == 4 ? 512 : 256)
     k_plane(PC<T>* __restrict__ buf, const T* __restrict__ kern, int nz, int ny, long R, int KQ,
             const PC<T>* __restrict__ tw) {
+    dep_wait();
     using C = PC<T>;
     constexpr int P = L1 * L2, LP = plane_pitch(L1, L2);
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -396,6 +407,7 @@ template <typename T, int L1, int L2, int DIR>
 __global__ void __launch_bounds__((kPyLines * (L1 > L2 ? L1 : L2) + 31) / 32 * 32)
     k_py(const PC<T>* __restrict__ in, PC<T>* __restrict__ out, int lines, long nlines, int ny, long in_plane,
          long out_plane, const PC<T>* __restrict__ tw) {
+    dep_wait();
     using C = PC<T>;
     constexpr int P = L1 * L2, LP = plane_pitch(L1, L2), B = kPyLines;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -477,6 +489,7 @@ template <typename T, int L1, int L2, int B> constexpr size_t zline_smem() {
 template <typename T, int L1, int L2, bool COLY, int B, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
     k_zline(PC<T>* __restrict__ buf, const T* __restrict__ kern, ZLine g, const PC<T>* __restrict__ tw) {
+    dep_wait();
     using C = PC<T>;
     constexpr int PZ = L1 * L2, PZ2 = PZ / 2 + 1, LQ = L2 + 1, CP = L1 * LQ * B;   // component pitch
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -18,6 +18,7 @@ __global__ void __launch_bounds__(kThreads)
     k_ffx_fwd(const double* __restrict__ in, int nx, const double* __restrict__ Ms, ff ms, long ms_rows,
               ffc* __restrict__ out, long R, long rows, int lgL, int lgB, const ffc* __restrict__ twL,
               const ffc* __restrict__ twP) {
+    dep_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     ffc* s = reinterpret_cast<ffc*>(smem_raw);
     const int L = 1 << lgL, B = 1 << lgB;
@@ -61,6 +62,7 @@ __global__ void __launch_bounds__(kThreads)
 __global__ void __launch_bounds__(kThreads)
     k_ffx_inv(const ffc* __restrict__ in, long R, double* __restrict__ out, int nx, long rows, ff scale, int lgL,
               int lgB, const ffc* __restrict__ twL, const ffc* __restrict__ twP) {
+    dep_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     ffc* s = reinterpret_cast<ffc*>(smem_raw);
     const int L = 1 << lgL, B = 1 << lgB;
@@ -97,6 +99,7 @@ template <int NZ>
 __global__ void __launch_bounds__(kPlaneThreads)
     k_ff_plane(ffc* __restrict__ buf, const ff* __restrict__ kern, int ny, long R, int KQ, int lgP,
                const ffc* __restrict__ tw) {
+    dep_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     ffc* s = reinterpret_cast<ffc*>(smem_raw);
     const int P = 1 << lgP;
@@ -159,7 +162,7 @@ int launch_ff_plane(mm_ctx* ctx, ffc* buf, const ffc* tw) {
         MM_CUDA_CHECK(ctx, cudaFuncSetAttribute((const void*)k_ff_plane<NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 (int)smem));
     const int nt = (3 * NZ * p.P / 8 + 31) / 32 * 32;     // the Stockham stages need 3 nz P / 8 threads
-    k_ff_plane<NZ><<<(unsigned)p.K, nt, smem, ctx->stream>>>(buf, (const ff*)p.kern_ff, ctx->ny, p.R, p.KQ, ilog2(p.P),
+    dep(k_ff_plane<NZ>, (unsigned)p.K, nt, smem, ctx->stream)(buf, (const ff*)p.kern_ff, ctx->ny, p.R, p.KQ, ilog2(p.P),
                                                              tw + p.off_y);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
@@ -186,7 +189,7 @@ int plane_apply_ff(mm_ctx* ctx, const double* m, const double* Ms, double ms, do
     int rc;
     {
         KernelTimer kt(ctx, MM_K_XFWD);
-        k_ffx_fwd<<<nb, nt, smem, ctx->stream>>>(m, ctx->nx, Ms, ff(ms), (long)ctx->nz * ctx->ny, buf, p.R, rows, lgL,
+        dep(k_ffx_fwd, nb, nt, smem, ctx->stream)(m, ctx->nx, Ms, ff(ms), (long)ctx->nz * ctx->ny, buf, p.R, rows, lgL,
                                                  lgB, tw, tw + p.off_p);
         MM_LAUNCH_CHECK(ctx);
     }
@@ -197,7 +200,7 @@ int plane_apply_ff(mm_ctx* ctx, const double* m, const double* Ms, double ms, do
     }
     if (rc) return rc;
     KernelTimer kt(ctx, MM_K_XINV);
-    k_ffx_inv<<<nb, nt, smem, ctx->stream>>>(buf, p.R, H, ctx->nx, rows, ff(1.0 / ((double)p.L * p.P * ctx->Pz)), lgL,
+    dep(k_ffx_inv, nb, nt, smem, ctx->stream)(buf, p.R, H, ctx->nx, rows, ff(1.0 / ((double)p.L * p.P * ctx->Pz)), lgL,
                                              lgB, tw, tw + p.off_p);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;

@@ -60,7 +60,7 @@ int launch_px_fwd(mm_ctx* ctx, const S* in, const S* Ms, T ms, long ms_rows, PC<
             constexpr int L1 = decltype(A)::value, L2 = decltype(B)::value, L = L1 * L2;
             if constexpr (L <= 512) {
                 constexpr int BR = px_rows<T>(L);
-                k_px_fwd<T, S, L1, L2><<<(unsigned)((rows + BR - 1) / BR), px_threads(BR, L1, L2), 0, ctx->stream>>>(
+                dep(k_px_fwd<T, S, L1, L2>, (unsigned)((rows + BR - 1) / BR), px_threads(BR, L1, L2), 0, ctx->stream)(
                     in, ctx->nx, Ms, ms, ms_rows, out, p.R, rows, tw + p.off_x4, tw + p.off_p);
             }
         }))
@@ -79,7 +79,7 @@ int launch_px_inv(mm_ctx* ctx, const PC<T>* in, S* out, long rows, T scale, cons
             constexpr int L1 = decltype(A)::value, L2 = decltype(B)::value, L = L1 * L2;
             if constexpr (L <= 512) {
                 constexpr int BR = px_rows<T>(L);
-                k_px_inv<T, S, L1, L2><<<(unsigned)((rows + BR - 1) / BR), px_threads(BR, L1, L2), 0, ctx->stream>>>(
+                dep(k_px_inv<T, S, L1, L2>, (unsigned)((rows + BR - 1) / BR), px_threads(BR, L1, L2), 0, ctx->stream)(
                     in, p.R, out, ctx->nx, rows, scale, tw + p.off_x4, tw + p.off_p);
             }
         }))
@@ -108,7 +108,7 @@ int launch_plane(mm_ctx* ctx, PC<T>* buf, const T* kern, const PC<T>* tw) {
             if (nt > cap) nt = (tasks + (tasks + cap - 1) / cap - 1) / ((tasks + cap - 1) / cap);
             nt = (nt + 31) / 32 * 32;
             if (nt > cap) nt = cap;
-            fn<<<(unsigned)p.K, nt, smem, ctx->stream>>>(buf, kern, ctx->nz, ctx->ny, p.R, p.KQ, tw + p.off_y4);
+            dep(fn, (unsigned)p.K, nt, smem, ctx->stream)(buf, kern, ctx->nz, ctx->ny, p.R, p.KQ, tw + p.off_y4);
         }))
         rc = fail(ctx, MM_ERR_INVALID_ARG, "y length %d", p.P);
     if (rc) return rc;
@@ -128,8 +128,7 @@ int launch_py(mm_ctx* ctx, const PC<T>* in, PC<T>* out, const PC<T>* tw) {
             auto fn = k_py<T, L1, L2, DIR>;
             const size_t smem = (size_t)kPyLines * plane_pitch(L1, L2) * sizeof(PC<T>);
             if ((rc = plane_smem(ctx, (const void*)fn, smem))) return;
-            fn<<<(unsigned)((nlines + kPyLines - 1) / kPyLines), (kPyLines * (L1 > L2 ? L1 : L2) + 31) / 32 * 32, smem,
-                 ctx->stream>>>(in, out, lines, nlines, ctx->ny, DIR < 0 ? p.R : wide, DIR < 0 ? wide : p.R,
+            dep(fn, (unsigned)((nlines + kPyLines - 1) / kPyLines), (kPyLines * (L1 > L2 ? L1 : L2) + 31) / 32 * 32, smem, ctx->stream)(in, out, lines, nlines, ctx->ny, DIR < 0 ? p.R : wide, DIR < 0 ? wide : p.R,
                                                       tw + p.off_y4);
         }))
         rc = fail(ctx, MM_ERR_INVALID_ARG, "y length %d", p.P);
@@ -172,7 +171,7 @@ int launch_zline_t(mm_ctx* ctx, PC<T>* buf, const T* kern, const ZLine& g, int n
     int rc = plane_smem(ctx, (const void*)fn, smem);
     if (rc) return rc;
     dim3 grid((unsigned)((g.ncol + B - 1) / B), (unsigned)nrows);
-    fn<<<grid, NT, smem, ctx->stream>>>(buf, kern, g, tw);
+    dep(fn, grid, NT, smem, ctx->stream)(buf, kern, g, tw);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
