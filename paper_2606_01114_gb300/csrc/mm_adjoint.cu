@@ -94,8 +94,9 @@ __global__ void k_vjp_norm(Params<T> p, const T* __restrict__ m0, const T* __res
     V3<T> lu = {0, 0, 0};
     if (Msi != (T)0) {
         V3<T> X3 = load3(x3, i, p.N);
-        V3<T> h = exchange_at(p, x3, i, x, y, z, X3, Msi);
-        V3<T> l = local_at(p, X3, Msi);
+        const T inv = inv_ms_at(p, Msi);
+        V3<T> h = exchange_at(p, x3, i, x, y, z, X3, inv);
+        V3<T> l = local_at(p, X3, inv);
         V3<T> d = load3(hd3, i, p.N);
         V3<T> k3 = llg_rhs(p, X3, V3<T>{h.x + l.x + d.x, h.y + l.y + d.y, h.z + l.z + d.z});
         V3<T> a = load3(k0, i, p.N), b = load3(k1, i, p.N), c = load3(k2, i, p.N), m = load3(m0, i, p.N);
@@ -130,8 +131,9 @@ __global__ void k_vjp_rhs_a(Params<T> p, const T* __restrict__ X, const T* __res
     V3<T> gH = {0, 0, 0}, gm = {0, 0, 0};
     if (Msi != (T)0) {
         V3<T> m = load3(X, i, p.N);
-        V3<T> h = exchange_at(p, X, i, x, y, z, m, Msi);
-        V3<T> l = local_at(p, m, Msi);
+        const T inv = inv_ms_at(p, Msi);
+        V3<T> h = exchange_at(p, X, i, x, y, z, m, inv);
+        V3<T> l = local_at(p, m, inv);
         V3<T> d = load3(hd, i, p.N);
         V3<T> H = {h.x + l.x + d.x, h.y + l.y + d.y, h.z + l.z + d.z};
         V3<T> W = load3(w, i, p.N);
@@ -164,7 +166,8 @@ __global__ void k_vjp_rhs_b(Params<T> p, const T* __restrict__ X, const T* __res
     V3<T> g = load3(G, i, p.N);
     V3<T> dd = load3(D, i, p.N);
     V3<T> e = stencil_g_over_ms(p, G, i, x, y, z, Msi);
-    const T ka = p.anis / Msi;
+    const T inv = inv_ms_at(p, Msi);
+    const T ka = p.anis * inv;
     const T gu = g.x * p.ux + g.y * p.uy + g.z * p.uz;
     V3<T> pr = load3(P, i, p.N);
     V3<T> lx = {pr.x + Msi * dd.x + e.x + ka * gu * p.ux, pr.y + Msi * dd.y + e.y + ka * gu * p.uy,
@@ -176,10 +179,10 @@ __global__ void k_vjp_rhs_b(Params<T> p, const T* __restrict__ X, const T* __res
         store3(lk_prev, i, p.N, axpy(coef, lx, K));
     }
     // Ms pull-back: demag through M = Ms m, exchange and anisotropy through 1/Ms
-    V3<T> hex = exchange_at(p, X, i, x, y, z, m, Msi);
+    V3<T> hex = exchange_at(p, X, i, x, y, z, m, inv);
     const T mu = m.x * p.ux + m.y * p.uy + m.z * p.uz;
     V3<T> han = {ka * mu * p.ux, ka * mu * p.uy, ka * mu * p.uz};
-    gMs[i] += dot(m, dd) - (dot(g, hex) + dot(g, han)) / Msi;
+    gMs[i] += dot(m, dd) - (dot(g, hex) + dot(g, han)) * inv;
 }
 
 // transposes of the single field terms (autograd of demag_field / exchange_field)
@@ -211,7 +214,8 @@ __global__ void k_exchange_vjp(Params<T> p, const T* __restrict__ m, const T* __
     store3(gm, i, p.N, stencil_g_over_ms(p, g, i, x, y, z, Msi));
     if (gMs) {
         V3<T> mi = load3(m, i, p.N);
-        gMs[i] += -dot(load3(g, i, p.N), exchange_at(p, m, i, x, y, z, mi, Msi)) / Msi;
+        const T inv = inv_ms_at(p, Msi);
+        gMs[i] += -dot(load3(g, i, p.N), exchange_at(p, m, i, x, y, z, mi, inv)) * inv;
     }
 }
 

@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(256) k_field4(Params<float> p, float wx, float
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const V3<float> mi = {el(c.x, j), el(c.y, j), el(c.z, j)};
-            const V3<float> l = local_at(p, mi, p.Ms);
+            const V3<float> l = local_at(p, mi, p.inv_Ms);
             el(h.x, j) += l.x + el(d.x, j);
             el(h.y, j) += l.y + el(d.y, j);
             el(h.z, j) += l.z + el(d.z, j);

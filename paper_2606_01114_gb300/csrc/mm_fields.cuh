@@ -14,6 +14,7 @@ template <typename T> struct Params {
     const T* Ms_cell;   // nullable
     const T* A_cell;    // nullable
     T Ms, A;
+    T inv_Ms;           // 1 / Ms (0 when Ms is 0)
     T cx, cy, cz;       // 2 / (mu0 d^2) per axis
     T anis;             // 2 Ku / mu0
     T ux, uy, uz;
@@ -39,6 +40,7 @@ inline Params<T> make_params(const mm_ctx* ctx) {
     p.A_cell = ctx->has_A_cell ? (const T*)ctx->A_cell : nullptr;
     p.Ms = (T)ctx->Ms;
     p.A = (T)ctx->A;
+    p.inv_Ms = p.Ms != (T)0 ? (T)1 / p.Ms : (T)0;
     p.cx = (T)(2.0 / (kMu0 * ctx->dx * ctx->dx));
     p.cy = (T)(2.0 / (kMu0 * ctx->dy * ctx->dy));
     p.cz = (T)(2.0 / (kMu0 * ctx->dz * ctx->dz));
@@ -79,10 +81,18 @@ __device__ __forceinline__ void store3(T* __restrict__ a, long i, long N, V3<T> 
     a[i + 2 * N] = v.z;
 }
 
-// exchange field at cell i (x, y, z) of state m; Msi > 0
+// 1 / Ms of a magnetic cell.  Every term of the field divides by Ms: the
+// reciprocal is taken once per cell, and on the host for uniform Ms (an FP64
+// division is about 25 instructions of a pipe that issues one warp
+// instruction per 64 cycles; the uniform FP64 cell took three of them).
+template <typename T> __device__ __forceinline__ T inv_ms_at(const Params<T>& p, T Msi) {
+    return p.Ms_cell ? (T)1 / Msi : p.inv_Ms;
+}
+
+// exchange field at cell i (x, y, z) of state m; inv = 1 / Ms_i
 template <typename T>
 __device__ __forceinline__ V3<T> exchange_at(const Params<T>& p, const T* __restrict__ m, long i, int x, int y,
-                                             int z, V3<T> mi, T Msi) {
+                                             int z, V3<T> mi, T inv) {
     const T Ai = p.A_cell ? p.A_cell[i] : p.A;
     T ax = 0, ay = 0, az = 0;
     auto nb = [&](long j, T c) {
@@ -108,26 +118,26 @@ __device__ __forceinline__ V3<T> exchange_at(const Params<T>& p, const T* __rest
     if (y < p.ny - 1) nb(i + sy, p.cy);
     if (z > 0) nb(i - sz, p.cz);
     if (z < p.nz - 1) nb(i + sz, p.cz);
-    T inv = (T)1 / Msi;
     return {ax * inv, ay * inv, az * inv};
 }
 
 // anisotropy + Zeeman at a magnetic cell
 template <typename T>
-__device__ __forceinline__ V3<T> local_at(const Params<T>& p, V3<T> mi, T Msi) {
+__device__ __forceinline__ V3<T> local_at(const Params<T>& p, V3<T> mi, T inv) {
+    if (p.anis == (T)0) return {p.hx, p.hy, p.hz};
     T mu = mi.x * p.ux + mi.y * p.uy + mi.z * p.uz;
-    T k = p.anis / Msi * mu;
+    T k = p.anis * inv * mu;
     return {k * p.ux + p.hx, k * p.uy + p.hy, k * p.uz + p.hz};
 }
 
-// DMI field (Eq. 3) at cell i of unit m; Msi > 0:
+// DMI field (Eq. 3) at cell i of unit m; inv = 1 / Ms_i:
 //   H = 2 D / (mu0 Ms) sum_k e_k x (m[+k] - m[-k]) / (2 d_k),
 // e_k = (e_y, -e_x, 0) interfacial or (e_x, e_y, e_z) bulk; a neighbour
 // outside the magnet (mesh edge or Ms = 0) contributes nothing (the field
 // of the bond energy (D V / d_k) sum_bonds e_k . (m_i x m_(i+k))).
 template <typename T>
 __device__ __forceinline__ V3<T> dmi_at(const Params<T>& p, const T* __restrict__ m, long i, int x, int y, int z,
-                                        T Msi) {
+                                        T inv) {
     T hx = 0, hy = 0, hz = 0;
     // sum over the present neighbours of sign * (m_nb) per axis: v_axis
     auto acc = [&](long j, T sgn, T& vx, T& vy, T& vz) {
@@ -161,7 +171,6 @@ __device__ __forceinline__ V3<T> dmi_at(const Params<T>& p, const T* __restrict_
         hx += -p.dz_c * cy;
         hy += p.dz_c * cx;
     }
-    const T inv = (T)1 / Msi;
     return {hx * inv, hy * inv, hz * inv};
 }
 
@@ -171,10 +180,10 @@ __device__ __forceinline__ V3<T> dmi_at(const Params<T>& p, const T* __restrict_
 // (L^2 - 1) m.p), solved for dm/dt:
 //   gamma beta / (1 + alpha^2) [(eps + alpha eps') m x (p x m) - (eps' - alpha eps) m x p]
 template <typename T>
-__device__ __forceinline__ V3<T> stt_at(const Params<T>& p, V3<T> m, T Msi) {
+__device__ __forceinline__ V3<T> stt_at(const Params<T>& p, V3<T> m, T inv) {
     const T mp = m.x * p.px + m.y * p.py + m.z * p.pz;
     const T eps = p.stt_P * p.stt_L2 / ((p.stt_L2 + (T)1) + (p.stt_L2 - (T)1) * mp);
-    const T c = p.stt_c / Msi;
+    const T c = p.stt_c * inv;
     const T a = c * (eps + p.alpha * p.stt_eps2), b = c * (p.stt_eps2 - p.alpha * eps);
     // m x (p x m) = (m.m) p - (m.p) m (stage states are not unit vectors);  m x p
     const T mm = m.x * m.x + m.y * m.y + m.z * m.z;
@@ -190,11 +199,13 @@ __device__ __forceinline__ V3<T> llg_rhs(const Params<T>& p, V3<T> m, V3<T> H) {
     return {p.pref * (a.x + p.alpha * b.x), p.pref * (a.y + p.alpha * b.y), p.pref * (a.z + p.alpha * b.z)};
 }
 
+// i < 2^31 (meshes hold at most 512^3 cells): 32-bit division, a fraction of
+// the 64-bit sequence
 __device__ __forceinline__ void decompose(long i, int nx, int ny, int& x, int& y, int& z) {
-    x = (int)(i % nx);
-    long r = i / nx;
-    y = (int)(r % ny);
-    z = (int)(r / ny);
+    const unsigned u = (unsigned)i, r = u / (unsigned)nx, q = r / (unsigned)ny;
+    x = (int)(u - r * nx);
+    y = (int)(r - q * ny);
+    z = (int)q;
 }
 
 }  // namespace mm

@@ -15,6 +15,7 @@
 // reduction + one atomic max per block) and the renormalisation.  The RKF45
 // step control (k_controller) runs on the device, so a step needs no host
 // synchronisation.  Energies and the torque maximum (K9) accumulate in FP64.
+#include <algorithm>
 #include <cmath>
 
 #include "mm_ff.cuh"
@@ -65,18 +66,25 @@ __host__ __device__ constexpr double rk_e(int method, int j) {
 }
 __host__ __device__ constexpr int rk_stages(int method) { return method == MM_RK4 ? 4 : 6; }
 
-// block-wide max of a non-negative double, then one atomicMax of its bits
+// Block-wide max of a non-negative double, then one atomicMax of its bits.
+// Non-negative doubles order like their bit patterns, so the maxima are
+// integer reductions and none of it runs on the FP64 pipe.
+__device__ __forceinline__ unsigned long long warp_max_bits(unsigned long long v) {
+    const unsigned hi = (unsigned)(v >> 32);
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)v : 0u);
+    return ((unsigned long long)mh << 32) | ml;
+}
 __device__ __forceinline__ void block_max_atomic(double v, unsigned long long* target) {
-    __shared__ double red[32];
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) red[w] = v;
+    __shared__ unsigned long long red[32];
+    unsigned long long u = warp_max_bits((unsigned long long)__double_as_longlong(v));
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (lane == 0) red[w] = u;
     __syncthreads();
     if (w == 0) {
-        int nw = (blockDim.x + 31) >> 5;
-        v = lane < nw ? red[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-        if (lane == 0 && v > 0.0) atomicMax(target, (unsigned long long)__double_as_longlong(v));
+        const int nw = (blockDim.x + 31) >> 5;
+        u = warp_max_bits(lane < nw ? red[lane] : 0ull);
+        if (lane == 0 && u != 0ull) atomicMax(target, u);
     }
 }
 
@@ -134,13 +142,14 @@ __global__ void k_field(Params<T> p, const T* __restrict__ m, const T* __restric
     V3<T> h = {0, 0, 0};
     if (Msi != (T)0) {
         V3<T> mi = load3(m, i, p.N);
-        h = exchange_at(p, m, i, x, y, z, mi, Msi);
+        const T inv = inv_ms_at(p, Msi);
+        h = exchange_at(p, m, i, x, y, z, mi, inv);
         if (MODE == 1) {
-            V3<T> l = local_at(p, mi, Msi);
+            V3<T> l = local_at(p, mi, inv);
             V3<T> d = load3(Hd, i, p.N);
             h = {h.x + l.x + d.x, h.y + l.y + d.y, h.z + l.z + d.z};
             if (p.dmi) {
-                const V3<T> q = dmi_at(p, m, i, x, y, z, Msi);
+                const V3<T> q = dmi_at(p, m, i, x, y, z, inv);
                 h = {h.x + q.x, h.y + q.y, h.z + q.z};
             }
         }
@@ -168,17 +177,18 @@ __global__ void k_stage(Params<T> p, const T* __restrict__ m_in, const T* __rest
         V3<T> ks = {0, 0, 0};
         V3<T> mi = load3(m_in, i, p.N);
         if (Msi != (T)0) {
-            V3<T> h = exchange_at(p, m_in, i, x, y, z, mi, Msi);
-            V3<T> l = local_at(p, mi, Msi);
+            const T inv = inv_ms_at(p, Msi);
+            V3<T> h = exchange_at(p, m_in, i, x, y, z, mi, inv);
+            V3<T> l = local_at(p, mi, inv);
             V3<T> d = load3(Hd, i, p.N);
             h = {h.x + l.x + d.x, h.y + l.y + d.y, h.z + l.z + d.z};
             if (p.dmi) {
-                const V3<T> q = dmi_at(p, m_in, i, x, y, z, Msi);
+                const V3<T> q = dmi_at(p, m_in, i, x, y, z, inv);
                 h = {h.x + q.x, h.y + q.y, h.z + q.z};
             }
             ks = llg_rhs(p, mi, h);
             if (p.stt) {
-                const V3<T> q = stt_at(p, mi, Msi);
+                const V3<T> q = stt_at(p, mi, inv);
                 ks = {ks.x + q.x, ks.y + q.y, ks.z + q.z};
             }
         }
@@ -311,7 +321,7 @@ __global__ void __launch_bounds__(256) k_stage4(Params<float> p, float wx, float
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const V3<float> mi = {at(c.x, j), at(c.y, j), at(c.z, j)};
-            const V3<float> l = local_at(p, mi, p.Ms);
+            const V3<float> l = local_at(p, mi, p.inv_Ms);
             const V3<float> H = {at(h.x, j) + l.x + at(d.x, j), at(h.y, j) + l.y + at(d.y, j),
                                  at(h.z, j) + l.z + at(d.z, j)};
             const V3<float> r = llg_rhs(p, mi, H);
@@ -532,17 +542,16 @@ __global__ void __launch_bounds__(256)
     }
     if constexpr (LAST && METHOD == MM_RKF45) {
         // block max of the squared norms; err = dt sqrt(max) for the controller
-        __shared__ double red[32];
-        for (int o = 16; o > 0; o >>= 1) w2 = fmax(w2, __shfl_xor_sync(0xffffffffu, w2, o));
+        __shared__ unsigned long long red[32];
+        unsigned long long u = warp_max_bits((unsigned long long)__double_as_longlong(w2));
         const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-        if (lane == 0) red[w] = w2;
+        if (lane == 0) red[w] = u;
         __syncthreads();
         if (w == 0) {
             const int nw = (blockDim.x + 31) >> 5;
-            w2 = lane < nw ? red[lane] : 0.0;
-            for (int o = 16; o > 0; o >>= 1) w2 = fmax(w2, __shfl_xor_sync(0xffffffffu, w2, o));
-            if (lane == 0 && w2 > 0.0) {
-                const double err = ctl->dt * sqrt(w2);
+            u = warp_max_bits(lane < nw ? red[lane] : 0ull);
+            if (lane == 0 && u != 0ull) {
+                const double err = ctl->dt * sqrt(__longlong_as_double((long long)u));
                 atomicMax(&ctl->err_bits, (unsigned long long)__double_as_longlong(err));
             }
         }
@@ -595,74 +604,157 @@ __global__ void k_controller(Control* ctl, int method) {
     ctl->dt = dtn;
 }
 
-template <typename T>
-__global__ void k_commit(long n3, const T* __restrict__ src, T* __restrict__ dst, const Control* ctl) {
+// V: float4 or double2 where both arrays are 16-byte aligned (the scalar form
+// copied 512x512x16 at 2.6 TB/s), else T
+template <typename V>
+__global__ void __launch_bounds__(256) k_commit(long n, const V* __restrict__ src, V* __restrict__ dst, const Control* ctl) {
     dep_wait();
     if (!ctl->accepted) return;
-    long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n3) dst[i] = src[i];
+    const long i0 = (long)blockIdx.x * (4 * blockDim.x) + threadIdx.x;
+    V v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (i0 + u * blockDim.x < n) v[u] = src[i0 + u * blockDim.x];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (i0 + u * blockDim.x < n) dst[i0 + u * blockDim.x] = v[u];
 }
 
 // ------------------------------------------------------------- K9
+constexpr int kReduceThreads = 128;
+
+// Energies: each thread sums its cells in double (grid stride), so the block
+// reduction of the five sums, 25 FP64 adds a thread, is paid once and not per
+// cell; terms whose constant is zero are skipped.
 template <typename T>
-__global__ void k_energy(Params<T> p, const T* __restrict__ m, const T* __restrict__ Hd, double V, double mu0,
-                         double Ku, Control* ctl) {
+__global__ void __launch_bounds__(kReduceThreads)
+    k_energy(Params<T> p, const T* __restrict__ m, const T* __restrict__ Hd, double V, double mu0, double Ku,
+             Control* ctl) {
     dep_wait();
-    long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     double ed = 0, ex = 0, ea = 0, ez = 0, em = 0;
-    if (i < p.N) {
+    const double c = -mu0 * V;
+    const bool zeeman = p.hx != (T)0 || p.hy != (T)0 || p.hz != (T)0;
+    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < p.N; i += (long)gridDim.x * blockDim.x) {
         int x, y, z;
         decompose(i, p.nx, p.ny, x, y, z);
-        T Msi = p.Ms_cell ? p.Ms_cell[i] : p.Ms;
-        if (Msi != (T)0) {
-            V3<T> mi = load3(m, i, p.N);
-            V3<T> h = exchange_at(p, m, i, x, y, z, mi, Msi);
-            V3<T> d = load3(Hd, i, p.N);
-            double ms = (double)Msi;
-            ed = -0.5 * mu0 * V * ms * ((double)mi.x * d.x + (double)mi.y * d.y + (double)mi.z * d.z);
-            ex = -0.5 * mu0 * V * ms * ((double)mi.x * h.x + (double)mi.y * h.y + (double)mi.z * h.z);
-            double mu = (double)mi.x * p.ux + (double)mi.y * p.uy + (double)mi.z * p.uz;
-            ea = -Ku * V * mu * mu;
-            ez = -mu0 * V * ms * ((double)mi.x * p.hx + (double)mi.y * p.hy + (double)mi.z * p.hz);
-            if (p.dmi) {
-                const V3<T> q = dmi_at(p, m, i, x, y, z, Msi);
-                em = -0.5 * mu0 * V * ms * ((double)mi.x * q.x + (double)mi.y * q.y + (double)mi.z * q.z);
-            }
+        const T Msi = p.Ms_cell ? p.Ms_cell[i] : p.Ms;
+        if (Msi == (T)0) continue;
+        const T inv = inv_ms_at(p, Msi);
+        const V3<T> mi = load3(m, i, p.N);
+        const V3<T> h = exchange_at(p, m, i, x, y, z, mi, inv);
+        const V3<T> d = load3(Hd, i, p.N);
+        const double mx = mi.x, my = mi.y, mz = mi.z, w = c * (double)Msi, hw = 0.5 * w;
+        ed += hw * (mx * d.x + my * d.y + mz * d.z);
+        ex += hw * (mx * h.x + my * h.y + mz * h.z);
+        if (Ku != 0.0) {
+            const double mu = mx * p.ux + my * p.uy + mz * p.uz;
+            ea += -Ku * V * mu * mu;
+        }
+        if (zeeman) ez += w * (mx * p.hx + my * p.hy + mz * p.hz);
+        if (p.dmi) {
+            const V3<T> q = dmi_at(p, m, i, x, y, z, inv);
+            em += hw * (mx * q.x + my * q.y + mz * q.z);
         }
     }
     block_sum_atomic(ed, &ctl->energy[0]);
     __syncthreads();
     block_sum_atomic(ex, &ctl->energy[1]);
-    __syncthreads();
-    block_sum_atomic(ea, &ctl->energy[2]);
-    __syncthreads();
-    block_sum_atomic(ez, &ctl->energy[3]);
-    __syncthreads();
-    block_sum_atomic(em, &ctl->energy[4]);
+    if (Ku != 0.0) {
+        __syncthreads();
+        block_sum_atomic(ea, &ctl->energy[2]);
+    }
+    if (zeeman) {
+        __syncthreads();
+        block_sum_atomic(ez, &ctl->energy[3]);
+    }
+    if (p.dmi) {
+        __syncthreads();
+        block_sum_atomic(em, &ctl->energy[4]);
+    }
 }
 
+// |m x H_eff| / Ms of one cell in double (1e300 where it is not finite), from
+// the fields in the path's type
+template <typename T>
+__device__ double torque_of(const V3<T>& mi, const V3<T>& h, const V3<T>& l, const V3<T>& d, const V3<T>& q, T Msi) {
+    const double Hx = (double)h.x + l.x + d.x + q.x, Hy = (double)h.y + l.y + d.y + q.y,
+                 Hz = (double)h.z + l.z + d.z + q.z;
+    const double cx = mi.y * Hz - mi.z * Hy, cy = mi.z * Hx - mi.x * Hz, cz = mi.x * Hy - mi.y * Hx;
+    const double tq = sqrt(cx * cx + cy * cy + cz * cz) / (double)Msi;
+    return isfinite(tq) ? tq : 1e300;
+}
+
+// The largest torque.  FP32 contexts: the double evaluation per cell (about
+// 80 FP64 instructions) took 290 us on 512x512x16, three times the field
+// terms' own traffic.  Only the largest value is wanted, so each cell is first
+// evaluated in float with a bound on that evaluation's error (componentwise
+// sums and products of at most six roundings: 8 eps |m| |H| over Ms), and only
+// cells whose upper bound reaches the block's largest lower bound are
+// evaluated in double.  The result is the double maximum over all cells.
 template <typename T>
 __global__ void k_torque(Params<T> p, const T* __restrict__ m, const T* __restrict__ Hd, Control* ctl) {
     dep_wait();
-    long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     double tq = 0.0;
-    if (i < p.N) {
+    const T Msi = i < p.N ? (p.Ms_cell ? p.Ms_cell[i] : p.Ms) : (T)0;
+    V3<T> mi = {0, 0, 0}, h = mi, l = mi, d = mi, q = mi;
+    if (Msi != (T)0) {
         int x, y, z;
         decompose(i, p.nx, p.ny, x, y, z);
-        T Msi = p.Ms_cell ? p.Ms_cell[i] : p.Ms;
+        const T inv = inv_ms_at(p, Msi);
+        mi = load3(m, i, p.N);
+        h = exchange_at(p, m, i, x, y, z, mi, inv);
+        l = local_at(p, mi, inv);
+        d = load3(Hd, i, p.N);
+        if (p.dmi) q = dmi_at(p, m, i, x, y, z, inv);
+    }
+    if constexpr (sizeof(T) == 4) {
+        __shared__ float red[32];
+        float lo = -1.f, up = -1.f;      // bounds of this cell's torque; -1 outside the magnet
         if (Msi != (T)0) {
-            V3<T> mi = load3(m, i, p.N);
-            V3<T> h = exchange_at(p, m, i, x, y, z, mi, Msi);
-            V3<T> l = local_at(p, mi, Msi);
-            V3<T> d = load3(Hd, i, p.N);
-            V3<T> q = {0, 0, 0};
-            if (p.dmi) q = dmi_at(p, m, i, x, y, z, Msi);
-            double Hx = (double)h.x + l.x + d.x + q.x, Hy = (double)h.y + l.y + d.y + q.y,
-                   Hz = (double)h.z + l.z + d.z + q.z;
-            double cx = mi.y * Hz - mi.z * Hy, cy = mi.z * Hx - mi.x * Hz, cz = mi.x * Hy - mi.y * Hx;
-            tq = sqrt(cx * cx + cy * cy + cz * cz) / (double)Msi;
-            if (!isfinite(tq)) tq = 1e300;
+            const float Hx = h.x + l.x + d.x + q.x, Hy = h.y + l.y + d.y + q.y, Hz = h.z + l.z + d.z + q.z;
+            const float cx = mi.y * Hz - mi.z * Hy, cy = mi.z * Hx - mi.x * Hz, cz = mi.x * Hy - mi.y * Hx;
+            const float am = fabsf(mi.x) + fabsf(mi.y) + fabsf(mi.z);
+            const float ah = fabsf(h.x) + fabsf(l.x) + fabsf(d.x) + fabsf(q.x) + fabsf(h.y) + fabsf(l.y) +
+                             fabsf(d.y) + fabsf(q.y) + fabsf(h.z) + fabsf(l.z) + fabsf(d.z) + fabsf(q.z);
+            const float t = sqrtf(cx * cx + cy * cy + cz * cz), e = 1e-6f * am * ah;
+            lo = (t - e) / Msi * 0.99999f;
+            up = (t + e) / Msi * 1.00001f;
+            if (!(up <= 3.0e38f)) {          // not finite in float: decided in double
+                lo = -1.f;
+                up = 3.0e38f;
+            }
         }
+        float b = lo;
+        for (int o = 16; o > 0; o >>= 1) b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, o));
+        __shared__ float found;          // what other blocks have found already, rounded down
+        if (threadIdx.x == 0)
+            found = __double2float_rd(__longlong_as_double(
+                (long long)*(volatile unsigned long long*)&ctl->torque_bits));
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = b;
+        __syncthreads();
+        b = fmaxf(b, found);
+        for (unsigned w = 0; w < (blockDim.x + 31) >> 5; ++w) b = fmaxf(b, red[w]);
+        if (Msi != (T)0 && up >= b) tq = torque_of(mi, h, l, d, q, Msi);
+    } else {
+        // the same in double: squares within 1e-12 of the block's largest are
+        // candidates, the others need neither square root nor division
+        __shared__ unsigned long long red[32];
+        double s2 = 0.0;
+        if (Msi != (T)0) {
+            const double Hx = h.x + l.x + d.x + q.x, Hy = h.y + l.y + d.y + q.y, Hz = h.z + l.z + d.z + q.z;
+            const double cx = mi.y * Hz - mi.z * Hy, cy = mi.z * Hx - mi.x * Hz, cz = mi.x * Hy - mi.y * Hx;
+            const double inv = inv_ms_at(p, Msi);
+            s2 = (cx * cx + cy * cy + cz * cz) * inv * inv;
+        }
+        unsigned long long u = warp_max_bits((unsigned long long)__double_as_longlong(fabs(s2)));
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = u;
+        __syncthreads();
+        for (unsigned w = 0; w < (blockDim.x + 31) >> 5; ++w) u = u > red[w] ? u : red[w];
+        const double top = __longlong_as_double((long long)u);
+        // (a NaN or an overflowed or vanishing square is decided by the full evaluation)
+        if (Msi != (T)0 && (!(s2 < top * (1.0 - 1e-12)) || !(s2 > 1e-280)))
+            tq = torque_of(mi, h, l, d, q, Msi);
     }
     block_max_atomic(tq, &ctl->torque_bits);
 }
@@ -670,12 +762,19 @@ __global__ void k_torque(Params<T> p, const T* __restrict__ m, const T* __restri
 template <typename T>
 __global__ void k_finite(long n3, const T* __restrict__ m, Control* ctl) {
     dep_wait();
-    long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n3 && !isfinite((double)m[i])) atomicCAS(&ctl->status, 0, (int)MM_ERR_NONFINITE);
+    bool bad = false;
+    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += (long)gridDim.x * blockDim.x)
+        bad |= !isfinite(m[i]);
+    if (bad) atomicCAS(&ctl->status, 0, (int)MM_ERR_NONFINITE);
 }
 
+// Cells per block of the one-pass kernels.  Small meshes take 64 threads, so
+// that they reach all 152 SMs (64x64x4 in quads is 16 blocks of 256); FP64
+// kernels always do: a sub-partition issues one FP64 warp instruction per 64
+// cycles, and small blocks spread the warps evenly over the 608 of them.
 constexpr int kThreads = 256;
-inline unsigned blocks_for(long n) { return (unsigned)((n + kThreads - 1) / kThreads); }
+inline int threads_for(long n, size_t elem) { return n < 152L * 2 * kThreads || elem == 8 ? 64 : kThreads; }
+inline unsigned blocks_for(long n, int threads = kThreads) { return (unsigned)((n + threads - 1) / threads); }
 
 // ------------------------------------------------ Barzilai-Borwein minimiser
 // Steepest descent on the unit sphere with Barzilai-Borwein step lengths
@@ -701,12 +800,12 @@ __global__ void k_bb_grad(Params<T> p, const T* __restrict__ m, const T* __restr
         V3<T> gi = {0, 0, 0};
         const V3<T> mi = load3(m, i, p.N);
         if (Msi != (T)0) {
-            const V3<T> hx = exchange_at(p, m, i, x, y, z, mi, Msi);
-            const V3<T> l = local_at(p, mi, Msi);
+            const T inv = inv_ms_at(p, Msi);
+            const V3<T> hx = exchange_at(p, m, i, x, y, z, mi, inv);
+            const V3<T> l = local_at(p, mi, inv);
             const V3<T> d = load3(Hd, i, p.N);
             V3<T> q = {0, 0, 0};
-            if (p.dmi) q = dmi_at(p, m, i, x, y, z, Msi);
-            const T inv = (T)1 / Msi;
+            if (p.dmi) q = dmi_at(p, m, i, x, y, z, inv);
             const V3<T> h = {(hx.x + l.x + d.x + q.x) * inv, (hx.y + l.y + d.y + q.y) * inv,
                              (hx.z + l.z + d.z + q.z) * inv};
             const V3<T> a = {mi.y * h.z - mi.z * h.y, mi.z * h.x - mi.x * h.z, mi.x * h.y - mi.y * h.x};   // m x h
@@ -803,7 +902,8 @@ int launch_stage(mm_ctx* ctx, const Params<T>& p, const void* m_in, const void* 
             c.hz = ff((double)p.hz);
             c.pref = ff((double)p.pref);
             c.alpha = ff((double)p.alpha);
-            dep(k_stage_ff<METHOD, S>, blocks_for(p.N), kThreads, 0, ctx->stream)(
+            const int nt = threads_for(p.N, 4);
+            dep(k_stage_ff<METHOD, S>, blocks_for(p.N, nt), nt, 0, ctx->stream)(
                 c, p.nx, p.ny, p.nz, p.N, (const double*)m_in, (const double*)ctx->Hd, (const double*)m0, kb,
                 (double*)m_out, ctx->ctl);
             MM_LAUNCH_CHECK(ctx);
@@ -815,14 +915,16 @@ int launch_stage(mm_ctx* ctx, const Params<T>& p, const void* m_in, const void* 
             KPtrs kb;
             for (int s = 0; s < 6; ++s) kb.k[s] = (float*)ctx->k[s];
             const float inv = 1.f / p.Ms;
-            dep(k_stage4<METHOD, S>, blocks_for(p.N / 4), kThreads, 0, ctx->stream)(
+            const int nt = threads_for(p.N / 4, sizeof(T));
+            dep(k_stage4<METHOD, S>, blocks_for(p.N / 4, nt), nt, 0, ctx->stream)(
                 p, p.A * p.cx * inv, p.A * p.cy * inv, p.A * p.cz * inv, (const float*)m_in, (const float*)ctx->Hd,
                 (const float*)m0, kb, (float*)m_out, ctx->ctl);
             MM_LAUNCH_CHECK(ctx);
             return MM_OK;
         }
     }
-    dep(k_stage<T, METHOD, S>, blocks_for(p.N), kThreads, 0, ctx->stream)(p, (const T*)m_in, (const T*)ctx->Hd,
+    const int nt = threads_for(p.N, sizeof(T));
+    dep(k_stage<T, METHOD, S>, blocks_for(p.N, nt), nt, 0, ctx->stream)(p, (const T*)m_in, (const T*)ctx->Hd,
                                                                           (const T*)m0, kdev, (T*)m_out, ctx->ctl);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
@@ -851,7 +953,8 @@ template <typename T>
 int exchange_t(mm_ctx* ctx, const void* m, void* H) {
     KernelTimer kt(ctx, MM_K_REDUCE);
     Params<T> p = make_params<T>(ctx);
-    dep(k_field<T, 0>, blocks_for(p.N), kThreads, 0, ctx->stream)(p, (const T*)m, nullptr, (T*)H);
+    const int nt = threads_for(p.N, sizeof(T));
+    dep(k_field<T, 0>, blocks_for(p.N, nt), nt, 0, ctx->stream)(p, (const T*)m, nullptr, (T*)H);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
@@ -859,7 +962,8 @@ template <typename T>
 int effective_t(mm_ctx* ctx, const void* m, const void* Hd, void* H) {
     KernelTimer kt(ctx, MM_K_REDUCE);
     Params<T> p = make_params<T>(ctx);
-    dep(k_field<T, 1>, blocks_for(p.N), kThreads, 0, ctx->stream)(p, (const T*)m, (const T*)Hd, (T*)H);
+    const int nt = threads_for(p.N, sizeof(T));
+    dep(k_field<T, 1>, blocks_for(p.N, nt), nt, 0, ctx->stream)(p, (const T*)m, (const T*)Hd, (T*)H);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
@@ -868,7 +972,8 @@ int energy_t(mm_ctx* ctx, const void* m, const void* Hd) {
     KernelTimer kt(ctx, MM_K_REDUCE);
     Params<T> p = make_params<T>(ctx);
     double V = ctx->dx * ctx->dy * ctx->dz;
-    dep(k_energy<T>, blocks_for(p.N), kThreads, 0, ctx->stream)(p, (const T*)m, (const T*)Hd, V, kMu0, ctx->Ku, ctx->ctl);
+    const unsigned nb = std::min(blocks_for(p.N, kReduceThreads), 152u * 8);
+    dep(k_energy<T>, nb, kReduceThreads, 0, ctx->stream)(p, (const T*)m, (const T*)Hd, V, kMu0, ctx->Ku, ctx->ctl);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
@@ -876,7 +981,8 @@ template <typename T>
 int torque_t(mm_ctx* ctx, const void* m, const void* Hd) {
     KernelTimer kt(ctx, MM_K_REDUCE);
     Params<T> p = make_params<T>(ctx);
-    dep(k_torque<T>, blocks_for(p.N), kThreads, 0, ctx->stream)(p, (const T*)m, (const T*)Hd, ctx->ctl);
+    const int nt = threads_for(p.N, sizeof(T));
+    dep(k_torque<T>, blocks_for(p.N, nt), nt, 0, ctx->stream)(p, (const T*)m, (const T*)Hd, ctx->ctl);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
@@ -915,11 +1021,16 @@ int rk_controller(mm_ctx* ctx, int method) {
 
 int rk_commit(mm_ctx* ctx, void* m0) {
     KernelTimer kt(ctx, MM_K_CONTROL);
-    long n3 = 3 * ctx->N;
-    if (ctx->prec == MM_F64)
-        dep(k_commit<double>, blocks_for(n3), kThreads, 0, ctx->stream)(n3, (const double*)ctx->mnext, (double*)m0, ctx->ctl);
+    const long n3 = 3 * ctx->N, e = ctx->prec == MM_F64 ? 8 : 4;
+    const bool wide = n3 * e % 16 == 0 && reinterpret_cast<uintptr_t>(m0) % 16 == 0;
+    const long n = wide ? n3 * e / 16 : n3;
+    const unsigned nb = blocks_for(n, 4 * kThreads);
+    if (wide)
+        dep(k_commit<float4>, nb, kThreads, 0, ctx->stream)(n, (const float4*)ctx->mnext, (float4*)m0, ctx->ctl);
+    else if (e == 8)
+        dep(k_commit<double>, nb, kThreads, 0, ctx->stream)(n, (const double*)ctx->mnext, (double*)m0, ctx->ctl);
     else
-        dep(k_commit<float>, blocks_for(n3), kThreads, 0, ctx->stream)(n3, (const float*)ctx->mnext, (float*)m0, ctx->ctl);
+        dep(k_commit<float>, nb, kThreads, 0, ctx->stream)(n, (const float*)ctx->mnext, (float*)m0, ctx->ctl);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
@@ -929,11 +1040,12 @@ int bb_iteration_t(mm_ctx* ctx, void* m, void* g, const void* g_prev, void* m_pr
                    long max_iter) {
     KernelTimer kt(ctx, MM_K_REDUCE);
     const Params<T> p = make_params<T>(ctx);
-    dep(k_bb_grad<T>, blocks_for(p.N), kThreads, 0, ctx->stream)(p, (const T*)m, (const T*)ctx->Hd, (T*)g,
+    const int nt = threads_for(p.N, sizeof(T));
+    dep(k_bb_grad<T>, blocks_for(p.N, nt), nt, 0, ctx->stream)(p, (const T*)m, (const T*)ctx->Hd, (T*)g,
                                                                 (const T*)g_prev, (const T*)m_prev, have_prev ? 1 : 0,
                                                                 ctx->ctl);
     dep(k_bb_tau, 1, 32, 0, ctx->stream)(ctx->ctl, tol, max_iter);
-    dep(k_bb_update<T>, blocks_for(p.N), kThreads, 0, ctx->stream)(p, (T*)m, (const T*)g, (T*)m_prev, ctx->ctl);
+    dep(k_bb_update<T>, blocks_for(p.N, nt), nt, 0, ctx->stream)(p, (T*)m, (const T*)g, (T*)m_prev, ctx->ctl);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
@@ -946,11 +1058,12 @@ int bb_iteration(mm_ctx* ctx, void* m, void* g, const void* g_prev, void* m_prev
 
 int check_finite_launch(mm_ctx* ctx, const void* m) {
     KernelTimer kt(ctx, MM_K_REDUCE);
-    long n3 = 3 * ctx->N;
+    const long n3 = 3 * ctx->N;
+    const unsigned nb = std::min(blocks_for(n3, 4 * kThreads), 152u * 8);
     if (ctx->prec == MM_F64)
-        dep(k_finite<double>, blocks_for(n3), kThreads, 0, ctx->stream)(n3, (const double*)m, ctx->ctl);
+        dep(k_finite<double>, nb, kThreads, 0, ctx->stream)(n3, (const double*)m, ctx->ctl);
     else
-        dep(k_finite<float>, blocks_for(n3), kThreads, 0, ctx->stream)(n3, (const float*)m, ctx->ctl);
+        dep(k_finite<float>, nb, kThreads, 0, ctx->stream)(n3, (const float*)m, ctx->ctl);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
