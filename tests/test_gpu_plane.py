@@ -69,6 +69,23 @@ def test_demag_on_padded_lengths_matches_oracle(n, prec):
     mm.mm_destroy(ctx)
 
 
+# FP64 meshes just above the size up to which a thread forms one output of a
+# transform: the four-step of every x length, and of y on single layers
+WIDE = [(16, 400, 16), (30, 320, 16), (33, 256, 16), (48, 256, 16), (64, 200, 8), (70, 160, 8), (90, 136, 8), (128, 100, 8),
+        (150, 64, 16), (190, 64, 16), (256, 50, 8), (300, 40, 8), (350, 36, 8), (512, 25, 8), (200, 129, 1), (257, 81, 1)]
+
+
+@pytest.mark.parametrize("n", WIDE, ids=lambda n: "x".join(map(str, n)))
+def test_fp64_above_the_one_output_size_matches_oracle(n):
+    m = wl.random_unit(n, seed=sum(n))
+    ctx = context(n, "f64")
+    md = dev(m, "f64")
+    H = torch.full_like(md, float("nan"))
+    mm.mm_demag_field(ctx, md, H)
+    assert rel(H, micromag.Problem(n, D).demag_fft(m)) < TOL["f64"]
+    mm.mm_destroy(ctx)
+
+
 @pytest.mark.parametrize("n", [(16, 8, 1), (32, 64, 2), (64, 32, 4), (8, 512, 1), (256, 16, 1), (512, 4, 2), (4, 4, 4)],
                          ids=lambda n: "x".join(map(str, n)))
 def test_float_float_planes_match_oracle(n):
