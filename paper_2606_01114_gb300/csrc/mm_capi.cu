@@ -195,19 +195,34 @@ int stage_field(mm_ctx* ctx, const void* m_in) {
     return demag_apply(ctx, m_in, ctx->Hd);
 }
 
-// one trial step from m (RK4 writes m in place; RKF45 writes mnext and commits)
-int trial(mm_ctx* ctx, void* m, int method) {
+// one trial step from m (RK4 writes m in place; RKF45 writes mnext and
+// commits); have_field: ctx->Hd holds the demag field of m already
+int trial(mm_ctx* ctx, void* m, int method, bool have_field = false, volatile int* mark = nullptr, int number = 0) {
     const int S = method == MM_RK4 ? 4 : 6;
     int rc;
     for (int s = 0; s < S; ++s) {
         const void* m_in = s == 0 ? m : ctx->ms[s % 2];
         void* m_out = s < S - 1 ? ctx->ms[(s + 1) % 2] : (method == MM_RK4 ? m : ctx->mnext);
-        if ((rc = stage_field(ctx, m_in))) return rc;
+        if (!(s == 0 && have_field) && (rc = stage_field(ctx, m_in))) return rc;
         if ((rc = rk_stage(ctx, method, s, m_in, m, m_out))) return rc;
     }
-    if ((rc = rk_controller(ctx, method))) return rc;
+    if ((rc = rk_controller(ctx, method, mark, number))) return rc;
     if (method == MM_RKF45 && (rc = rk_commit(ctx, m))) return rc;
     return MM_OK;
+}
+
+// Waits until trial `number` of relax()'s batch has been decided; true when no
+// further trial can change the state.  Ends when the stream has run dry, so an
+// error on the device does not hold it.
+bool trials_over(mm_ctx* ctx, int number) {
+    while (true) {
+        for (int spin = 0; spin < 2000; ++spin) {
+            const int v = *ctx->mark;
+            if (v < 0 || v >= number) return v < 0;
+        }
+        if (cudaStreamQuery(ctx->stream) != cudaErrorNotReady) return *ctx->mark < 0;
+        cudaGetLastError();   // not ready is no error
+    }
 }
 
 int device_status(mm_ctx* ctx) {
@@ -298,10 +313,11 @@ int mm_init_mesh(mm_ctx** out, int nx, int ny, int nz, double dx, double dy, dou
     A(&ctx->Ms_cell, (size_t)ctx->N * e);
     A(&ctx->A_cell, (size_t)ctx->N * e);
     A((void**)&ctx->ctl, sizeof(Control));
-    if (rc == MM_OK && cudaMallocHost((void**)&ctx->ctl_host, sizeof(Control)) != cudaSuccess) {
+    if (rc == MM_OK && cudaMallocHost((void**)&ctx->ctl_host, 2 * sizeof(Control)) != cudaSuccess) {
         cudaGetLastError();
         rc = fail(ctx, MM_ERR_NOMEM, "pinned allocation failed");
     }
+    if (rc == MM_OK) ctx->mark = (volatile int*)(ctx->ctl_host + 1);
     if (rc == MM_OK) {
         ctx->newell_host = (double*)malloc(sizeof(double) * 6 * ctx->N);
         if (!ctx->newell_host) rc = fail(ctx, MM_ERR_NOMEM, "host allocation failed");
@@ -494,8 +510,16 @@ int mm_relax(mm_ctx* ctx, void* m, double t_max, double torque_tol, long max_ste
         // steps still allowed stops relax at exactly max_steps
         const long room = max_steps - (long)c->steps;
         const int batch = room < kCheck ? (int)room : kCheck;
-        for (int k = 0; k < batch; ++k, ++attempts)
-            if ((rc = trial(ctx, m, MM_RKF45))) return rc;
+        // The first trial's first stage is the state whose demag field the
+        // torque was taken with.  The host stays two trials ahead of the
+        // device and stops when the end time is reached: the batch used to
+        // run to its end, with every field evaluation of up to nine trials
+        // that change nothing (100x25x1 FP64 to 8 ps: 4.03 -> 3.23 ms).
+        *ctx->mark = 0;
+        for (int k = 0; k < batch; ++k, ++attempts) {
+            if (k >= 2 && trials_over(ctx, k - 1)) break;
+            if ((rc = trial(ctx, m, MM_RKF45, k == 0, ctx->mark, k + 1))) return rc;
+        }
     }
 }
 

@@ -152,6 +152,7 @@ struct mm_ctx {
     void* m_stage;            // [3][N] device copy of a host state (mm_llg_step_host), allocated on first use
     mm::Control* ctl;         // device control block
     mm::Control* ctl_host;    // pinned host mirror
+    volatile int* mark;       // pinned, behind it: how far the trials of relax() have come
     double* newell_host;      // [6][nz][ny][nx] real-space tensor (host copy)
     mm::Tables tw;
     mm::Blue blue_x, blue_y;  // Bluestein data of Px and Py when they are not powers of two
@@ -321,7 +322,8 @@ int torque_launch(mm_ctx* ctx, const void* m, const void* Hd);   // max into ctl
 // One RK stage: k[s] = LLG(ms_in, H_eff(ms_in)); writes next trial state or,
 // at the last stage, the candidate mnext (+ error).  method MM_RK4/MM_RKF45.
 int rk_stage(mm_ctx* ctx, int method, int s, const void* m_in, const void* m0, void* m_out);
-int rk_controller(mm_ctx* ctx, int method);            // accept / reject, dt
+// accept / reject, dt; mark: see k_controller
+int rk_controller(mm_ctx* ctx, int method, volatile int* mark, int number);
 int rk_commit(mm_ctx* ctx, void* m0);                  // m0 <- mnext if accepted
 int check_finite_launch(mm_ctx* ctx, const void* m);
 // One Barzilai-Borwein iteration after the demag field of m is in ctx->Hd:

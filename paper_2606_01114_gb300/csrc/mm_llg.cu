@@ -558,10 +558,10 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// RKF45 step control on the device.
-__global__ void k_controller(Control* ctl, int method) {
-    dep_wait();
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// RKF45 step control on the device.  mark (pinned host memory, or NULL): the
+// trial's number once it has been decided, -1 when no further trial can change
+// the state.
+__device__ __forceinline__ void control_step(Control* ctl, int method) {
     if (ctl->status != 0 || ctl->done) {
         ctl->accepted = 0;
         return;
@@ -602,6 +602,12 @@ __global__ void k_controller(Control* ctl, int method) {
         dtn = rem;
     }
     ctl->dt = dtn;
+}
+__global__ void k_controller(Control* ctl, int method, volatile int* mark, int number) {
+    dep_wait();
+    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    control_step(ctl, method);
+    if (mark) *mark = ctl->status != 0 || ctl->done ? -1 : number;
 }
 
 // V: float4 or double2 where both arrays are 16-byte aligned (the scalar form
@@ -1012,9 +1018,9 @@ int rk_stage(mm_ctx* ctx, int method, int s, const void* m_in, const void* m0, v
                             : stage_dispatch<float, MM_RKF45>(ctx, s, m_in, m0, m_out);
 }
 
-int rk_controller(mm_ctx* ctx, int method) {
+int rk_controller(mm_ctx* ctx, int method, volatile int* mark, int number) {
     KernelTimer kt(ctx, MM_K_CONTROL);
-    dep(k_controller, 1, 32, 0, ctx->stream)(ctx->ctl, method);
+    dep(k_controller, 1, 32, 0, ctx->stream)(ctx->ctl, method, mark, number);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
