@@ -246,23 +246,27 @@ struct StepTape {
 // One RK4 step from m, recording its tape; m_next = NULL stops after the
 // demag field of X3 (the last step of a segment, whose successor is known).
 int rk4_step_record(mm_ctx* ctx, const void* m, void* m_next, const StepTape& tp) {
-    const size_t v = 3 * (size_t)ctx->N * (ctx->prec == MM_F64 ? sizeof(double) : sizeof(float));
-    void* hd_saved = ctx->Hd;
+    void* const hd_saved = ctx->Hd;
+    void* const k_saved[3] = {ctx->k[0], ctx->k[1], ctx->k[2]};
+    for (int q = 0; q < 3; ++q) ctx->k[q] = tp.k[q];     // the slopes are written into the tape
+    const bool fused = plane_fused(ctx);
     int rc = MM_OK;
     const void* Xs = m;
     for (int s = 0; s < 4 && rc == MM_OK; ++s) {
-        ctx->Hd = tp.H[s];
-        rc = demag_apply(ctx, Xs, tp.H[s]);
-        if (rc || (s == 3 && !m_next)) break;
         void* out = s < 3 ? tp.X[s] : m_next;
-        rc = rk_stage(ctx, MM_RK4, s, Xs, m, out);
-        if (!rc && s < 3) {
-            cudaError_t ce = cudaMemcpyAsync(tp.k[s], ctx->k[s], v, cudaMemcpyDeviceToDevice, ctx->stream);
-            if (ce != cudaSuccess) rc = fail(ctx, MM_ERR_CUDA, "tape copy: %s", cudaGetErrorString(ce));
+        if (fused && out) {
+            if (s == 0) rc = plane_xfwd(ctx, m);
+            if (!rc) rc = plane_yzy(ctx);
+            if (!rc) rc = plane_stage(ctx, MM_RK4, s, Xs, m, out, tp.H[s], s < 2 || (s == 2 && m_next));
+        } else {
+            ctx->Hd = tp.H[s];
+            rc = demag_apply(ctx, Xs, tp.H[s]);
+            if (!rc && out) rc = rk_stage(ctx, MM_RK4, s, Xs, m, out);
         }
         Xs = out;
     }
     ctx->Hd = hd_saved;
+    for (int q = 0; q < 3; ++q) ctx->k[q] = k_saved[q];
     return rc;
 }
 
@@ -352,11 +356,19 @@ int exchange_vjp_t(mm_ctx* ctx, const T* g, const T* m, T* gm, T* gMs) {
 // n fixed RK4 steps of m in place, no host synchronisation (the caller's
 // control block must hold dt)
 int rk4_steps(mm_ctx* ctx, void* m, long n) {
+    const bool fused = plane_fused(ctx);
     int rc;
     for (long k = 0; k < n; ++k) {
         for (int s = 0; s < 4; ++s) {
             const void* m_in = s == 0 ? m : ctx->ms[s % 2];
             void* m_out = s < 3 ? ctx->ms[(s + 1) % 2] : m;
+            if (fused) {
+                // every step is taken, so its last stage transforms the new state for the next step
+                if (k == 0 && s == 0 && (rc = plane_xfwd(ctx, m))) return rc;
+                if ((rc = plane_yzy(ctx))) return rc;
+                if ((rc = plane_stage(ctx, MM_RK4, s, m_in, m, m_out, nullptr, s < 3 || k + 1 < n))) return rc;
+                continue;
+            }
             if ((rc = demag_apply(ctx, m_in, ctx->Hd))) return rc;
             if ((rc = rk_stage(ctx, MM_RK4, s, m_in, m, m_out))) return rc;
         }

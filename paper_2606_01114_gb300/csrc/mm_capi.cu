@@ -97,7 +97,7 @@ size_t elem(const mm_ctx* ctx) { return ctx->prec == MM_F64 ? sizeof(double) : s
 
 void free_all(mm_ctx* ctx) {
     void* ptrs[] = {ctx->Ms_cell, ctx->A_cell, ctx->kern, ctx->bufA, ctx->bufB, ctx->Hd, ctx->Hs_field,
-                    ctx->m0, ctx->ms[0], ctx->ms[1], ctx->mnext, ctx->kptrs, ctx->ctl, ctx->tw.f64, ctx->tw.f32,
+                    ctx->m0, ctx->ms[0], ctx->ms[1], ctx->mnext, ctx->ctl, ctx->tw.f64, ctx->tw.f32,
                     ctx->tw.ff, ctx->kern_ff, ctx->adj, ctx->m_stage, ctx->kern_f4, ctx->tw_f4,
                     ctx->blue_x.chirp, ctx->blue_x.filt, ctx->blue_x.tw, ctx->blue_y.chirp, ctx->blue_y.filt,
                     ctx->blue_y.tw, ctx->blue_x.chirp32, ctx->blue_x.filt32, ctx->blue_x.tw32, ctx->blue_y.chirp32,
@@ -199,10 +199,21 @@ int stage_field(mm_ctx* ctx, const void* m_in) {
 // commits); have_field: ctx->Hd holds the demag field of m already
 int trial(mm_ctx* ctx, void* m, int method, bool have_field = false, volatile int* mark = nullptr, int number = 0) {
     const int S = method == MM_RK4 ? 4 : 6;
+    const bool fused = !ctx->stage_surrogate && plane_fused(ctx);
     int rc;
     for (int s = 0; s < S; ++s) {
         const void* m_in = s == 0 ? m : ctx->ms[s % 2];
         void* m_out = s < S - 1 ? ctx->ms[(s + 1) % 2] : (method == MM_RK4 ? m : ctx->mnext);
+        if (fused) {
+            // have_field: the planes hold that field's spectrum still
+            if (!(s == 0 && have_field)) {
+                ++ctx->exact_evals;
+                if (s == 0 && (rc = plane_xfwd(ctx, m))) return rc;
+                if ((rc = plane_yzy(ctx))) return rc;
+            }
+            if ((rc = plane_stage(ctx, method, s, m_in, m, m_out, nullptr, s < S - 1))) return rc;
+            continue;
+        }
         if (!(s == 0 && have_field) && (rc = stage_field(ctx, m_in))) return rc;
         if ((rc = rk_stage(ctx, method, s, m_in, m, m_out))) return rc;
     }
@@ -309,7 +320,6 @@ int mm_init_mesh(mm_ctx** out, int nx, int ny, int nz, double dx, double dy, dou
     A(&ctx->ms[1], v3);
     A(&ctx->mnext, v3);
     for (int s = 0; s < 6; ++s) A(&ctx->k[s], v3);
-    A(&ctx->kptrs, 6 * sizeof(void*));
     A(&ctx->Ms_cell, (size_t)ctx->N * e);
     A(&ctx->A_cell, (size_t)ctx->N * e);
     A((void**)&ctx->ctl, sizeof(Control));
@@ -321,10 +331,6 @@ int mm_init_mesh(mm_ctx** out, int nx, int ny, int nz, double dx, double dy, dou
     if (rc == MM_OK) {
         ctx->newell_host = (double*)malloc(sizeof(double) * 6 * ctx->N);
         if (!ctx->newell_host) rc = fail(ctx, MM_ERR_NOMEM, "host allocation failed");
-    }
-    if (rc == MM_OK) {
-        cudaError_t ce = cudaMemcpy(ctx->kptrs, ctx->k, 6 * sizeof(void*), cudaMemcpyHostToDevice);
-        if (ce != cudaSuccess) rc = fail(ctx, MM_ERR_CUDA, "cudaMemcpy: %s", cudaGetErrorString(ce));
     }
     if (rc == MM_OK) rc = make_tables(ctx);
     if (rc == MM_OK) {
@@ -420,6 +426,7 @@ int mm_effective_field(mm_ctx* ctx, const void* m, void* H) {
     if (!ctx) return fail(nullptr, MM_ERR_INVALID_ARG, "ctx is NULL");
     MM_BIND(ctx);
     if (!m || !H) return fail(ctx, MM_ERR_INVALID_ARG, "m and H must be device pointers");
+    if (plane_fused(ctx)) return plane_field(ctx, m, H);
     int rc = demag_apply(ctx, m, ctx->Hd);
     if (rc) return rc;
     bool done = false;

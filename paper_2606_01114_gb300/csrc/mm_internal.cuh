@@ -147,7 +147,6 @@ struct mm_ctx {
     void* ms[2];              // [3][N] trial states (ping-pong)
     void* mnext;              // [3][N] accepted-candidate state
     void* k[6];               // [3][N] RK stage slopes
-    void* kptrs;              // device copy of k[0..5]
     void* adj;                // adjoint workspace (14 fields of [3][N]), allocated on first use
     void* m_stage;            // [3][N] device copy of a host state (mm_llg_step_host), allocated on first use
     mm::Control* ctl;         // device control block
@@ -289,6 +288,15 @@ int plane_setup(mm_ctx* ctx);
 void plane_free(mm_ctx* ctx);
 int plane_apply(mm_ctx* ctx, const void* m, void* H, bool unit);
 int plane_prepare_ff(mm_ctx* ctx);
+// fused x inverse, cells and x forward (mm_plane_step.cu): plane_fused tells
+// whether the context's current mode takes it.  plane_stage runs Runge-Kutta
+// stage s on the planes that plane_yzy left and, with `forward`, leaves the
+// planes of m_out for the next plane_yzy; hd (or NULL) receives the demag field.
+bool plane_fused(const mm_ctx* ctx);
+int plane_xfwd(mm_ctx* ctx, const void* m);
+int plane_yzy(mm_ctx* ctx);
+int plane_stage(mm_ctx* ctx, int method, int s, const void* m_in, const void* m0, void* m_out, void* hd, bool forward);
+int plane_field(mm_ctx* ctx, const void* m, void* H);
 // appends the four-step tables w^(t k1), [k1][t] and then [t][k1], of an x or
 // y length (or a z length) of mm_plane_launch.cuh; nothing for other lengths
 void four_step_table(int len, bool z, std::vector<double>& out);

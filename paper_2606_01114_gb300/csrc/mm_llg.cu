@@ -20,73 +20,10 @@
 
 #include "mm_ff.cuh"
 #include "mm_fields.cuh"
+#include "mm_rk.cuh"
 
 namespace mm {
 namespace {
-
-// ---------------------------------------------------- Butcher tableaux
-// classic RK4 and Fehlberg's RKF45 (4th-order weights propagated)
-__host__ __device__ constexpr double rk_a(int method, int i, int j) {
-    if (method == MM_RK4) {
-        if (i == 1 && j == 0) return 0.5;
-        if (i == 2 && j == 1) return 0.5;
-        if (i == 3 && j == 2) return 1.0;
-        return 0.0;
-    }
-    switch (i * 8 + j) {
-        case 1 * 8 + 0: return 1.0 / 4.0;
-        case 2 * 8 + 0: return 3.0 / 32.0;
-        case 2 * 8 + 1: return 9.0 / 32.0;
-        case 3 * 8 + 0: return 1932.0 / 2197.0;
-        case 3 * 8 + 1: return -7200.0 / 2197.0;
-        case 3 * 8 + 2: return 7296.0 / 2197.0;
-        case 4 * 8 + 0: return 439.0 / 216.0;
-        case 4 * 8 + 1: return -8.0;
-        case 4 * 8 + 2: return 3680.0 / 513.0;
-        case 4 * 8 + 3: return -845.0 / 4104.0;
-        case 5 * 8 + 0: return -8.0 / 27.0;
-        case 5 * 8 + 1: return 2.0;
-        case 5 * 8 + 2: return -3544.0 / 2565.0;
-        case 5 * 8 + 3: return 1859.0 / 4104.0;
-        case 5 * 8 + 4: return -11.0 / 40.0;
-        default: return 0.0;
-    }
-}
-__host__ __device__ constexpr double rk_b(int method, int j) {
-    if (method == MM_RK4) {
-        return j == 0 ? 1.0 / 6.0 : j == 1 ? 1.0 / 3.0 : j == 2 ? 1.0 / 3.0 : j == 3 ? 1.0 / 6.0 : 0.0;
-    }
-    return j == 0 ? 25.0 / 216.0 : j == 2 ? 1408.0 / 2565.0 : j == 3 ? 2197.0 / 4104.0 : j == 4 ? -1.0 / 5.0 : 0.0;
-}
-// b5 - b4 (RKF45 error weights)
-__host__ __device__ constexpr double rk_e(int method, int j) {
-    if (method == MM_RK4) return 0.0;
-    constexpr double b5[6] = {16.0 / 135.0, 0.0, 6656.0 / 12825.0, 28561.0 / 56430.0, -9.0 / 50.0, 2.0 / 55.0};
-    return b5[j] - rk_b(method, j);
-}
-__host__ __device__ constexpr int rk_stages(int method) { return method == MM_RK4 ? 4 : 6; }
-
-// Block-wide max of a non-negative double, then one atomicMax of its bits.
-// Non-negative doubles order like their bit patterns, so the maxima are
-// integer reductions and none of it runs on the FP64 pipe.
-__device__ __forceinline__ unsigned long long warp_max_bits(unsigned long long v) {
-    const unsigned hi = (unsigned)(v >> 32);
-    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
-    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)v : 0u);
-    return ((unsigned long long)mh << 32) | ml;
-}
-__device__ __forceinline__ void block_max_atomic(double v, unsigned long long* target) {
-    __shared__ unsigned long long red[32];
-    unsigned long long u = warp_max_bits((unsigned long long)__double_as_longlong(v));
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) red[w] = u;
-    __syncthreads();
-    if (w == 0) {
-        const int nw = (blockDim.x + 31) >> 5;
-        u = warp_max_bits(lane < nw ? red[lane] : 0ull);
-        if (lane == 0 && u != 0ull) atomicMax(target, u);
-    }
-}
 
 __device__ __forceinline__ void block_sum_atomic(double v, double* target) {
     __shared__ double red[32];
@@ -162,7 +99,7 @@ __global__ void k_field(Params<T> p, const T* __restrict__ m, const T* __restric
 // ------------------------------------------------------------- K7 stage
 template <typename T, int METHOD, int S>
 __global__ void k_stage(Params<T> p, const T* __restrict__ m_in, const T* __restrict__ Hd, const T* m0,
-                        T* const* __restrict__ kbuf, T* m_out, Control* ctl) {
+                        KPtrs<T> kb, T* m_out, Control* ctl) {
     dep_wait();
     constexpr int NS = rk_stages(METHOD);
     constexpr bool LAST = (S == NS - 1);
@@ -200,7 +137,7 @@ __global__ void k_stage(Params<T> p, const T* __restrict__ m_in, const T* __rest
             for (int j = 0; j < S; ++j) {
                 const T c = (T)rk_a(METHOD, S + 1, j);
                 if (c != (T)0) {
-                    V3<T> kj = load3(kbuf[j], i, p.N);
+                    V3<T> kj = load3((const T*)kb.k[j], i, p.N);
                     acc.x += c * kj.x;
                     acc.y += c * kj.y;
                     acc.z += c * kj.z;
@@ -210,7 +147,7 @@ __global__ void k_stage(Params<T> p, const T* __restrict__ m_in, const T* __rest
             acc.x += cs * ks.x;
             acc.y += cs * ks.y;
             acc.z += cs * ks.z;
-            store3(kbuf[S], i, p.N, ks);
+            store3(kb.k[S], i, p.N, ks);
             store3(m_out, i, p.N, V3<T>{a0.x + dt * acc.x, a0.y + dt * acc.y, a0.z + dt * acc.z});
         } else {
             V3<T> acc = {0, 0, 0}, e = {0, 0, 0};
@@ -218,7 +155,7 @@ __global__ void k_stage(Params<T> p, const T* __restrict__ m_in, const T* __rest
             for (int j = 0; j < NS; ++j) {
                 const T cb = (T)rk_b(METHOD, j), ce = (T)rk_e(METHOD, j);
                 if (cb != (T)0 || ce != (T)0) {
-                    V3<T> kj = j == S ? ks : load3(kbuf[j], i, p.N);
+                    V3<T> kj = j == S ? ks : load3((const T*)kb.k[j], i, p.N);
                     acc.x += cb * kj.x;
                     acc.y += cb * kj.y;
                     acc.z += cb * kj.z;
@@ -249,12 +186,7 @@ __global__ void k_stage(Params<T> p, const T* __restrict__ m_in, const T* __rest
 
 // K7, FP32, uniform material, nx % 4 == 0: four x-consecutive cells per
 // thread with 16-byte loads and stores (the same arithmetic per cell as
-// k_stage; the exchange weights A c_axis / Ms folded once).  Slope pointers
-// travel by value.
-struct KPtrs {
-    float* k[6];
-};
-
+// k_stage; the exchange weights A c_axis / Ms folded once).
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
 __device__ __forceinline__ float& at(float4& v, int j) { return (&v.x)[j]; }
@@ -285,7 +217,7 @@ __device__ __forceinline__ void add_diff(Cells4& acc, const Cells4& nb, const Ce
 template <int METHOD, int S>
 __global__ void __launch_bounds__(256) k_stage4(Params<float> p, float wx, float wy, float wz,
                                                 const float* __restrict__ m_in, const float* __restrict__ Hd,
-                                                const float* m0, KPtrs kb, float* m_out, Control* ctl) {
+                                                const float* m0, KPtrs<float> kb, float* m_out, Control* ctl) {
     dep_wait();
     constexpr int NS = rk_stages(METHOD);
     constexpr bool LAST = (S == NS - 1);
@@ -424,9 +356,6 @@ __global__ void __launch_bounds__(256) k_stage4(Params<float> p, float wx, float
 // RKF45 error is reduced as the squared norm per block, with one square root
 // per block; the renormalisation uses a float-float Newton inverse square
 // root started from rsqrtf.
-struct KPtrsD {
-    double* k[6];
-};
 struct FFStageCoef {
     ff wx, wy, wz;     // A (2 / (mu0 d^2)) / Ms per axis
     ff anis;           // 2 Ku / (mu0 Ms)
@@ -447,7 +376,7 @@ __device__ __forceinline__ ff half_of(ff a) { return ff(0.5f * a.h, 0.5f * a.l);
 template <int METHOD, int S>
 __global__ void __launch_bounds__(256)
     k_stage_ff(FFStageCoef c, int nx, int ny, int nz, long N, const double* __restrict__ m_in,
-               const double* __restrict__ Hd, const double* m0, KPtrsD kb, double* m_out, Control* ctl) {
+               const double* __restrict__ Hd, const double* m0, KPtrs<double> kb, double* m_out, Control* ctl) {
     dep_wait();
     constexpr int NS = rk_stages(METHOD);
     constexpr bool LAST = (S == NS - 1);
@@ -888,12 +817,11 @@ __global__ void k_bb_update(Params<T> p, T* __restrict__ m, const T* __restrict_
 }
 
 template <typename T, int METHOD, int S>
-int launch_stage(mm_ctx* ctx, const Params<T>& p, const void* m_in, const void* m0, void* m_out, T* const* kdev) {
+int launch_stage(mm_ctx* ctx, const Params<T>& p, const void* m_in, const void* m0, void* m_out) {
     KernelTimer kt(ctx, MM_K_STAGE);
+    const KPtrs<T> kb = slopes<T>(ctx);
     if constexpr (sizeof(T) == 8) {
         if (ctx->fft_mode == MM_FFT_FF && !p.Ms_cell && !p.A_cell && p.Ms != 0.0 && !p.dmi && !p.stt) {
-            KPtrsD kb;
-            for (int s = 0; s < 6; ++s) kb.k[s] = (double*)ctx->k[s];
             const double inv = 1.0 / (double)p.Ms;
             FFStageCoef c;
             c.wx = ff((double)(p.A * p.cx) * inv);
@@ -918,8 +846,6 @@ int launch_stage(mm_ctx* ctx, const Params<T>& p, const void* m_in, const void* 
     }
     if constexpr (sizeof(T) == 4) {
         if (!p.Ms_cell && !p.A_cell && p.Ms != 0.f && p.nx % 4 == 0 && !p.dmi && !p.stt) {
-            KPtrs kb;
-            for (int s = 0; s < 6; ++s) kb.k[s] = (float*)ctx->k[s];
             const float inv = 1.f / p.Ms;
             const int nt = threads_for(p.N / 4, sizeof(T));
             dep(k_stage4<METHOD, S>, blocks_for(p.N / 4, nt), nt, 0, ctx->stream)(
@@ -931,7 +857,7 @@ int launch_stage(mm_ctx* ctx, const Params<T>& p, const void* m_in, const void* 
     }
     const int nt = threads_for(p.N, sizeof(T));
     dep(k_stage<T, METHOD, S>, blocks_for(p.N, nt), nt, 0, ctx->stream)(p, (const T*)m_in, (const T*)ctx->Hd,
-                                                                          (const T*)m0, kdev, (T*)m_out, ctx->ctl);
+                                                                          (const T*)m0, kb, (T*)m_out, ctx->ctl);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
 }
@@ -939,17 +865,16 @@ int launch_stage(mm_ctx* ctx, const Params<T>& p, const void* m_in, const void* 
 template <typename T, int METHOD>
 int stage_dispatch(mm_ctx* ctx, int s, const void* m_in, const void* m0, void* m_out) {
     Params<T> p = make_params<T>(ctx);
-    T* const* kdev = (T* const*)ctx->kptrs;
     switch (s) {
-        case 0: return launch_stage<T, METHOD, 0>(ctx, p, m_in, m0, m_out, kdev);
-        case 1: return launch_stage<T, METHOD, 1>(ctx, p, m_in, m0, m_out, kdev);
-        case 2: return launch_stage<T, METHOD, 2>(ctx, p, m_in, m0, m_out, kdev);
-        case 3: return launch_stage<T, METHOD, 3>(ctx, p, m_in, m0, m_out, kdev);
+        case 0: return launch_stage<T, METHOD, 0>(ctx, p, m_in, m0, m_out);
+        case 1: return launch_stage<T, METHOD, 1>(ctx, p, m_in, m0, m_out);
+        case 2: return launch_stage<T, METHOD, 2>(ctx, p, m_in, m0, m_out);
+        case 3: return launch_stage<T, METHOD, 3>(ctx, p, m_in, m0, m_out);
         case 4:
-            if constexpr (METHOD == MM_RKF45) return launch_stage<T, METHOD, 4>(ctx, p, m_in, m0, m_out, kdev);
+            if constexpr (METHOD == MM_RKF45) return launch_stage<T, METHOD, 4>(ctx, p, m_in, m0, m_out);
             break;
         case 5:
-            if constexpr (METHOD == MM_RKF45) return launch_stage<T, METHOD, 5>(ctx, p, m_in, m0, m_out, kdev);
+            if constexpr (METHOD == MM_RKF45) return launch_stage<T, METHOD, 5>(ctx, p, m_in, m0, m_out);
             break;
     }
     return fail(ctx, MM_ERR_INVALID_ARG, "bad stage %d", s);

@@ -11,6 +11,8 @@ namespace mm {
 int plane_apply_f32(mm_ctx* ctx, const float* m, const float* Ms, float ms, float* H);
 int plane_apply_f64(mm_ctx* ctx, const double* m, const double* Ms, double ms, double* H);
 int plane_apply_ff(mm_ctx* ctx, const double* m, const double* Ms, double ms, double* H);
+int plane_xfwd_f32(mm_ctx* ctx, const float* m, const float* Ms, float ms);
+int plane_yzy_f32(mm_ctx* ctx);
 int plane_line_len(int P);
 
 namespace {
@@ -267,5 +269,11 @@ int plane_apply(mm_ctx* ctx, const void* m, void* H, bool unit) {
         return plane_apply_ff(ctx, (const double*)m, (const double*)Ms, ms, (double*)H);
     return plane_apply_f64(ctx, (const double*)m, (const double*)Ms, ms, (double*)H);
 }
+
+// the two parts of a field evaluation before the fused kernel (FP32)
+int plane_xfwd(mm_ctx* ctx, const void* m) {
+    return plane_xfwd_f32(ctx, (const float*)m, ctx->has_Ms_cell ? (const float*)ctx->Ms_cell : nullptr, (float)ctx->Ms);
+}
+int plane_yzy(mm_ctx* ctx) { return plane_yzy_f32(ctx); }
 
 }  // namespace mm

@@ -23,15 +23,17 @@ void four_step_table(int len, bool z, std::vector<double>& out) {
     else with_length(len, [&](auto A, auto B) { put(decltype(A)::value, decltype(B)::value); });
 }
 
+int plane_xfwd_f32(mm_ctx* ctx, const float* m, const float* Ms, float ms) {
+    return launch_px_fwd<float, float>(ctx, m, Ms, ms, (long)ctx->nz * ctx->ny, (float2*)ctx->plane.buf,
+                                       3L * ctx->nz * ctx->ny, (const float2*)ctx->plane.tw);
+}
+
 int plane_apply_f32(mm_ctx* ctx, const float* m, const float* Ms, float ms, float* H) {
     const PlanePlan& p = ctx->plane;
-    const long rows = 3L * ctx->nz * ctx->ny;
-    const float2* tw = (const float2*)p.tw;
-    float2* buf = (float2*)p.buf;
-    int rc = launch_px_fwd<float, float>(ctx, m, Ms, ms, (long)ctx->nz * ctx->ny, buf, rows, tw);
+    int rc = plane_xfwd_f32(ctx, m, Ms, ms);
     if (rc || (rc = plane_yzy_f32(ctx))) return rc;
     const float scale = (float)(1.0 / ((double)p.L * p.P * ctx->Pz));
-    return launch_px_inv<float, float>(ctx, buf, H, rows, scale, tw);
+    return launch_px_inv<float, float>(ctx, (const float2*)p.buf, H, 3L * ctx->nz * ctx->ny, scale, (const float2*)p.tw);
 }
 
 }  // namespace mm
