@@ -51,30 +51,26 @@ __device__ __forceinline__ V3<T> stencil_g_over_ms(const Params<T>& p, const T* 
     const T Ai = p.A_cell ? p.A_cell[i] : p.A;
     const T inv_i = (T)1 / Msi;
     const V3<T> qi = {g[i] * inv_i, g[i + p.N] * inv_i, g[i + 2 * p.N] * inv_i};
-    V3<T> acc = {0, 0, 0};
-    auto nb = [&](long j, T c) {
-        T Msj = ms_at(p, j);
-        if (Msj == (T)0) return;
-        T Ah;
-        if (p.A_cell) {
-            T Aj = p.A_cell[j];
-            T s = Ai + Aj;
-            Ah = s > (T)0 ? (T)2 * Ai * Aj / s : (T)0;
-        } else {
-            Ah = p.A;
+    const int nb = p.nz > 1 ? 6 : 4;
+    const Bonds<T> q = bonds_of(p, i, x, y, z);
+    V3<T> v[6];
+    T Ms[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+        if (k < nb) {
+            v[k] = load3(g, q.j[k], p.N);
+            Ms[k] = ms_at(p, q.j[k]);
         }
-        const T w = Ah * c, inv_j = (T)1 / Msj;
-        acc.x += w * (g[j] * inv_j - qi.x);
-        acc.y += w * (g[j + p.N] * inv_j - qi.y);
-        acc.z += w * (g[j + 2 * p.N] * inv_j - qi.z);
-    };
-    const long sy = p.nx, sz = (long)p.nx * p.ny;
-    if (x > 0) nb(i - 1, p.cx);
-    if (x < p.nx - 1) nb(i + 1, p.cx);
-    if (y > 0) nb(i - sy, p.cy);
-    if (y < p.ny - 1) nb(i + sy, p.cy);
-    if (z > 0) nb(i - sz, p.cz);
-    if (z < p.nz - 1) nb(i + sz, p.cz);
+    V3<T> acc = {0, 0, 0};
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        if (k < nb && q.on[k]) {
+            const T w = bond_weight(p, q, k, Ai), inv_j = (T)1 / Ms[k];
+            acc.x += w * (v[k].x * inv_j - qi.x);
+            acc.y += w * (v[k].y * inv_j - qi.y);
+            acc.z += w * (v[k].z * inv_j - qi.z);
+        }
+    }
     return acc;
 }
 

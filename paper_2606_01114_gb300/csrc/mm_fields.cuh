@@ -89,35 +89,67 @@ template <typename T> __device__ __forceinline__ T inv_ms_at(const Params<T>& p,
     return p.Ms_cell ? (T)1 / Msi : p.inv_Ms;
 }
 
+// The six bonds of a cell, loads first.  A neighbour outside the mesh is read as
+// the cell itself (its difference is zero) and a vacuum neighbour's difference
+// is replaced by zero after the loads, so nothing a load needs waits for
+// another load: with the test before each neighbour's loads the cell kernels
+// went through six dependent pairs of L2 accesses when Ms varies.
+template <typename T> struct Bonds {
+    long j[6];           // -x, +x, -y, +y, -z, +z
+    bool on[6];          // inside the mesh and magnetic
+};
+template <typename T>
+__device__ __forceinline__ Bonds<T> bonds_of(const Params<T>& p, long i, int x, int y, int z) {
+    const long sy = p.nx, sz = (long)p.nx * p.ny;
+    Bonds<T> q;
+    q.on[0] = x > 0;
+    q.on[1] = x < p.nx - 1;
+    q.on[2] = y > 0;
+    q.on[3] = y < p.ny - 1;
+    q.on[4] = z > 0;
+    q.on[5] = z < p.nz - 1;
+    const long s[3] = {1, sy, sz};
+#pragma unroll
+    for (int k = 0; k < 6; ++k) q.j[k] = q.on[k] ? i + (k & 1 ? s[k / 2] : -s[k / 2]) : i;
+    if (p.Ms_cell) {
+        T Ms[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) Ms[k] = p.Ms_cell[q.j[k]];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) q.on[k] = q.on[k] && Ms[k] != (T)0;
+    }
+    return q;
+}
+// A_h times the axis constant of bond k (harmonic mean of both cells' A)
+template <typename T>
+__device__ __forceinline__ T bond_weight(const Params<T>& p, const Bonds<T>& q, int k, T Ai) {
+    const T c = k < 2 ? p.cx : k < 4 ? p.cy : p.cz;
+    if (!p.A_cell) return p.A * c;
+    const T Aj = p.A_cell[q.j[k]], s = Ai + Aj;
+    return (s > (T)0 ? (T)2 * Ai * Aj / s : (T)0) * c;
+}
+
 // exchange field at cell i (x, y, z) of state m; inv = 1 / Ms_i
 template <typename T>
 __device__ __forceinline__ V3<T> exchange_at(const Params<T>& p, const T* __restrict__ m, long i, int x, int y,
                                              int z, V3<T> mi, T inv) {
     const T Ai = p.A_cell ? p.A_cell[i] : p.A;
+    const int nb = p.nz > 1 ? 6 : 4;
+    V3<T> v[6];
+    const Bonds<T> q = bonds_of(p, i, x, y, z);
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+        if (k < nb) v[k] = load3(m, q.j[k], p.N);
     T ax = 0, ay = 0, az = 0;
-    auto nb = [&](long j, T c) {
-        T Msj = p.Ms_cell ? p.Ms_cell[j] : p.Ms;
-        if (Msj == (T)0) return;
-        T Ah;
-        if (p.A_cell) {
-            T Aj = p.A_cell[j];
-            T s = Ai + Aj;
-            Ah = s > (T)0 ? (T)2 * Ai * Aj / s : (T)0;
-        } else {
-            Ah = p.A;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        if (k < nb && q.on[k]) {
+            const T w = bond_weight(p, q, k, Ai);
+            ax += w * (v[k].x - mi.x);
+            ay += w * (v[k].y - mi.y);
+            az += w * (v[k].z - mi.z);
         }
-        T w = Ah * c;
-        ax += w * (m[j] - mi.x);
-        ay += w * (m[j + p.N] - mi.y);
-        az += w * (m[j + 2 * p.N] - mi.z);
-    };
-    const long sx = 1, sy = p.nx, sz = (long)p.nx * p.ny;
-    if (x > 0) nb(i - sx, p.cx);
-    if (x < p.nx - 1) nb(i + sx, p.cx);
-    if (y > 0) nb(i - sy, p.cy);
-    if (y < p.ny - 1) nb(i + sy, p.cy);
-    if (z > 0) nb(i - sz, p.cz);
-    if (z < p.nz - 1) nb(i + sz, p.cz);
+    }
     return {ax * inv, ay * inv, az * inv};
 }
 
@@ -139,23 +171,29 @@ template <typename T>
 __device__ __forceinline__ V3<T> dmi_at(const Params<T>& p, const T* __restrict__ m, long i, int x, int y, int z,
                                         T inv) {
     T hx = 0, hy = 0, hz = 0;
-    // sum over the present neighbours of sign * (m_nb) per axis: v_axis
-    auto acc = [&](long j, T sgn, T& vx, T& vy, T& vz) {
-        if (p.Ms_cell && p.Ms_cell[j] == (T)0) return;
-        vx += sgn * m[j];
-        vy += sgn * m[j + p.N];
-        vz += sgn * m[j + 2 * p.N];
-    };
-    const long sx = 1, sy = p.nx, sz = (long)p.nx * p.ny;
-    T ax = 0, ay = 0, az = 0, bx = 0, by = 0, bz = 0, cx = 0, cy = 0, cz = 0;
-    if (x < p.nx - 1) acc(i + sx, (T)1, ax, ay, az);
-    if (x > 0) acc(i - sx, (T)-1, ax, ay, az);
-    if (y < p.ny - 1) acc(i + sy, (T)1, bx, by, bz);
-    if (y > 0) acc(i - sy, (T)-1, bx, by, bz);
-    if (p.dmi == 2) {
-        if (z < p.nz - 1) acc(i + sz, (T)1, cx, cy, cz);
-        if (z > 0) acc(i - sz, (T)-1, cx, cy, cz);
+    // per axis: the neighbour above minus the neighbour below, present ones only
+    const Bonds<T> q = bonds_of(p, i, x, y, z);
+    const int nb = p.dmi == 2 && p.nz > 1 ? 6 : 4;
+    V3<T> v[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+        if (k < nb) v[k] = load3(m, q.j[k], p.N);
+    T d[3][3] = {};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        if (2 * k < nb && q.on[2 * k + 1]) {
+            d[k][0] += v[2 * k + 1].x;
+            d[k][1] += v[2 * k + 1].y;
+            d[k][2] += v[2 * k + 1].z;
+        }
+        if (2 * k < nb && q.on[2 * k]) {
+            d[k][0] -= v[2 * k].x;
+            d[k][1] -= v[2 * k].y;
+            d[k][2] -= v[2 * k].z;
+        }
     }
+    const T ax = d[0][0], ay = d[0][1], az = d[0][2], bx = d[1][0], by = d[1][1], bz = d[1][2], cx = d[2][0],
+            cy = d[2][1];
     if (p.dmi == 1) {
         // e_y x a (x axis) and -e_x x b (y axis)
         hx = p.dx_c * az;
