@@ -135,6 +135,7 @@ int make_tables(mm_ctx* ctx) {
     twiddles(ctx->Pz, t);
     ctx->tw.off_z4 = (long)t.size() / 2;
     four_step_table(ctx->Pz, true, t);
+    ctx->tw.len = (long)t.size() / 2;
     MM_CUDA_CHECK(ctx, cudaMalloc(&ctx->tw.f64, t.size() * sizeof(double)));
     MM_CUDA_CHECK(ctx, cudaMemcpy(ctx->tw.f64, t.data(), t.size() * sizeof(double), cudaMemcpyHostToDevice));
     if (ctx->prec == MM_F32) {

@@ -36,6 +36,8 @@ namespace mm {
 
 // mm_zline.cu: the FP32 z pass of long z lines (Pz >= 64)
 int zline_f32(mm_ctx* ctx, float2* buf, const float* kern, const float2* tw);
+bool zline_ff_takes(int Pz);
+int zline_ff(mm_ctx* ctx, ffc* buf, const ff* kern, const ffc* tw);
 
 namespace {
 
@@ -1858,7 +1860,10 @@ int apply_ff(mm_ctx* ctx, const double* m, double* H, bool unit) {
         if ((rc = run_cols<ff, -1>(ctx, A, Bf, ctx->Py, ctx->ny, ctx->Py, 3 * ctx->nz, g, tw + ctx->tw.off_py)))
             return rc;
     }
-    {   // K4
+    // K4
+    if (zline_ff_takes(ctx->Pz)) {
+        if ((rc = zline_ff(ctx, Bf, (const ff*)ctx->kern_ff, tw + ctx->tw.off_z4))) return rc;
+    } else {
         KernelTimer kt(ctx, MM_K_ZCONV);
         const int Pz = ctx->Pz;
         const int B = z_tile(Pz, sizeof(C));
@@ -1948,7 +1953,7 @@ int demag_prepare_ff(mm_ctx* ctx) {
     if (plane_ff_fits(ctx)) return plane_prepare_ff(ctx);
     if (ctx->kern_ff && ctx->tw.ff) return MM_OK;
     const long nk = 6L * ctx->Pz2 * ctx->Py2 * ctx->Hs;
-    const long nt = 2L * (ctx->tw.off_pz + ctx->Pz);          // doubles in the twiddle table
+    const long nt = 2L * ctx->tw.len;                         // doubles in the twiddle table
     if (!ctx->kern_ff) MM_CUDA_CHECK(ctx, cudaMalloc(&ctx->kern_ff, nk * sizeof(ff)));
     if (!ctx->tw.ff) MM_CUDA_CHECK(ctx, cudaMalloc(&ctx->tw.ff, nt * sizeof(ff)));
     k_split_ff<<<(unsigned)((nk + 255) / 256), 256, 0, ctx->stream>>>((const double*)ctx->kern, (ff*)ctx->kern_ff, nk);

@@ -64,6 +64,7 @@ struct Tables {
     void* ff = nullptr;    // float-float copy of f64 (MM_FFT_FF on an MM_F64 context)
     long off_lx = 0, off_px = 0, off_py = 0, off_pz = 0;
     long off_z4 = 0;       // four-step tables of Pz (mm_zline.cu)
+    long len = 0;          // complex values in all
 };
 
 // Bluestein (chirp-z) data of one padded axis whose length P is not a power

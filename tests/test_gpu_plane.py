@@ -99,6 +99,20 @@ def test_float_float_planes_match_oracle(n):
     mm.mm_destroy(ctx)
 
 
+# float-float z lines in registers (Pz = 16, 32, 64) and the Stockham pass
+# beyond; column tiles that are not full, ny = 1
+@pytest.mark.parametrize("n", [(16, 8, 8), (64, 4, 16), (8, 16, 32), (32, 1, 16), (4, 2, 64), (2, 4, 8)],
+                         ids=lambda n: "x".join(map(str, n)))
+def test_float_float_z_lines_match_oracle(n):
+    m = wl.random_unit(n, seed=sum(n))
+    ctx = context(n, "ff")
+    md = dev(m, "ff")
+    H = torch.full_like(md, float("nan"))
+    mm.mm_demag_field(ctx, md, H)
+    assert rel(H, micromag.Problem(n, D).demag_fft(m)) < TOL["ff"]
+    mm.mm_destroy(ctx)
+
+
 @pytest.mark.parametrize("prec", ["f64", "ff", "f32"])
 @pytest.mark.parametrize("n", [(32, 16, 2), (30, 21, 4), (19, 12, 16)], ids=lambda n: "x".join(map(str, n)))
 def test_cell_wise_ms_and_the_unit_operator(n, prec):
