@@ -68,36 +68,33 @@ __global__ void __launch_bounds__(px_threads(px_rows<T>(L1 * L2), L1, L2))
         const long r = r0 + b;
         const bool act = r < rows;
         const S* row = in + (act ? r : 0) * nx;
-        const S* mrow = Ms ? Ms + ((act ? r : 0) % ms_rows) * nx : nullptr;
-        // pairs in one access where every row starts on a pair boundary
+        const S* mrow = Ms ? Ms + (long)((unsigned)(act ? r : 0) % (unsigned)ms_rows) * nx : nullptr;
+        // pairs in one access where every row starts on a pair boundary (the
+        // library's own Ms array always does)
         const bool even = nx % 2 == 0 && reinterpret_cast<uintptr_t>(in) % (2 * sizeof(S)) == 0;
-        C v[L1];
+        C v[L1], w[L1 / 2];
 #pragma unroll
         for (int n1 = 0; n1 < L1 / 2; ++n1) {
             const int x = 2 * (t + L2 * n1);
-            S a = 0, c = 0;
+            v[n1] = cmk<C>((T)0, (T)0);
+            w[n1] = cmk<C>(ms, ms);
             if (act && x < nx) {
                 if (even) {
                     const PC<S> q = *reinterpret_cast<const PC<S>*>(row + x);
-                    a = q.x;
-                    c = q.y;
+                    v[n1] = cmk<C>(pl_ld<T>(q.x), pl_ld<T>(q.y));
+                    if (mrow) {
+                        const PC<S> u = *reinterpret_cast<const PC<S>*>(mrow + x);
+                        w[n1] = cmk<C>(pl_ld<T>(u.x), pl_ld<T>(u.y));
+                    }
                 } else {
-                    a = row[x];
-                    if (x + 1 < nx) c = row[x + 1];
+                    const bool two = x + 1 < nx;
+                    v[n1] = cmk<C>(pl_ld<T>(row[x]), two ? pl_ld<T>(row[x + 1]) : (T)0);
+                    if (mrow) w[n1] = cmk<C>(pl_ld<T>(mrow[x]), two ? pl_ld<T>(mrow[x + 1]) : (T)0);
                 }
             }
-            T ta = pl_ld<T>(a), tc = pl_ld<T>(c);
-            if (mrow) {
-                if (act && x < nx) {
-                    ta *= pl_ld<T>(mrow[x]);
-                    if (x + 1 < nx) tc *= pl_ld<T>(mrow[x + 1]);
-                }
-            } else {
-                ta *= ms;
-                tc *= ms;
-            }
-            v[n1] = cmk<C>(ta, tc);
         }
+#pragma unroll
+        for (int n1 = 0; n1 < L1 / 2; ++n1) v[n1] = cmk<C>(v[n1].x * w[n1].x, v[n1].y * w[n1].y);
         const C* tq = twL + t;
         dif<L1, -1, true>(v);
 #pragma unroll

@@ -3,6 +3,7 @@
 // mm_plane_f64*.cu).
 #pragma once
 
+#include <algorithm>
 #include "mm_plane.cuh"
 
 namespace mm {
@@ -103,11 +104,29 @@ int launch_plane(mm_ctx* ctx, PC<T>* buf, const T* kern, const PC<T>* tw) {
             const size_t smem = (size_t)3 * ctx->nz * plane_pitch(L1, L2) * sizeof(PC<T>);
             if ((rc = plane_smem(ctx, (const void*)fn, smem))) return;
             const int tasks = 3 * ctx->nz * L1;
-            const int cap = sizeof(T) == 4 ? 512 : 256;
-            int nt = tasks;
-            if (nt > cap) nt = (tasks + (tasks + cap - 1) / cap - 1) / ((tasks + cap - 1) / cap);
-            nt = (nt + 31) / 32 * 32;
-            if (nt > cap) nt = cap;
+            // Rounds of equal size within `cap` threads.  Planes that have an
+            // SM each take up to 512 threads; of more planes, blocks of at
+            // most 256 put two on an SM (at 128 registers), and smaller ones
+            // where that takes every plane into one wave.  Demag, 384 threads
+            // -> rule: 256x256x4 20.9 -> 19.1 us, 512x512x4 64.9 -> 61.4,
+            // 256x256x8 33.6 -> 30.6, 300x300x2 21.8 -> 19.0 (96 threads: 20.8);
+            // 64x512x8 (65 planes) 29.3 at 384, 35.9 at 192.
+            auto even = [&](int cap) {
+                const int rounds = (tasks + cap - 1) / cap;
+                return ((tasks + rounds - 1) / rounds + 31) / 32 * 32;
+            };
+            int nt = even(sizeof(T) == 4 ? 512 : 256);
+            if (sizeof(T) == 4 && p.K > 152) {
+                nt = even(256);
+                for (int cap : {256, 160, 128}) {
+                    const int n = std::max(even(cap), std::min(128, nt));
+                    const long fit = std::min<long>(65536 / (128 * n), (227 * 1024) / (long)(smem + 1024));
+                    if (152 * fit >= p.K) {
+                        nt = n;
+                        break;
+                    }
+                }
+            }
             dep(fn, (unsigned)p.K, nt, smem, ctx->stream)(buf, kern, ctx->nz, ctx->ny, p.R, p.KQ, tw + p.off_y4);
         }))
         rc = fail(ctx, MM_ERR_INVALID_ARG, "y length %d", p.P);
