@@ -39,31 +39,33 @@ __device__ __forceinline__ void block_sum_atomic(double v, double* target) {
     }
 }
 
-// Block reductions of per-thread values of the path's type T: the warp
-// stage runs in T (FP32 adds for FP32 contexts: GB300's FP64 rate is far
-// lower), the eight warp results are combined in double by warp 0, then one
-// atomic per block.  Must be called by every thread of the block.
+// Block sum of per-thread values of the path's type T: the warp stage runs in
+// T (FP32 adds for FP32 contexts: GB300's FP64 rate is far lower), thread 0
+// adds the few warp results in double.  Must be called by every thread.
 template <typename T>
-__device__ __forceinline__ double block_reduce_t(T v, bool is_max) {
+__device__ __forceinline__ double block_sum_t(T v) {
     __shared__ double red[32];
-    for (int o = 16; o > 0; o >>= 1) {
-        const T u = __shfl_xor_sync(0xffffffffu, v, o);
-        v = is_max ? (u > v ? u : v) : v + u;
-    }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     __syncthreads();
-    if (lane == 0) red[w] = (double)v;
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = (double)v;
     __syncthreads();
     double r = 0.0;
-    if (w == 0) {
-        const int nw = (blockDim.x + 31) >> 5;
-        r = lane < nw ? red[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) {
-            const double u = __shfl_xor_sync(0xffffffffu, r, o);
-            r = is_max ? fmax(r, u) : r + u;
-        }
+    if (threadIdx.x == 0) {
+        r = red[0];
+        for (int w = 1; w < (int)((blockDim.x + 31) >> 5); ++w) r += red[w];
     }
     return r;   // valid in thread 0
+}
+// Block maximum of a non-negative value, through the bit patterns
+template <typename T>
+__device__ __forceinline__ double block_max_t(T v) {
+    __shared__ unsigned long long red[32];
+    unsigned long long u = warp_max_bits((unsigned long long)__double_as_longlong((double)v));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = u;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < (int)((blockDim.x + 31) >> 5); ++w) u = red[w] > u ? red[w] : u;
+    return __longlong_as_double((long long)u);   // valid in thread 0
 }
 
 // ------------------------------------------------------------- fields
@@ -759,19 +761,19 @@ __global__ void k_bb_grad(Params<T> p, const T* __restrict__ m, const T* __restr
         store3(g, i, p.N, gi);
     }
     // the torque maximum as the maximum squared norm, one square root per block
-    const double t2 = block_reduce_t<T>(tq2, true);
+    const double t2 = block_max_t<T>(tq2);
     if (threadIdx.x == 0 && t2 > 0.0) {
         const double tq = t2 >= (sizeof(T) == 4 ? 3.0e38 : 1e300) ? 1e300 : sqrt(t2);
         atomicMax(&ctl->torque_bits, (unsigned long long)__double_as_longlong(tq));
     }
     if (have_prev) {
-        const double a0 = block_reduce_t<T>(ss, false);
+        const double a0 = block_sum_t<T>(ss);
         if (threadIdx.x == 0) atomicAdd(&ctl->bb[0], a0);
         // s.y is a difference-like sum (the BB quotients divide by it and
         // read its sign), so its warp stage runs in double even in FP32
-        const double a1 = block_reduce_t<double>((double)sy, false);
+        const double a1 = block_sum_t<double>((double)sy);
         if (threadIdx.x == 0) atomicAdd(&ctl->bb[1], a1);
-        const double a2 = block_reduce_t<T>(yy, false);
+        const double a2 = block_sum_t<T>(yy);
         if (threadIdx.x == 0) atomicAdd(&ctl->bb[2], a2);
     }
 }
@@ -812,7 +814,10 @@ __global__ void k_bb_update(Params<T> p, T* __restrict__ m, const T* __restrict_
     const V3<T> gi = load3(g, i, p.N);
     V3<T> mn = {mi.x - tau * gi.x, mi.y - tau * gi.y, mi.z - tau * gi.z};
     const T nrm = sqrt(mn.x * mn.x + mn.y * mn.y + mn.z * mn.z);
-    if (nrm > (T)0) mn = {mn.x / nrm, mn.y / nrm, mn.z / nrm};
+    if (nrm > (T)0) {
+        const T inv = (T)1 / nrm;       // one FP64 division of about 25 instructions, not three
+        mn = {mn.x * inv, mn.y * inv, mn.z * inv};
+    }
     store3(m, i, p.N, mn);
 }
 

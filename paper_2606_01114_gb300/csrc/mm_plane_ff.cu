@@ -182,7 +182,9 @@ int plane_apply_ff(mm_ctx* ctx, const double* m, const double* Ms, double ms, do
     const ffc* tw = (const ffc*)p.tw_ff;
     ffc* buf = (ffc*)p.buf;
     const int lgL = ilog2(p.L);
-    const int lgB = lgL >= 6 ? 2 : 3;                      // 64-byte segments per plane; 8 rows of short lines
+    // 64-byte segments per plane (8 rows of short lines); 32-byte ones while the
+    // larger blocks are too few to share the SMs evenly (256x256x1: 192 blocks)
+    const int lgB = lgL < 6 ? 3 : rows < 16 * 152 ? 1 : 2;
     const int nt = ((1 << (lgL + lgB - 3)) + 31) / 32 * 32;
     const size_t smem = sizeof(ffc) << (lgL + lgB);
     const unsigned nb = (unsigned)((rows + (1 << lgB) - 1) >> lgB);
