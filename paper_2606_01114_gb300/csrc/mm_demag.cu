@@ -329,7 +329,9 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512)
 }
 
 // ------------------------------------------------ direct DFT passes
-// Transform lengths that are not powers of two (meshes such as 100 x 25)
+// Transform lengths that are not powers of two in the [c][z][y][kx] passes
+// (nx = 1 or ny = 1, the fft modes and the k-space product of such meshes; their
+// plain field runs in the plane layout, mm_plane.cuh)
 // take these O(L^2)-per-line kernels: every output is the plain sum of its
 // DFT definition, one thread per output, twiddles from the length's table
 // (index (n k) mod L, advanced additively).  A correctness path beside the
@@ -337,7 +339,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512)
 inline bool pow2(int n) { return n > 0 && (n & (n - 1)) == 0; }
 
 // Bluestein (chirp-z) passes for padded lengths P that are not powers of two
-// (meshes such as 100 x 25 or 350^3): with nk = (n^2 + k^2 - (k - n)^2) / 2,
+// of the same passes: with nk = (n^2 + k^2 - (k - n)^2) / 2,
 //   X[k] = sum_{n < nin} x[n] w^{nk} = a[k] sum_n (x[n] a[n]) b[k - n],
 // w = exp(DIR 2 pi i / P), a[n] = exp(DIR i pi n^2 / P), b = conj(a): a
 // linear convolution, done as a circular one of length M (the power of two
