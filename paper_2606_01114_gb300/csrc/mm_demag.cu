@@ -1290,13 +1290,6 @@ template <typename T> const C_t<T>* table(const mm_ctx* ctx, long off);
 template <> const double2* table<double>(const mm_ctx* ctx, long off) { return (const double2*)ctx->tw.f64 + off; }
 template <> const float2* table<float>(const mm_ctx* ctx, long off) { return (const float2*)ctx->tw.f32 + off; }
 
-int set_smem(mm_ctx* ctx, const void* fn, size_t bytes) {
-    if (bytes > 48 * 1024) {
-        MM_CUDA_CHECK(ctx, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    }
-    return MM_OK;
-}
-
 template <int L1, int L2>
 int launch_xfwd_reg(mm_ctx* ctx, const float* in, const float* Ms, float ms, long ms_rows, float2* out, long rows,
                     const float2* twL, const float2* twP) {
@@ -1304,14 +1297,14 @@ int launch_xfwd_reg(mm_ctx* ctx, const float* in, const float* Ms, float ms, lon
     const size_t smem = (size_t)B * L1 * L2 * sizeof(float2);
     if constexpr (L1 == 32 && L2 == 16) {
         // level 1 split by output parity over all 128 threads: 39.0 -> 33.4 us on the 512 x 512 x 16 film
-        int rc = set_smem(ctx, (const void*)k_xfwd_reg<L1, L2, true>, smem);
+        int rc = smem_opt_in(ctx, (const void*)k_xfwd_reg<L1, L2, true>, smem);
         if (rc) return rc;
         dep(k_xfwd_reg<L1, L2, true>, (unsigned)((rows + B - 1) / B), B * L1, smem, ctx->stream)(
             in, Ms, ms, ms_rows, out, ctx->Hs, rows, twL, twP);
         MM_LAUNCH_CHECK(ctx);
         return MM_OK;
     }
-    int rc = set_smem(ctx, (const void*)k_xfwd_reg<L1, L2>, smem);
+    int rc = smem_opt_in(ctx, (const void*)k_xfwd_reg<L1, L2>, smem);
     if (rc) return rc;
     dep(k_xfwd_reg<L1, L2>, (unsigned)((rows + B - 1) / B), B * L1, smem, ctx->stream)(in, Ms, ms, ms_rows, out,
                                                                                    ctx->Hs, rows, twL, twP);
@@ -1343,14 +1336,14 @@ int launch_xinv_reg(mm_ctx* ctx, const float2* in, float* out, long rows, float 
     const size_t smem = (size_t)B * L1 * L2 * sizeof(float2);
     if constexpr (L1 * L2 == 512) {
         // 16 x 32 with the packing folded into the level-1 loads: 53.3 -> 35.5 us on the 512 x 512 x 16 film
-        int rc = set_smem(ctx, (const void*)k_xinv_pk<16, 32>, smem);
+        int rc = smem_opt_in(ctx, (const void*)k_xinv_pk<16, 32>, smem);
         if (rc) return rc;
         dep(k_xinv_pk<16, 32>, (unsigned)((rows + B - 1) / B), 128, smem, ctx->stream)(in, ctx->Hs, out, rows, scale,
                                                                                      twL, twP);
         MM_LAUNCH_CHECK(ctx);
         return MM_OK;
     }
-    int rc = set_smem(ctx, (const void*)k_xinv_reg<L1, L2>, smem);
+    int rc = smem_opt_in(ctx, (const void*)k_xinv_reg<L1, L2>, smem);
     if (rc) return rc;
     dep(k_xinv_reg<L1, L2>, (unsigned)((rows + B - 1) / B), B * L1, smem, ctx->stream)(in, ctx->Hs, out, rows, scale,
                                                                                    twL, twP);
@@ -1399,7 +1392,7 @@ int run_xfwd(mm_ctx* ctx, const T* in, long in_ld, int nin, const T* Ms, T ms, l
         const BlueArrays<T> ba = blue_arrays<T>(ctx->blue_x);
         const int M = ctx->blue_x.M, B = blue_lines(M, sizeof(C_t<T>));
         const size_t smem = (size_t)B * M * sizeof(C_t<T>);
-        int rc = set_smem(ctx, (const void*)k_xfwd_blue<T>, smem);
+        int rc = smem_opt_in(ctx, (const void*)k_xfwd_blue<T>, smem);
         if (rc) return rc;
         k_xfwd_blue<T><<<(unsigned)((rows + B - 1) / B), block_threads(B * M / 8), smem, ctx->stream>>>(
             in, in_ld, nin, Ms, ms, ms_rows, out, ctx->Hs, ctx->Hx, rows, ilog2(M), ilog2(B), ba.chirp, ba.filt, ba.tw);
@@ -1431,7 +1424,7 @@ int run_xfwd(mm_ctx* ctx, const T* in, long in_ld, int nin, const T* Ms, T ms, l
     const int B = x_rows_per_block(L);
     size_t smem = (size_t)L * B * sizeof(C_t<T>);
     auto fn = nin <= L ? k_xfwd<T, T, true> : k_xfwd<T, T, false>;
-    int rc = set_smem(ctx, (const void*)fn, smem);
+    int rc = smem_opt_in(ctx, (const void*)fn, smem);
     if (rc) return rc;
     dep(fn, (unsigned)((rows + B - 1) / B), block_threads(B * L / 8), smem, ctx->stream)(
         in, in_ld, nin, Ms, ms, ms_rows, out, ctx->Hs, ilog2(L), rows, ilog2(B), twL, twP);
@@ -1448,7 +1441,7 @@ int launch_cols_reg(mm_ctx* ctx, const float2* in, float2* out, int nplanes, Col
     constexpr int B = 8;   // 64-byte row segments: 15 % faster than 4 columns at L = 1024
     const size_t smem = (size_t)L * B * sizeof(float2);
     auto fn = k_cols_reg<L1, L2, DIR, (DIR < 0), (DIR > 0)>;
-    int rc = set_smem(ctx, (const void*)fn, smem);
+    int rc = smem_opt_in(ctx, (const void*)fn, smem);
     if (rc) return rc;
     dim3 grid((unsigned)((c1 - c0 + B - 1) / B), (unsigned)nplanes);
     dep(fn, grid, B * (L1 > L2 ? L1 : L2), smem, ctx->stream)(in, out, c0, c1, 3, g, tw);
@@ -1564,7 +1557,7 @@ int run_cols(mm_ctx* ctx, const C_t<T>* in, C_t<T>* out, int L, int nin, int nou
         const BlueArrays<T> ba = blue_arrays<T>(ctx->blue_y);
         const int M = ctx->blue_y.M, B = blue_lines(M, sizeof(C_t<T>));
         const size_t smem = (size_t)B * M * sizeof(C_t<T>);
-        int rc = set_smem(ctx, (const void*)k_cols_blue<T, DIR>, smem);
+        int rc = smem_opt_in(ctx, (const void*)k_cols_blue<T, DIR>, smem);
         if (rc) return rc;
         dim3 grid((unsigned)((ctx->Hx + B - 1) / B), (unsigned)nplanes);
         k_cols_blue<T, DIR><<<grid, block_threads(B * M / 8), smem, ctx->stream>>>(
@@ -1596,7 +1589,7 @@ int run_cols(mm_ctx* ctx, const C_t<T>* in, C_t<T>* out, int L, int nin, int nou
     const bool hin = 2 * nin <= L, hout = 2 * nout <= L;
     auto fn = hin ? (hout ? k_cols<T, DIR, true, true> : k_cols<T, DIR, true, false>)
                   : (hout ? k_cols<T, DIR, false, true> : k_cols<T, DIR, false, false>);
-    int rc = set_smem(ctx, (const void*)fn, smem);
+    int rc = smem_opt_in(ctx, (const void*)fn, smem);
     if (rc) return rc;
     dim3 grid((unsigned)((ctx->Hx + B - 1) / B), (unsigned)nplanes);
     dep(fn, grid, block_threads(B * L / 8), smem, ctx->stream)(in, out, ilog2(L), nin, nout, ctx->Hx,
@@ -1610,7 +1603,7 @@ int launch_zconv_reg_t(mm_ctx* ctx, float2* buf, const float* kern, int c0, int 
     constexpr int PZ2 = PZ / 2 + 1;
     const size_t smem = (size_t)3 * PZ * kZB * sizeof(float2) + (size_t)6 * PZ2 * kZB * sizeof(float);
     if (c0 % 4) return fail(ctx, MM_ERR_INVALID_ARG, "z pass: first column %d not a multiple of 4", c0);
-    int rc = set_smem(ctx, (const void*)k_zconv_reg<PZ>, smem);
+    int rc = smem_opt_in(ctx, (const void*)k_zconv_reg<PZ>, smem);
     if (rc) return rc;
     dim3 grid((unsigned)((c1 - c0 + kZB - 1) / kZB), (unsigned)ctx->Py);
     dep(k_zconv_reg<PZ>, grid, 3 * kZB, smem, ctx->stream)(buf, kern, ctx->Py, ctx->Hs, c0, c1, ctx->Py2);
@@ -1674,7 +1667,7 @@ int apply(mm_ctx* ctx, const T* m, T* H, bool unit = false) {
         const int Pz = ctx->Pz;
         const int B = z_tile(Pz, sizeof(C));
         size_t smem = (size_t)3 * Pz * B * sizeof(C) + (size_t)6 * ctx->Pz2 * B * sizeof(T);
-        rc = set_smem(ctx, (const void*)k_zconv<T>, smem);
+        rc = smem_opt_in(ctx, (const void*)k_zconv<T>, smem);
         if (rc) return rc;
         dim3 grid((unsigned)((ctx->Hx + B - 1) / B), (unsigned)(ctx->Py / 2 + 1));
         dep(k_zconv<T>, grid, block_threads(3 * B * Pz / 8), smem, ctx->stream)(
@@ -1703,7 +1696,7 @@ int xinv_pass(mm_ctx* ctx, const C_t<T>* xin, T* H, long rows) {
         const BlueArrays<T> ba = blue_arrays<T>(ctx->blue_x);
         const int M = ctx->blue_x.M, B = blue_lines(M, sizeof(C));
         const size_t smem = (size_t)B * M * sizeof(C);
-        rc = set_smem(ctx, (const void*)k_xinv_blue<T>, smem);
+        rc = smem_opt_in(ctx, (const void*)k_xinv_blue<T>, smem);
         if (rc) return rc;
         k_xinv_blue<T><<<(unsigned)((rows + B - 1) / B), block_threads(B * M / 8), smem, ctx->stream>>>(
             xin, ctx->Hs, H, ctx->nx, rows, scale, ilog2(M), ilog2(B), ba.chirp, ba.filt, ba.tw);
@@ -1746,7 +1739,7 @@ int xinv_pass(mm_ctx* ctx, const C_t<T>* xin, T* H, long rows) {
         }
         const int B = x_rows_per_block(L);
         size_t smem = (size_t)L * B * sizeof(C);
-        rc = set_smem(ctx, (const void*)k_xinv<T>, smem);
+        rc = smem_opt_in(ctx, (const void*)k_xinv<T>, smem);
         if (rc) return rc;
         dep(k_xinv<T>, (unsigned)((rows + B - 1) / B), block_threads(B * L / 8), smem, ctx->stream)(
             xin, ctx->Hs, H, ctx->nx, ilog2(L), rows, ilog2(B), scale, table<T>(ctx, ctx->tw.off_lx),
@@ -1849,7 +1842,7 @@ int apply_ff(mm_ctx* ctx, const double* m, double* H, bool unit) {
             const int B = x_rows_per_block(L);
             const size_t smem = (size_t)L * B * sizeof(C);
             // nin = nx = L: the upper half of each packed line is zero padding
-            if ((rc = set_smem(ctx, (const void*)k_xfwd<ff, double, true>, smem))) return rc;
+            if ((rc = smem_opt_in(ctx, (const void*)k_xfwd<ff, double, true>, smem))) return rc;
             dep(k_xfwd<ff, double, true>, (unsigned)((rows + B - 1) / B), block_threads(B * L / 8), smem, ctx->stream)(
                 m, ctx->nx, ctx->nx, Ms, ms, ms_rows, xout, ctx->Hs, ilog2(L), rows, ilog2(B), tw + ctx->tw.off_lx,
                 tw + ctx->tw.off_px);
@@ -1870,7 +1863,7 @@ int apply_ff(mm_ctx* ctx, const double* m, double* H, bool unit) {
         const int Pz = ctx->Pz;
         const int B = z_tile(Pz, sizeof(C));
         const size_t smem = (size_t)3 * Pz * B * sizeof(C) + (size_t)6 * ctx->Pz2 * B * sizeof(ff);
-        if ((rc = set_smem(ctx, (const void*)k_zconv<ff>, smem))) return rc;
+        if ((rc = smem_opt_in(ctx, (const void*)k_zconv<ff>, smem))) return rc;
         dim3 grid((unsigned)((ctx->Hx + B - 1) / B), (unsigned)(ctx->Py / 2 + 1));
         dep(k_zconv<ff>, grid, block_threads(3 * B * Pz / 8), smem, ctx->stream)(
             Bf, (const ff*)ctx->kern_ff, ctx->nz, ilog2(Pz), ctx->Py, ctx->Hs, ctx->Hx, ctx->Py2, ctx->Pz2, ilog2(B),
@@ -1893,7 +1886,7 @@ int apply_ff(mm_ctx* ctx, const double* m, double* H, bool unit) {
             const int L = ctx->Lx;
             const int B = x_rows_per_block(L);
             const size_t smem = (size_t)L * B * sizeof(C);
-            if ((rc = set_smem(ctx, (const void*)k_xinv<ff, double>, smem))) return rc;
+            if ((rc = smem_opt_in(ctx, (const void*)k_xinv<ff, double>, smem))) return rc;
             dep(k_xinv<ff, double>, (unsigned)((rows + B - 1) / B), block_threads(B * L / 8), smem, ctx->stream)(
                 xin, ctx->Hs, H, ctx->nx, ilog2(L), rows, ilog2(B), scale, tw + ctx->tw.off_lx, tw + ctx->tw.off_px);
         }

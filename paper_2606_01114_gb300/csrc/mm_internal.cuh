@@ -254,6 +254,19 @@ __device__ __forceinline__ void dep_wait() {
 }
 #endif
 
+// Opts a kernel in to dynamic shared memory above 48 KB.  The limit belongs to
+// the kernel, for the whole process, and one kernel serves contexts of
+// different sizes in different host threads: every call sets the same value
+// (226 KB: a block's 227 KB less what these kernels declare statically), so no
+// thread lowers a limit between another one's call and its launch.
+constexpr size_t kSmemOptIn = 226 * 1024;
+inline int smem_opt_in(mm_ctx* ctx, const void* fn, size_t bytes) {
+    if (bytes <= 48 * 1024) return MM_OK;
+    if (bytes > kSmemOptIn) return fail(ctx, MM_ERR_CUDA, "%zu bytes of shared memory per block", bytes);
+    MM_CUDA_CHECK(ctx, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemOptIn));
+    return MM_OK;
+}
+
 // Brackets the launches in its scope with CUDA events when timing is on.
 struct KernelTimer {
     mm_ctx* ctx;

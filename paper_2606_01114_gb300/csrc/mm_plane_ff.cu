@@ -158,9 +158,8 @@ int launch_ff_plane(mm_ctx* ctx, ffc* buf, const ffc* tw) {
     const PlanePlan& p = ctx->plane;
     KernelTimer kt(ctx, MM_K_ZCONV);
     const size_t smem = (size_t)3 * NZ * p.P * sizeof(ffc);
-    if (smem > 48 * 1024)
-        MM_CUDA_CHECK(ctx, cudaFuncSetAttribute((const void*)k_ff_plane<NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)smem));
+    int rc = smem_opt_in(ctx, (const void*)k_ff_plane<NZ>, smem);
+    if (rc) return rc;
     const int nt = (3 * NZ * p.P / 8 + 31) / 32 * 32;     // the Stockham stages need 3 nz P / 8 threads
     dep(k_ff_plane<NZ>, (unsigned)p.K, nt, smem, ctx->stream)(buf, (const ff*)p.kern_ff, ctx->ny, p.R, p.KQ, ilog2(p.P),
                                                              tw + p.off_y);

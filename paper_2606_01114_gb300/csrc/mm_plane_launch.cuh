@@ -39,12 +39,6 @@ template <typename F> bool with_length(int len, F&& f) {
     return false;
 }
 
-inline int plane_smem(mm_ctx* ctx, const void* fn, size_t bytes) {
-    if (bytes > 48 * 1024)
-        MM_CUDA_CHECK(ctx, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    return MM_OK;
-}
-
 // complex stride of a line of length P in the plane kernel's shared memory
 inline int plane_line(int P) {
     int lp = 0;
@@ -102,7 +96,7 @@ int launch_plane(mm_ctx* ctx, PC<T>* buf, const T* kern, const PC<T>* tw) {
             const bool fused = CANF && ctx->nz == 1;
             auto fn = fused ? k_plane<T, L1, L2, CANF> : k_plane<T, L1, L2, false>;
             const size_t smem = (size_t)3 * ctx->nz * plane_pitch(L1, L2) * sizeof(PC<T>);
-            if ((rc = plane_smem(ctx, (const void*)fn, smem))) return;
+            if ((rc = smem_opt_in(ctx, (const void*)fn, smem))) return;
             const int tasks = 3 * ctx->nz * L1;
             // Rounds of equal size within `cap` threads.  Planes that have an
             // SM each take up to 512 threads; of more planes, blocks of at
@@ -146,7 +140,7 @@ int launch_py(mm_ctx* ctx, const PC<T>* in, PC<T>* out, const PC<T>* tw) {
             constexpr int L1 = decltype(A)::value, L2 = decltype(B)::value;
             auto fn = k_py<T, L1, L2, DIR>;
             const size_t smem = (size_t)kPyLines * plane_pitch(L1, L2) * sizeof(PC<T>);
-            if ((rc = plane_smem(ctx, (const void*)fn, smem))) return;
+            if ((rc = smem_opt_in(ctx, (const void*)fn, smem))) return;
             dep(fn, (unsigned)((nlines + kPyLines - 1) / kPyLines), (kPyLines * (L1 > L2 ? L1 : L2) + 31) / 32 * 32, smem, ctx->stream)(in, out, lines, nlines, ctx->ny, DIR < 0 ? p.R : wide, DIR < 0 ? wide : p.R,
                                                       tw + p.off_y4);
         }))
@@ -187,7 +181,7 @@ int launch_zline_t(mm_ctx* ctx, PC<T>* buf, const T* kern, const ZLine& g, int n
     constexpr int MINB = sizeof(T) == 8 ? 1 : PZ <= 32 ? 4 : PZ == 64 ? 4 : PZ == 128 ? 3 : PZ == 256 ? 2 : 1;
     auto fn = k_zline<T, L1, L2, COLY, B, NT, MINB>;
     const size_t smem = zline_smem<T, L1, L2, B>();
-    int rc = plane_smem(ctx, (const void*)fn, smem);
+    int rc = smem_opt_in(ctx, (const void*)fn, smem);
     if (rc) return rc;
     dim3 grid((unsigned)((g.ncol + B - 1) / B), (unsigned)nrows);
     dep(fn, grid, NT, smem, ctx->stream)(buf, kern, g, tw);

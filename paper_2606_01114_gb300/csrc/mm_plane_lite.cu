@@ -255,7 +255,7 @@ int lite_plane(mm_ctx* ctx) {
     const PlanePlan& p = ctx->plane;
     const double2* tw = (const double2*)p.tw;
     const size_t smem = (size_t)7 * p.P * sizeof(double2) + (size_t)6 * p.KQ * sizeof(double);
-    int rc = plane_smem(ctx, (const void*)k_lplane, smem);
+    int rc = smem_opt_in(ctx, (const void*)k_lplane, smem);
     if (rc) return rc;
     const int tasks = 3 * p.P;
     const int nt = tasks >= 256 ? 256 : (tasks + 31) / 32 * 32;

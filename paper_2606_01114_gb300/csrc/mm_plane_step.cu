@@ -32,7 +32,7 @@ int launch_px_cell(mm_ctx* ctx, const float* m_in, float* H, const RkStage<float
                 const int nt = width > 256 ? (width + 31) / 32 * 32 : 256;
                 const size_t smem = (size_t)lines * (plane_pitch(L1, L2) + 4) * sizeof(float2);
                 auto fn = k_px_cell<float, L1, L2, STAGE>;
-                if ((rc = plane_smem(ctx, (const void*)fn, smem))) return;
+                if ((rc = smem_opt_in(ctx, (const void*)fn, smem))) return;
                 dep(fn, (unsigned)((nrows + (1 << lgB) - 1) >> lgB), nt, smem, ctx->stream)(
                     (float2*)p.buf, p.R, par, folded, lgB, scale, tw + p.off_x4, tw + p.off_p, m_in, H, g, ctx->ctl);
             }

@@ -19,7 +19,7 @@ int zline_ff_t(mm_ctx* ctx, ffc* buf, const ff* kern, const ZLine& g, const ffc*
     KernelTimer kt(ctx, MM_K_ZCONV);
     auto fn = k_zline<ff, L1, L2, false, B, NT, MINB>;
     const size_t smem = zline_smem<ff, L1, L2, B>();
-    int rc = plane_smem(ctx, (const void*)fn, smem);
+    int rc = smem_opt_in(ctx, (const void*)fn, smem);
     if (rc) return rc;
     dim3 grid((unsigned)((g.ncol + B - 1) / B), (unsigned)ctx->Py);
     dep(fn, grid, NT, smem, ctx->stream)(buf, kern, g, tw);
