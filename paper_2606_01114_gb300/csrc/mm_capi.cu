@@ -338,8 +338,9 @@ int mm_init_mesh(mm_ctx** out, int nx, int ny, int nz, double dx, double dy, dou
         reset_ctl(ctx->ctl_host, 0.0, 1e-14, std::numeric_limits<double>::infinity(), 1e-5);
         rc = push_ctl(ctx);
     }
-    // meshes with a side that is not a power of two need the octant of the
-    // 2n lengths only in the fft modes and for mm_kspace_product
+    // meshes with a side that is not a power of two need the [c][z][y][kx]
+    // arrays only in the fft modes; plane_setup fills the octant of their 2n
+    // lengths
     auto p2 = [](int n) { return (n & (n - 1)) == 0; };
     if (rc == MM_OK) rc = plane_plan(ctx);
     if (rc == MM_OK && (!ctx->plane.on || (p2(nx) && p2(ny)))) rc = classic_prepare(ctx);

@@ -1960,8 +1960,6 @@ int demag_prepare_ff(mm_ctx* ctx) {
 }
 
 int demag_kspace_product(mm_ctx* ctx, void* spec) {
-    int rc = classic_prepare(ctx);
-    if (rc) return rc;
     const long n = (long)ctx->Pz * ctx->Py * ctx->Hx;
     const unsigned blocks = (unsigned)((n + 255) / 256);
     if (ctx->prec == MM_F64)
@@ -2060,7 +2058,9 @@ int classic_prepare(mm_ctx* ctx) {
     if (!ctx->kern && (rc = dev_alloc(ctx, &ctx->kern, 6 * (size_t)ctx->Pz2 * ctx->Py2 * ctx->Hs * e))) return rc;
     if (!ctx->bufA && (rc = dev_alloc(ctx, &ctx->bufA, 3 * (size_t)ctx->nz * ctx->ny * ctx->Hs * 2 * e))) return rc;
     if (!ctx->bufB && (rc = dev_alloc(ctx, &ctx->bufB, 3 * (size_t)ctx->nz * ctx->Py * ctx->Hs * 2 * e))) return rc;
-    if ((rc = blue_prepare(ctx)) || (rc = demag_setup(ctx))) return rc;
+    if ((rc = blue_prepare(ctx))) return rc;
+    if (!ctx->kern_ready && (rc = demag_setup(ctx))) return rc;
+    ctx->kern_ready = true;
     ctx->classic_ready = true;
     return MM_OK;
 }

@@ -166,7 +166,8 @@ struct mm_ctx {
     int xtma_grid;            // its persistent grid
 
     mm::PlanePlan plane;
-    bool classic_ready;       // kern, bufA, bufB and the transform tables of the [c][z][y][kx] passes exist
+    bool kern_ready;          // kern holds the octant (from mm_init_mesh on)
+    bool classic_ready;       // bufA, bufB and the transform tables of the [c][z][y][kx] passes exist
 
     long launches;
     std::string err;
@@ -292,9 +293,9 @@ int tc_prepare(mm_ctx* ctx);
 
 // ----- demag (mm_demag.cu)
 int demag_setup(mm_ctx* ctx);                          // K1: Newell tensor -> k-space octant
-// kern, bufA, bufB and tables of the [c][z][y][kx] passes: at once for
-// contexts that run them, on first use for the others (fft modes,
-// mm_kspace_product)
+// kern, bufA, bufB and tables of the [c][z][y][kx] passes: in mm_init_mesh for
+// power-of-two meshes and those that run them, else when an fft mode that
+// needs them is set (kern exists from mm_init_mesh on)
 int classic_prepare(mm_ctx* ctx);
 // plane layout (mm_plane.cu): chooses and allocates the plan, fills its octant
 int plane_plan(mm_ctx* ctx);

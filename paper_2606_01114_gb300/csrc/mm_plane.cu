@@ -1,5 +1,6 @@
 // The plane-layout demag path: plan, octant and sequencing (the kernels and
 // their layout: mm_plane.cuh).
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -65,6 +66,16 @@ __global__ void k_octant_place(const double* __restrict__ in, T* __restrict__ ke
     const long kx = idx / ((long)KQ * Pz2);
     kern[((kx * 6 + comp) * Pz2 + kz) * KQ + ky] =
         ky < Py2 ? (T)(sign * in[((long)kz * Py2 + ky) * K + kx]) : (T)0;
+}
+
+// [kz][ky][kx] of one component -> its part [Pz2][Py2][Hs] of the [c][z][y][kx] octant
+template <typename T>
+__global__ void k_octant_rows(const double* __restrict__ in, T* __restrict__ kern, int Hx, int Hs, long rows,
+                              double sign) {
+    const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= rows * Hs) return;
+    const int kx = (int)(idx % Hs);
+    kern[idx] = kx < Hx ? (T)(sign * in[idx / Hs * Hx + kx]) : (T)0;
 }
 
 // octant of the [c][z][y][kx] passes, [6][Pz2][Py2][Hs] -> [K][6][Pz2][KQ]
@@ -167,13 +178,15 @@ void plane_free(mm_ctx* ctx) {
 }
 
 // Fills the plan's octant.  Same padded lengths as the [c][z][y][kx] passes
-// (powers of two from 16 up): their octant, turned.  Otherwise the Newell
-// tensor transformed axis by axis from its definition; that also fills
-// ctx->newell_host.
+// (powers of two): their octant, turned.  Otherwise the Newell tensor
+// transformed axis by axis from its definition; that also fills
+// ctx->newell_host and, on meshes with a side that is not a power of two, the
+// octant of the 2n lengths (mm_kspace_product reads it and must neither
+// allocate nor wait).
 int plane_setup(mm_ctx* ctx) {
     PlanePlan& p = ctx->plane;
     const int Pz2 = ctx->Pz2, Py2 = p.P / 2 + 1;
-    if (ctx->classic_ready && p.L == ctx->nx && p.P == ctx->Py) {
+    if (ctx->kern_ready && p.L == ctx->nx && p.P == ctx->Py) {
         const long n = kern_count(ctx);
         if (ctx->prec == MM_F64)
             k_octant_turn<double><<<blocks(n), 256, 0, ctx->stream>>>((const double*)ctx->kern, (double*)p.kern, p.K, Pz2,
@@ -184,17 +197,23 @@ int plane_setup(mm_ctx* ctx) {
         MM_LAUNCH_CHECK(ctx);
         return MM_OK;
     }
-    const int len[3] = {2 * p.L, p.P, ctx->Pz}, n[3] = {ctx->nx, ctx->ny, ctx->nz}, m[3] = {p.K, Py2, Pz2};
+    const int n[3] = {ctx->nx, ctx->ny, ctx->nz};
+    // lengths and kept frequencies of the plan, and of the 2n octant
+    const int len[2][3] = {{2 * p.L, p.P, ctx->Pz}, {ctx->Px, ctx->Py, ctx->Pz}};
+    const int m[2][3] = {{p.K, Py2, Pz2}, {ctx->Hx, ctx->Py2, Pz2}};
+    const int sets = ctx->kern_ready ? 1 : 2;
     std::vector<double> t;
-    long off[3];
-    for (int a = 0; a < 3; ++a) {
-        off[a] = (long)t.size();
-        std::vector<double> e;
-        table(len[a], e);
-        for (int s = 0; s < 2; ++s)
-            for (int q = 0; q < len[a]; ++q) t.push_back(s ? -e[2 * q + 1] : e[2 * q]);   // cos, then sin
-    }
+    long off[2][3];
+    for (int q = 0; q < sets; ++q)
+        for (int a = 0; a < 3; ++a) {
+            off[q][a] = (long)t.size();
+            std::vector<double> e;
+            table(len[q][a], e);
+            for (int s = 0; s < 2; ++s)
+                for (int i = 0; i < len[q][a]; ++i) t.push_back(s ? -e[2 * i + 1] : e[2 * i]);   // cos, then sin
+        }
     const long fsize = (long)(ctx->nx + 1) * (ctx->ny + 1) * (ctx->nz + 1);
+    const size_t K = sets > 1 ? std::max(p.K, ctx->Hx) : p.K, Y = sets > 1 ? std::max(Py2, ctx->Py2) : Py2;
     void *oct = nullptr, *fg = nullptr, *a1 = nullptr, *a2 = nullptr, *a3 = nullptr, *tab = nullptr;
     auto cleanup = [&]() {
         for (void* q : {oct, fg, a1, a2, a3, tab}) cudaFree(q);
@@ -203,11 +222,12 @@ int plane_setup(mm_ctx* ctx) {
     auto A = [&](void** q, size_t b) {
         if (rc == MM_OK) rc = dev_alloc(ctx, q, b);
     };
+    if (sets > 1) A(&ctx->kern, 6 * (size_t)Pz2 * ctx->Py2 * ctx->Hs * elem(ctx));
     A(&oct, sizeof(double) * 6 * ctx->N);
     A(&fg, sizeof(double2) * fsize);
-    A(&a1, sizeof(double) * (size_t)ctx->nz * ctx->ny * p.K);
-    A(&a2, sizeof(double) * (size_t)ctx->nz * Py2 * p.K);
-    A(&a3, sizeof(double) * (size_t)Pz2 * Py2 * p.K);
+    A(&a1, sizeof(double) * (size_t)ctx->nz * ctx->ny * K);
+    A(&a2, sizeof(double) * (size_t)ctx->nz * Y * K);
+    A(&a3, sizeof(double) * (size_t)Pz2 * Y * K);
     A(&tab, sizeof(double) * t.size());
     if (rc == MM_OK && cudaMemcpy(tab, t.data(), sizeof(double) * t.size(), cudaMemcpyHostToDevice) != cudaSuccess)
         rc = fail(ctx, MM_ERR_CUDA, "octant table copy failed");
@@ -215,23 +235,36 @@ int plane_setup(mm_ctx* ctx) {
         double* oc = (double*)oct + c * ctx->N;
         if ((rc = newell_component(ctx, c, nullptr, oc, fg))) break;
         const int odd[3] = {c == 3 || c == 4, c == 3 || c == 5, c == 4 || c == 5};
+        const double sign = c >= 3 ? -1.0 : 1.0;
         const double* src[3] = {oc, (const double*)a1, (const double*)a2};
         double* dst[3] = {(double*)a1, (double*)a2, (double*)a3};
-        const long O[3] = {(long)ctx->nz * ctx->ny, ctx->nz, 1}, I[3] = {1, p.K, (long)Py2 * p.K};
-        for (int a = 0; a < 3; ++a) {
-            const long total = O[a] * m[a] * I[a];
-            k_octant_axis<<<blocks(total), 256, 0, ctx->stream>>>(src[a], dst[a], O[a], n[a], (int)I[a], m[a], len[a],
-                                                                 odd[a], (const double*)tab + off[a] + (odd[a] ? len[a] : 0));
+        for (int q = 0; q < sets; ++q) {
+            const long O[3] = {(long)ctx->nz * ctx->ny, ctx->nz, 1}, I[3] = {1, m[q][0], (long)m[q][1] * m[q][0]};
+            for (int a = 0; a < 3; ++a) {
+                const long total = O[a] * m[q][a] * I[a];
+                k_octant_axis<<<blocks(total), 256, 0, ctx->stream>>>(
+                    src[a], dst[a], O[a], n[a], (int)I[a], m[q][a], len[q][a], odd[a],
+                    (const double*)tab + off[q][a] + (odd[a] ? len[q][a] : 0));
+            }
+            if (q == 0) {
+                const long total = (long)p.K * Pz2 * p.KQ;
+                if (ctx->prec == MM_F64)
+                    k_octant_place<double><<<blocks(total), 256, 0, ctx->stream>>>(
+                        (const double*)a3, (double*)p.kern, c, p.K, Pz2, Py2, p.KQ, sign);
+                else
+                    k_octant_place<float><<<blocks(total), 256, 0, ctx->stream>>>((const double*)a3, (float*)p.kern, c,
+                                                                                  p.K, Pz2, Py2, p.KQ, sign);
+            } else {
+                const long rows = (long)Pz2 * ctx->Py2, total = rows * ctx->Hs;
+                if (ctx->prec == MM_F64)
+                    k_octant_rows<double><<<blocks(total), 256, 0, ctx->stream>>>(
+                        (const double*)a3, (double*)ctx->kern + c * total, ctx->Hx, ctx->Hs, rows, sign);
+                else
+                    k_octant_rows<float><<<blocks(total), 256, 0, ctx->stream>>>(
+                        (const double*)a3, (float*)ctx->kern + c * total, ctx->Hx, ctx->Hs, rows, sign);
+            }
+            ctx->launches += 4;
         }
-        const long total = (long)p.K * Pz2 * p.KQ;
-        const double sign = c >= 3 ? -1.0 : 1.0;
-        if (ctx->prec == MM_F64)
-            k_octant_place<double><<<blocks(total), 256, 0, ctx->stream>>>((const double*)a3, (double*)p.kern, c, p.K,
-                                                                           Pz2, Py2, p.KQ, sign);
-        else
-            k_octant_place<float><<<blocks(total), 256, 0, ctx->stream>>>((const double*)a3, (float*)p.kern, c, p.K, Pz2,
-                                                                          Py2, p.KQ, sign);
-        ctx->launches += 4;
         if (cudaGetLastError() != cudaSuccess) rc = fail(ctx, MM_ERR_CUDA, "octant kernel launch failed");
     }
     cudaError_t e = cudaSuccess;
@@ -241,6 +274,7 @@ int plane_setup(mm_ctx* ctx) {
     if (rc == MM_OK && (e != cudaSuccess || es != cudaSuccess))
         rc = fail(ctx, MM_ERR_CUDA, "octant setup failed: %s", cudaGetErrorString(e != cudaSuccess ? e : es));
     cleanup();
+    if (rc == MM_OK) ctx->kern_ready = true;
     return rc;
 }
 
