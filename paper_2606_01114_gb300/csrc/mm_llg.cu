@@ -562,7 +562,8 @@ constexpr int kReduceThreads = 128;
 
 // Energies: each thread sums its cells in double (grid stride), so the block
 // reduction of the five sums, 25 FP64 adds a thread, is paid once and not per
-// cell; terms whose constant is zero are skipped.
+// cell; terms whose constant is zero are skipped.  A magnetic cell that is not
+// finite makes a skipped anisotropy or Zeeman sum NaN, as 0 m does.
 template <typename T>
 __global__ void __launch_bounds__(kReduceThreads)
     k_energy(Params<T> p, const T* __restrict__ m, const T* __restrict__ Hd, double V, double mu0, double Ku,
@@ -571,6 +572,7 @@ __global__ void __launch_bounds__(kReduceThreads)
     double ed = 0, ex = 0, ea = 0, ez = 0, em = 0;
     const double c = -mu0 * V;
     const bool zeeman = p.hx != (T)0 || p.hy != (T)0 || p.hz != (T)0;
+    bool bad = false;
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < p.N; i += (long)gridDim.x * blockDim.x) {
         int x, y, z;
         decompose(i, p.nx, p.ny, x, y, z);
@@ -580,6 +582,7 @@ __global__ void __launch_bounds__(kReduceThreads)
         const V3<T> mi = load3(m, i, p.N);
         const V3<T> h = exchange_at(p, m, i, x, y, z, mi, inv);
         const V3<T> d = load3(Hd, i, p.N);
+        bad |= !(isfinite(mi.x) && isfinite(mi.y) && isfinite(mi.z));
         const double mx = mi.x, my = mi.y, mz = mi.z, w = c * (double)Msi, hw = 0.5 * w;
         ed += hw * (mx * d.x + my * d.y + mz * d.z);
         ex += hw * (mx * h.x + my * h.y + mz * h.z);
@@ -607,6 +610,10 @@ __global__ void __launch_bounds__(kReduceThreads)
     if (p.dmi) {
         __syncthreads();
         block_sum_atomic(em, &ctl->energy[4]);
+    }
+    if (__syncthreads_or(bad) && threadIdx.x == 0) {
+        if (Ku == 0.0) atomicAdd(&ctl->energy[2], NAN);
+        if (!zeeman) atomicAdd(&ctl->energy[3], NAN);
     }
 }
 
