@@ -1,0 +1,85 @@
+"""Routes of the demag passes and of the gradient that no other test reaches:
+the chirp-z and direct passes that one-cell sides keep, the copy-engine-fed
+passes on meshes that still take them, and gradients of several steps on
+meshes whose forward record runs in the fused kernels.
+
+Tolerances are the library's own (FP64 1e-12, FP32 1e-5 relative L2; 1e-4 for
+an FP32 gradient against the FP64 one)."""
+
+import numpy as np
+import pytest
+
+import workloads as wl
+from oracle import micromag
+
+torch = pytest.importorskip("torch")
+import paper_2606_01114_gb300 as mm  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+D = (2e-9, 2.5e-9, 3e-9)
+TOL = {"f64": 1e-12, "f32": 1e-5}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2606_01114_gb300 import build
+    build.build()
+
+
+def context(n, prec):
+    ctx = mm.mm_init_mesh(*n, *D, precision=mm.MM_F32 if prec == "f32" else mm.MM_F64)
+    mm.mm_set_material(ctx, 8e5, 1.3e-11, 0.1, 1e5)
+    return ctx
+
+
+def dev(a, prec):
+    return torch.tensor(a, dtype=torch.float32 if prec == "f32" else torch.float64, device="cuda")
+
+
+def rel(t, ref):
+    return np.linalg.norm(t.double().cpu().numpy() - ref) / np.linalg.norm(ref)
+
+
+# one-cell sides: chirp-z in y, in x, direct in both; then power-of-two meshes
+# of more layers than a plane block holds, whose y passes of length 512 and
+# 1024 and x inverse of 512 cells are fed by the copy engine (one, some and
+# many columns, a tile that is not full)
+ONE_CELL = [(1, 100, 4), (1, 350, 1), (100, 1, 2), (1, 511, 16), (333, 1, 1), (1, 31, 2), (29, 1, 8)]
+FED = [(8, 512, 16), (16, 256, 16), (512, 4, 16), (1, 512, 16), (2, 256, 32), (512, 256, 16)]
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("n", ONE_CELL + FED, ids=lambda n: "x".join(map(str, n)))
+def test_demag_on_the_routes_of_2n_lengths(n, prec):
+    m = wl.random_unit(n, seed=sum(n))
+    ctx = context(n, prec)
+    md = dev(m, prec)
+    H = torch.full_like(md, float("nan"))
+    mm.mm_demag_field(ctx, md, H)
+    assert rel(H, micromag.Problem(n, D).demag_fft(m)) < TOL[prec]
+    mm.mm_destroy(ctx)
+
+
+@pytest.mark.parametrize("every", [0, 3, 7])
+@pytest.mark.parametrize("n", [(64, 64, 4), (33, 61, 8), (130, 333, 2)], ids=lambda n: "x".join(map(str, n)))
+def test_gradient_of_several_fused_steps(n, every):
+    """Seven RK4 steps with cell-wise Ms and vacuum: the FP32 gradient, whose
+    record of the steps is written by the fused kernels, against the FP64
+    one."""
+    rng = np.random.default_rng(sum(n))
+    Ms = rng.uniform(4e5, 9e5, size=n[::-1]).astype(np.float32).astype(np.float64)
+    Ms[rng.random(Ms.shape) < 0.2] = 0.0
+    m = wl.random_unit(n, seed=5).astype(np.float32).astype(np.float64)
+    lam0 = wl.random_unit(n, seed=6).astype(np.float32).astype(np.float64)
+    out = []
+    for prec in ("f64", "f32"):
+        ctx = context(n, prec)
+        mm.mm_set_material_fields(ctx, Ms_cell=dev(Ms, prec))
+        lam = dev(lam0, prec)
+        gMs = torch.zeros(ctx.shape1, dtype=lam.dtype, device="cuda")
+        mm.mm_rk4_trajectory_vjp(ctx, dev(m, prec), 1e-14, 7, lam, gMs, every)
+        out.append((lam.double().cpu().numpy(), gMs.double().cpu().numpy()))
+        mm.mm_destroy(ctx)
+    for a, b in zip(*out):
+        assert np.isfinite(b).all() and np.linalg.norm(b - a) < 1e-4 * np.linalg.norm(a)
