@@ -479,8 +479,14 @@ template <typename T> __device__ __forceinline__ void cp_async_value(T* smem, co
     const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(a), "l"(gmem), "n"(sizeof(T)) : "memory");
 }
+// FP64 at Pz = 1024: three components of 32 values are 384 registers, which
+// spilled (12x12x512 477 us a field).  The middle level then goes one component
+// at a time, with the product between two barriers, and the octant is read from
+// global memory, so that four columns fit an SM (342; 60x60x512 6781 -> 4856).
+template <typename T> constexpr bool zline_split(int PZ) { return std::is_same<T, double>::value && PZ == 1024; }
 template <typename T, int L1, int L2, int B> constexpr size_t zline_smem() {
-    return (size_t)3 * L1 * (L2 + 1) * B * sizeof(PC<T>) + (size_t)6 * (L1 * L2 / 2 + 1) * B * sizeof(T);
+    return (size_t)3 * L1 * (L2 + 1) * B * sizeof(PC<T>) +
+           (zline_split<T>(L1 * L2) ? 0 : (size_t)6 * (L1 * L2 / 2 + 1) * B * sizeof(T));
 }
 
 template <typename T, int L1, int L2, bool COLY, int B, int NT, int MINB>
@@ -506,11 +512,16 @@ __global__ void __launch_bounds__(NT, MINB)
     }
     C* base = buf + (long)row * g.row_s + col0;
     const T* kbase = kern + (long)krow * g.k_row;
-    for (int i = tid; i < 6 * PZ2 * B; i += NT) {
-        const int b = i % B, ck = i / B, kz = ck % PZ2, c = ck / PZ2;
+    constexpr bool SPLIT = zline_split<T>(PZ);
+    auto octant_col = [&](int b) {
         const int col = col0 + b < g.ncol ? col0 + b : g.ncol - 1;
-        const int kcol = COLY && 2 * col > g.P ? g.P - col : col;
-        cp_async_value(Kn + i, kbase + c * g.kc_s + kz * g.kz_s + kcol);
+        return COLY && 2 * col > g.P ? g.P - col : col;
+    };
+    if constexpr (!SPLIT) {
+        for (int i = tid; i < 6 * PZ2 * B; i += NT) {
+            const int b = i % B, ck = i / B, kz = ck % PZ2, c = ck / PZ2;
+            cp_async_value(Kn + i, kbase + c * g.kc_s + kz * g.kz_s + octant_col(b));
+        }
     }
 #pragma unroll 1
     for (int i = tid; i < 3 * L2 * B; i += NT) {
@@ -530,45 +541,92 @@ __global__ void __launch_bounds__(NT, MINB)
             s[k1 * LQ * B] = y;
         }
     }
-    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    if constexpr (!SPLIT) {
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+    }
     __syncthreads();
+    if constexpr (SPLIT) {
 #pragma unroll 1
-    for (int i = tid; i < L1 * B; i += NT) {
-        const int b = i % B, k1 = i / B;
-        const bool yodd = COLY ? 2 * (col0 + b) > g.P : rodd;
-        C* s = Sm + k1 * LQ * B + b;
-        const C* tq = tw + PZ + k1;
-        C u[3][L2];
+        for (int i = tid; i < 3 * L1 * B; i += NT) {
+            const int b = i % B, ck = i / B, k1 = ck % L1;
+            C* s = Sm + (ck / L1) * CP + k1 * LQ * B + b;
+            C u[L2];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
+            for (int n2 = 0; n2 < L2; ++n2) u[n2] = s[n2 * B];
+            dif<L2, -1, false>(u);
 #pragma unroll
-            for (int n2 = 0; n2 < L2; ++n2) u[c][n2] = s[c * CP + n2 * B];
-            dif<L2, -1, false>(u[c]);
+            for (int k2 = 0; k2 < L2; ++k2) s[k2 * B] = u[dif_pos<L2>(k2)];
         }
-#pragma unroll
-        for (int k2 = 0; k2 < L2; ++k2) {
-            const int kz = k1 + L1 * k2;
-            const bool zodd = 2 * kz > PZ;
-            const T* kk = Kn + (zodd ? PZ - kz : kz) * B + b;
-            const T xx = kk[0], yy = kk[PZ2 * B], zz = kk[2 * PZ2 * B];
-            T xy = kk[3 * PZ2 * B], xz = kk[4 * PZ2 * B], yz = kk[5 * PZ2 * B];
+        __syncthreads();
+#pragma unroll 2
+        for (int i = tid; i < PZ * B; i += NT) {
+            const int b = i % B, kz = i / B, k2 = kz / L1, k1 = kz - k2 * L1;
+            const bool yodd = COLY ? 2 * (col0 + b) > g.P : rodd, zodd = 2 * kz > PZ;
+            const T* kk = kbase + (zodd ? PZ - kz : kz) * g.kz_s + octant_col(b);
+            const T xx = kk[0], yy = kk[g.kc_s], zz = kk[2 * g.kc_s];
+            T xy = kk[3 * g.kc_s], xz = kk[4 * g.kc_s], yz = kk[5 * g.kc_s];
             if (yodd) xy = -xy;
             if (zodd) xz = -xz;
             if (yodd != zodd) yz = -yz;
-            const int q = dif_pos<L2>(k2);
-            tensor_product<T>(u[0][q], u[1][q], u[2][q], xx, yy, zz, xy, xz, yz);
+            C* s = Sm + (k1 * LQ + k2) * B + b;
+            tensor_product<T>(s[0], s[CP], s[2 * CP], xx, yy, zz, xy, xz, yz);
         }
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
+        __syncthreads();
+#pragma unroll 1
+        for (int i = tid; i < 3 * L1 * B; i += NT) {
+            const int b = i % B, ck = i / B, k1 = ck % L1;
+            C* s = Sm + (ck / L1) * CP + k1 * LQ * B + b;
+            const C* tq = tw + PZ + k1;
             C w[L2];
 #pragma unroll
-            for (int k2 = 0; k2 < L2; ++k2) w[k2] = u[c][dif_pos<L2>(k2)];
+            for (int k2 = 0; k2 < L2; ++k2) w[k2] = s[k2 * B];
             dif<L2, +1, false>(w);
 #pragma unroll
             for (int t = 0; t < L2; ++t) {
                 C y = w[dif_pos<L2>(t)];
                 if (t > 0) y = cmul(y, cconj(tq[t * L1]));
-                s[c * CP + t * B] = y;
+                s[t * B] = y;
+            }
+        }
+    } else {
+#pragma unroll 1
+        for (int i = tid; i < L1 * B; i += NT) {
+            const int b = i % B, k1 = i / B;
+            const bool yodd = COLY ? 2 * (col0 + b) > g.P : rodd;
+            C* s = Sm + k1 * LQ * B + b;
+            const C* tq = tw + PZ + k1;
+            C u[3][L2];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+#pragma unroll
+                for (int n2 = 0; n2 < L2; ++n2) u[c][n2] = s[c * CP + n2 * B];
+                dif<L2, -1, false>(u[c]);
+            }
+#pragma unroll
+            for (int k2 = 0; k2 < L2; ++k2) {
+                const int kz = k1 + L1 * k2;
+                const bool zodd = 2 * kz > PZ;
+                const T* kk = Kn + (zodd ? PZ - kz : kz) * B + b;
+                const T xx = kk[0], yy = kk[PZ2 * B], zz = kk[2 * PZ2 * B];
+                T xy = kk[3 * PZ2 * B], xz = kk[4 * PZ2 * B], yz = kk[5 * PZ2 * B];
+                if (yodd) xy = -xy;
+                if (zodd) xz = -xz;
+                if (yodd != zodd) yz = -yz;
+                const int q = dif_pos<L2>(k2);
+                tensor_product<T>(u[0][q], u[1][q], u[2][q], xx, yy, zz, xy, xz, yz);
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                C w[L2];
+#pragma unroll
+                for (int k2 = 0; k2 < L2; ++k2) w[k2] = u[c][dif_pos<L2>(k2)];
+                dif<L2, +1, false>(w);
+#pragma unroll
+                for (int t = 0; t < L2; ++t) {
+                    C y = w[dif_pos<L2>(t)];
+                    if (t > 0) y = cmul(y, cconj(tq[t * L1]));
+                    s[c * CP + t * B] = y;
+                }
             }
         }
     }

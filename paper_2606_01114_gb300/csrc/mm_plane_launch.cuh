@@ -173,12 +173,8 @@ template <typename F> bool with_z_length(int len, F&& f) {
 // threads 952 us, 256 threads 1050 us (208 registers) or 1450 us (128, two
 // blocks per SM, spills), 128 threads 1243 us; 256 x 256 x 32 (Pz = 64,
 // whole field): 128 threads 194 us, 256 threads 234 us.
-template <typename T, int L1, int L2, bool COLY>
-int launch_zline_t(mm_ctx* ctx, PC<T>* buf, const T* kern, const ZLine& g, int nrows, const PC<T>* tw) {
-    constexpr int PZ = L1 * L2, CS = (int)sizeof(PC<T>);
-    constexpr int B = PZ <= 64 ? 128 / CS : PZ <= 512 ? 64 / CS : 32 / CS;
-    constexpr int NT = sizeof(T) == 8 ? (PZ == 512 ? 192 : 128) : PZ == 64 ? 128 : PZ == 256 ? 256 : PZ >= 512 ? 384 : 192;
-    constexpr int MINB = sizeof(T) == 8 ? 1 : PZ <= 32 ? 4 : PZ == 64 ? 4 : PZ == 128 ? 3 : PZ == 256 ? 2 : 1;
+template <typename T, int L1, int L2, bool COLY, int B, int NT, int MINB>
+int launch_zline_b(mm_ctx* ctx, PC<T>* buf, const T* kern, const ZLine& g, int nrows, const PC<T>* tw) {
     auto fn = k_zline<T, L1, L2, COLY, B, NT, MINB>;
     const size_t smem = zline_smem<T, L1, L2, B>();
     int rc = smem_opt_in(ctx, (const void*)fn, smem);
@@ -187,6 +183,21 @@ int launch_zline_t(mm_ctx* ctx, PC<T>* buf, const T* kern, const ZLine& g, int n
     dep(fn, grid, NT, smem, ctx->stream)(buf, kern, g, tw);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
+}
+template <typename T, int L1, int L2, bool COLY>
+int launch_zline_t(mm_ctx* ctx, PC<T>* buf, const T* kern, const ZLine& g, int nrows, const PC<T>* tw) {
+    constexpr int PZ = L1 * L2, CS = (int)sizeof(PC<T>);
+    if constexpr (zline_split<T>(PZ)) {
+        // one column a block while four of them would leave SMs idle (5x2x512:
+        // 264 us a field with four, 18 blocks; 97 with one)
+        if ((long)g.ncol * nrows <= 4 * 152) return launch_zline_b<T, L1, L2, COLY, 1, 96, 1>(ctx, buf, kern, g, nrows, tw);
+        return launch_zline_b<T, L1, L2, COLY, 4, 384, 1>(ctx, buf, kern, g, nrows, tw);
+    } else {
+        constexpr int B = PZ <= 64 ? 128 / CS : PZ <= 512 ? 64 / CS : 32 / CS;
+        constexpr int NT = sizeof(T) == 8 ? (PZ == 512 ? 192 : 128) : PZ == 64 ? 128 : PZ == 256 ? 256 : PZ >= 512 ? 384 : 192;
+        constexpr int MINB = sizeof(T) == 8 ? 1 : PZ <= 32 ? 4 : PZ == 64 ? 4 : PZ == 128 ? 3 : PZ == 256 ? 2 : 1;
+        return launch_zline_b<T, L1, L2, COLY, B, NT, MINB>(ctx, buf, kern, g, nrows, tw);
+    }
 }
 
 template <typename T, bool COLY>

@@ -83,3 +83,19 @@ def test_gradient_of_several_fused_steps(n, every):
         mm.mm_destroy(ctx)
     for a, b in zip(*out):
         assert np.isfinite(b).all() and np.linalg.norm(b - a) < 1e-4 * np.linalg.norm(a)
+
+
+# z length 1024 in FP64: the middle level by components, one and four columns a
+# block
+LONG = [(5, 2, 512), (12, 6, 512), (3, 3, 512), (7, 5, 512), (2, 9, 512), (20, 17, 512), (3, 70, 512)]
+
+
+@pytest.mark.parametrize("n", LONG, ids=lambda n: "x".join(map(str, n)))
+def test_demag_on_the_longest_z_lines_in_double(n):
+    m = wl.random_unit(n, seed=sum(n))
+    ctx = context(n, "f64")
+    md = dev(m, "f64")
+    H = torch.full_like(md, float("nan"))
+    mm.mm_demag_field(ctx, md, H)
+    assert rel(H, micromag.Problem(n, D).demag_fft(m)) < TOL["f64"]
+    mm.mm_destroy(ctx)
