@@ -85,11 +85,11 @@ struct Blue {
 };
 
 // The plane-layout demag path (mm_plane.cu).  Lengths are padded to the next
-// of {4, 5, 6, 8} 2^k >= 2n, so they differ from ctx->Px, Py when a side is
-// not a power of two.
+// of 8, 16, 32 and {4, 5, 6} 2^k (k >= 3) >= 2n, so they differ from ctx->Px,
+// Py when a side is not a power of two, or below 4.
 struct PlanePlan {
     int on = 0;          // the plain (fft_mode 0) and float-float passes run in the plane layout
-    int lines = 0;       // planes too large for one block: y, z, y as three kernels
+    int lines = 0;       // y, z, y as three kernels: planes too large for one block, or too few (FP64)
     int L = 0, P = 0;    // complex x length (P_x / 2), padded y length
     int K = 0;           // planes: L + 1 kept x frequencies
     int KQ = 0;          // octant row stride (P / 2 + 1 rounded up to 4)

@@ -20,10 +20,10 @@ namespace {
 
 bool pow2(int n) { return n > 0 && (n & (n - 1)) == 0; }
 
-// next of 16, 32 and {4, 5, 6} 2^k, k >= 3, that is >= n
-int next_len(int n) {
-    if (n <= 16) return 16;
-    if (n <= 32) return 32;
+// next of `least` (4 or 8), 8, 16, 32 and {4, 5, 6} 2^k, k >= 3, that is >= n
+int next_len(int n, int least) {
+    for (int l = least; l <= 32; l *= 2)
+        if (n <= l) return l;
     for (int p = 32;; p *= 2)
         for (int q = 4; q <= 6; ++q)
             if (q * p / 4 >= n) return q * p / 4;
@@ -124,19 +124,34 @@ void table(int L, std::vector<double>& out) {
 // 1804 against 1826 us.  On the near side of the line: 512x512x4 FP32 85
 // against 96 us, 64x512x8 (65 planes) 40 against 43 us, 256x256x8 44 against
 // 56 us.
+// The plane is a block's serial work, so few planes of many values leave most
+// SMs idle.  In FP64 (one warp instruction per sub-partition and 64 cycles) that
+// counts more than the two passes over memory it saves: up to 65 planes of nz P >= 256
+// run y, z and y as three kernels.  FP64 demag, plane -> three kernels (-> the
+// five passes of the power-of-two meshes): 16x512x4 342 -> 107 (150) us,
+// 64x512x4 375 -> 252 (333), 16x256x2 81 -> 62 (115), 64x128x2 49 -> 45 (129),
+// 32x64x4 43 -> 36 (123); at 97 planes 96x128x2 53 -> 53 and 96x64x2 37 -> 38.
+// A side of three cells beside a power of two and many layers keeps the 2n
+// passes: they are direct on that side (2n = 6, here 8) and need no chirp-z,
+// and from about 98 k cells in FP64, 197 k in FP32 with ny = 3, the columns
+// they save count more than launches: 512x3x256 FP64 939 against 1239 us,
+// 3x512x128 654 against 774, 512x3x128 FP32 67 against 78 (256x3x128 47
+// against 45, 3x512x512 356 against 271).
 int plane_plan(mm_ctx* ctx) {
     PlanePlan& p = ctx->plane;
     p = PlanePlan();
     if (ctx->nx < 2 || ctx->ny < 2) return MM_OK;
     const size_t cs = 2 * elem(ctx);
-    p.L = next_len(ctx->nx);
-    p.P = next_len(2 * ctx->ny);
+    p.L = next_len(ctx->nx, 4);
+    p.P = next_len(2 * ctx->ny, 8);     // (8: what the float-float stages need)
     const bool regular = pow2(ctx->nx) && pow2(ctx->ny);
     const size_t smem = 3 * (size_t)ctx->nz * plane_line_len(p.P) * cs;
     const bool fits = ctx->nz <= (ctx->prec == MM_F32 ? 8 : 4) && smem <= 227 * 1024;
     if (regular && (!fits || (smem > 113 * 1024 && p.L + 1 > 152))) return MM_OK;
+    const bool strip = (ctx->nx == 3 && pow2(ctx->ny)) || (ctx->ny == 3 && pow2(ctx->nx));
+    if (strip && (ctx->prec == MM_F64 ? ctx->N >= 98304 : ctx->ny == 3 && ctx->N >= 196608)) return MM_OK;
     p.on = 1;
-    p.lines = !fits;
+    p.lines = !fits || (ctx->prec == MM_F64 && ctx->nz > 1 && p.L <= 64 && ctx->nz * p.P >= 256);
     p.K = p.L + 1;
     p.KQ = (p.P / 2 + 1 + 3) / 4 * 4;
     p.R = (3L * ctx->nz * ctx->ny + 3) / 4 * 4;

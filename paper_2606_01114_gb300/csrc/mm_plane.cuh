@@ -12,10 +12,12 @@
 // z product and y inverse as three kernels in the same layout (k_py, k_zline).
 //
 // Lengths.  The convolution is linear, so the padded length P may be any
-// length >= 2n: it is the next of {4, 5, 6, 8} 2^k, not 2n itself.  Meshes
-// whose sides are not powers of two therefore run the same four-step
-// transforms as the others (at most a quarter of padding more) and need no
-// chirp-z convolution of length >= 4n - 1.
+// length >= 2n: it is the next of 8 (x: 2 L, L = 4), 16, 32 and {4, 5, 6} 2^k
+// from 32 on, not 2n itself.  Meshes whose sides are not powers of two
+// therefore run the same four-step transforms as the others and need no
+// chirp-z convolution of length >= 4n - 1.  The padding is at most a third more
+// above 32 (2n = 770 takes 1024); lengths 12, 20 and 24 below it were slower
+// than the 16 and 32 that hold them (FP64 12x11x16, P = 24: 33 us against 28).
 //
 // Every transform is a four-step L = L1 x L2 with both levels in registers:
 // level 1 (thread t < L2) DFT over n1 of x[t + L2 n1], twiddle w^(t k1);

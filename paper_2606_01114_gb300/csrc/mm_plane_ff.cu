@@ -172,7 +172,7 @@ int launch_ff_plane(mm_ctx* ctx, ffc* buf, const ffc* tw) {
 // whether the float-float plane kernel takes this mesh: the Stockham stages
 // need 3 nz P / 8 threads, and 384 leave the z phase its 168 registers
 bool plane_ff_fits(const mm_ctx* ctx) {
-    return ctx->plane.on && !ctx->plane.lines && 3 * ctx->nz * ctx->plane.P <= 8 * kPlaneThreads && ctx->nx % 2 == 0;
+    return ctx->plane.on && ctx->nz <= 4 && 3 * ctx->nz * ctx->plane.P <= 8 * kPlaneThreads && ctx->nx % 2 == 0;
 }
 
 int plane_apply_ff(mm_ctx* ctx, const double* m, const double* Ms, double ms, double* H) {

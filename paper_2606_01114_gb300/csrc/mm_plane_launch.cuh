@@ -16,6 +16,8 @@ template <typename F> bool with_length(int len, F&& f) {
 #define MM_LEN(N, A, B) \
     case N: f(std::integral_constant<int, A>{}, std::integral_constant<int, B>{}); return true
     switch (len) {
+        MM_LEN(4, 2, 2);
+        MM_LEN(8, 4, 2);
         MM_LEN(16, 4, 4);
         MM_LEN(32, 8, 4);
         MM_LEN(64, 8, 8);
@@ -155,6 +157,8 @@ template <typename F> bool with_z_length(int len, F&& f) {
 #define MM_LEN(N, A, B) \
     case N: f(std::integral_constant<int, A>{}, std::integral_constant<int, B>{}); return true
     switch (len) {
+        MM_LEN(4, 2, 2);
+        MM_LEN(8, 4, 2);
         MM_LEN(16, 4, 4);
         MM_LEN(32, 8, 4);
         MM_LEN(64, 8, 8);
@@ -172,7 +176,9 @@ template <typename F> bool with_z_length(int len, F&& f) {
 // NT threads: level 1 has 3 L2 B tasks, the middle level L1 B.  256^3: 384
 // threads 952 us, 256 threads 1050 us (208 registers) or 1450 us (128, two
 // blocks per SM, spills), 128 threads 1243 us; 256 x 256 x 32 (Pz = 64,
-// whole field): 128 threads 194 us, 256 threads 234 us.
+// whole field): 128 threads 194 us, 256 threads 234 us.  FP64 planes of two
+// and four layers that take this pass (mm_plane.cu) have 3 to 6 values a
+// column: 32 columns keep a block's warps full.
 template <typename T, int L1, int L2, bool COLY, int B, int NT, int MINB>
 int launch_zline_b(mm_ctx* ctx, PC<T>* buf, const T* kern, const ZLine& g, int nrows, const PC<T>* tw) {
     auto fn = k_zline<T, L1, L2, COLY, B, NT, MINB>;
@@ -193,7 +199,7 @@ int launch_zline_t(mm_ctx* ctx, PC<T>* buf, const T* kern, const ZLine& g, int n
         if ((long)g.ncol * nrows <= 4 * 152) return launch_zline_b<T, L1, L2, COLY, 1, 96, 1>(ctx, buf, kern, g, nrows, tw);
         return launch_zline_b<T, L1, L2, COLY, 4, 384, 1>(ctx, buf, kern, g, nrows, tw);
     } else {
-        constexpr int B = PZ <= 64 ? 128 / CS : PZ <= 512 ? 64 / CS : 32 / CS;
+        constexpr int B = PZ <= 8 ? 32 : PZ <= 64 ? 128 / CS : PZ <= 512 ? 64 / CS : 32 / CS;
         constexpr int NT = sizeof(T) == 8 ? (PZ == 512 ? 192 : 128) : PZ == 64 ? 128 : PZ == 256 ? 256 : PZ >= 512 ? 384 : 192;
         constexpr int MINB = sizeof(T) == 8 ? 1 : PZ <= 32 ? 4 : PZ == 64 ? 4 : PZ == 128 ? 3 : PZ == 256 ? 2 : 1;
         return launch_zline_b<T, L1, L2, COLY, B, NT, MINB>(ctx, buf, kern, g, nrows, tw);
@@ -205,7 +211,12 @@ int launch_zline(mm_ctx* ctx, int Pz, PC<T>* buf, const T* kern, const ZLine& g,
     KernelTimer kt(ctx, MM_K_ZCONV);
     int rc = MM_OK;
     if (!with_z_length(Pz, [&](auto A, auto B) {
-            rc = launch_zline_t<T, decltype(A)::value, decltype(B)::value, COLY>(ctx, buf, kern, g, nrows, tw);
+            constexpr int L1 = decltype(A)::value, L2 = decltype(B)::value;
+            // the lengths that reach this pass: FP32 planes from 16 on, kx columns from 64 on
+            if constexpr (sizeof(T) == 8 || L1 * L2 >= (COLY ? 16 : 64))
+                rc = launch_zline_t<T, L1, L2, COLY>(ctx, buf, kern, g, nrows, tw);
+            else
+                rc = fail(ctx, MM_ERR_INVALID_ARG, "z length %d", Pz);
         }))
         return fail(ctx, MM_ERR_INVALID_ARG, "z length %d", Pz);
     return rc;

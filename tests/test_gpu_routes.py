@@ -99,3 +99,54 @@ def test_demag_on_the_longest_z_lines_in_double(n):
     mm.mm_demag_field(ctx, md, H)
     assert rel(H, micromag.Problem(n, D).demag_fft(m)) < TOL["f64"]
     mm.mm_destroy(ctx)
+
+
+# FP64: three kernels in place of the plane kernel (few planes; z lengths 4 and
+# 8, every padded y length, up to 64 cells in x) and the sizes beside the line
+FEW = [(2, 100, 2), (4, 64, 2), (5, 61, 2), (8, 33, 4), (3, 32, 4), (16, 200, 2), (20, 160, 4), (33, 96, 4), (64, 256, 2),
+       (64, 48, 4), (50, 190, 2), (12, 512, 4), (6, 330, 4), (64, 512, 4), (65, 64, 4), (64, 31, 2), (2, 2, 2), (2, 2, 4)]
+# short x and y lengths, strips of three cells on both sides of their line
+STRIPS = [(4, 3, 128), (8, 4, 1), (3, 5, 1), (3, 128, 64), (3, 256, 128), (256, 3, 64), (256, 3, 256), (3, 64, 16), (128, 3, 8)]
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("n", FEW + STRIPS, ids=lambda n: "x".join(map(str, n)))
+def test_demag_on_narrow_meshes(n, prec):
+    m = wl.random_unit(n, seed=sum(n))
+    ctx = context(n, prec)
+    md = dev(m, prec)
+    H = torch.full_like(md, float("nan"))
+    mm.mm_demag_field(ctx, md, H)
+    assert rel(H, micromag.Problem(n, D).demag_fft(m)) < TOL[prec]
+    mm.mm_destroy(ctx)
+
+
+def demag_time(n, prec):
+    """Median time of one field, in us, over runs of about 5 ms."""
+    ctx = context(n, prec)
+    m = dev(wl.random_unit(n, seed=1), prec)
+    H = torch.empty_like(m)
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    times, reps = [], 4
+    for k in range(8):
+        a.record()
+        for _ in range(reps):
+            mm.mm_demag_field(ctx, m, H)
+        b.record()
+        torch.cuda.synchronize()
+        us = a.elapsed_time(b) * 1e3 / reps
+        if k < 3:
+            reps = max(2, min(200, int(5e3 / us)))
+        else:
+            times.append(us)
+    mm.mm_destroy(ctx)
+    return sorted(times)[len(times) // 2]
+
+
+# (narrow mesh, wider mesh, share of its time): an eighth of the columns may cost
+# half; three cells may cost what four do
+@pytest.mark.parametrize("prec,n,wide,share", [
+    ("f64", (16, 512, 4), (128, 512, 4), 0.5), ("f64", (2, 256, 4), (128, 256, 4), 0.5), ("f64", (3, 512, 512), (4, 512, 512), 1.05),
+    ("f64", (512, 3, 256), (512, 4, 256), 1.05), ("f32", (512, 3, 512), (512, 4, 512), 1.05)])
+def test_a_narrow_mesh_costs_less_than_a_wide_one(prec, n, wide, share):
+    assert demag_time(n, prec) < share * demag_time(wide, prec)
