@@ -170,9 +170,15 @@ int launch_ff_plane(mm_ctx* ctx, ffc* buf, const ffc* tw) {
 }  // namespace
 
 // whether the float-float plane kernel takes this mesh: the Stockham stages
-// need 3 nz P / 8 threads, and 384 leave the z phase its 168 registers
+// need 3 nz P / 8 threads, and 384 leave the z phase its 168 registers.  At
+// four layers and that size a block fills an SM for longer than the five
+// passes take once there are more than two planes an SM (512x128x4 170 us
+// against 177; 256x128x4 113 against 92).
 bool plane_ff_fits(const mm_ctx* ctx) {
-    return ctx->plane.on && ctx->nz <= 4 && 3 * ctx->nz * ctx->plane.P <= 8 * kPlaneThreads && ctx->nx % 2 == 0;
+    const PlanePlan& p = ctx->plane;
+    const int work = 3 * ctx->nz * p.P;
+    if (!p.on || ctx->nz > 4 || ctx->nx % 2 || work > 8 * kPlaneThreads) return false;
+    return ctx->nz < 4 || work <= 4 * kPlaneThreads || p.K <= 2 * 152;
 }
 
 int plane_apply_ff(mm_ctx* ctx, const double* m, const double* Ms, double ms, double* H) {

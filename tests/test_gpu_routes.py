@@ -121,6 +121,19 @@ def test_demag_on_narrow_meshes(n, prec):
     mm.mm_destroy(ctx)
 
 
+@pytest.mark.parametrize("n", [(2, 2, 1), (2, 4, 4), (4, 2, 2), (16, 512, 2), (32, 256, 4), (512, 128, 4), (256, 128, 4)],
+                         ids=lambda n: "x".join(map(str, n)))
+def test_float_float_on_narrow_and_wide_meshes(n):
+    m = wl.random_unit(n, seed=sum(n))
+    ctx = context(n, "f64")
+    mm.mm_set_fft_mode(ctx, mm.MM_FFT_FF)
+    md = dev(m, "f64")
+    H = torch.full_like(md, float("nan"))
+    mm.mm_demag_field(ctx, md, H)
+    assert rel(H, micromag.Problem(n, D).demag_fft(m)) < TOL["f64"]
+    mm.mm_destroy(ctx)
+
+
 def demag_time(n, prec):
     """Median time of one field, in us, over runs of about 5 ms."""
     ctx = context(n, prec)
