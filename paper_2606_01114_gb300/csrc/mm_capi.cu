@@ -87,8 +87,7 @@ KernelTimer::~KernelTimer() {
 
 namespace {
 
-// nx, ny: any size up to 512 (powers of two take the fast passes, other
-// sizes a direct DFT); nz: 1 or a power of two (the z pass is radix-2)
+// nx, ny: any size up to 512; nz: 1 or a power of two (the z pass is radix-2)
 bool valid_n(int n) { return n >= 1 && n <= 512; }
 bool valid_nz(int n) { return valid_n(n) && (n & (n - 1)) == 0; }
 bool valid_len(double d) { return std::isfinite(d) && d > 0.0; }
@@ -113,28 +112,18 @@ void free_all(mm_ctx* ctx) {
     ctx->ev_pool.clear();
 }
 
-// exp(-2 pi i m / L) for m < L, computed in long double and rounded
-void twiddles(int L, std::vector<double>& out) {
-    const long double pi = 3.141592653589793238462643383279502884L;
-    for (int m = 0; m < L; ++m) {
-        long double a = 2.0L * pi * (long double)m / (long double)L;
-        out.push_back((double)cosl(a));
-        out.push_back((double)-sinl(a));
-    }
-}
-
 int make_tables(mm_ctx* ctx) {
     std::vector<double> t;
-    ctx->tw.off_lx = 0;
-    twiddles(ctx->Lx, t);
-    ctx->tw.off_px = (long)t.size() / 2;
-    twiddles(ctx->Px, t);
-    ctx->tw.off_py = (long)t.size() / 2;
-    twiddles(ctx->Py, t);
-    ctx->tw.off_pz = (long)t.size() / 2;
-    twiddles(ctx->Pz, t);
+    const int len[4] = {ctx->Lx, ctx->Px, ctx->Py, ctx->Pz};
+    long* const off[4] = {&ctx->tw.off_lx, &ctx->tw.off_px, &ctx->tw.off_py, &ctx->tw.off_pz};
+    unit_circle(ctx, ctx->Px);       // before Lx, which it gives
+    for (int q = 0; q < 4; ++q) {
+        *off[q] = (long)t.size() / 2;
+        const std::vector<double>& c = unit_circle(ctx, len[q]);
+        t.insert(t.end(), c.begin(), c.end());
+    }
     ctx->tw.off_z4 = (long)t.size() / 2;
-    four_step_table(ctx->Pz, true, t);
+    four_step_table(ctx, ctx->Pz, true, t);
     ctx->tw.len = (long)t.size() / 2;
     MM_CUDA_CHECK(ctx, cudaMalloc(&ctx->tw.f64, t.size() * sizeof(double)));
     MM_CUDA_CHECK(ctx, cudaMemcpy(ctx->tw.f64, t.data(), t.size() * sizeof(double), cudaMemcpyHostToDevice));
@@ -147,6 +136,34 @@ int make_tables(mm_ctx* ctx) {
 }
 
 }  // namespace
+
+const std::vector<double>& unit_circle(mm_ctx* ctx, int len) {
+    for (const auto& e : ctx->circles)
+        if (e.first == len) return e.second;
+    std::vector<double> c;
+    c.reserve(2 * (size_t)len);
+    const std::vector<double>* wide = nullptr;
+    int step = 1;
+    for (const auto& e : ctx->circles)
+        for (int s = 2; len * s <= e.first; s *= 2)
+            if (len * s == e.first) {
+                wide = &e.second;
+                step = s;
+            }
+    const long double pi = 3.141592653589793238462643383279502884L;
+    for (int m = 0; m < len; ++m) {
+        if (wide) {
+            c.push_back((*wide)[2 * (size_t)m * step]);
+            c.push_back((*wide)[2 * (size_t)m * step + 1]);
+        } else {
+            const long double a = 2.0L * pi * (long double)m / (long double)len;
+            c.push_back((double)cosl(a));
+            c.push_back((double)-sinl(a));
+        }
+    }
+    ctx->circles.emplace_back(len, std::move(c));
+    return ctx->circles.back().second;
+}
 
 int dev_alloc(mm_ctx* ctx, void** p, size_t bytes) {
     cudaError_t e = cudaMalloc(p, bytes);
@@ -338,14 +355,16 @@ int mm_init_mesh(mm_ctx** out, int nx, int ny, int nz, double dx, double dy, dou
         reset_ctl(ctx->ctl_host, 0.0, 1e-14, std::numeric_limits<double>::infinity(), 1e-5);
         rc = push_ctl(ctx);
     }
-    // meshes with a side that is not a power of two need the [c][z][y][kx]
-    // arrays only in the fft modes; plane_setup fills the octant of their 2n
-    // lengths
+    // Contexts of the plane layout need the arrays of the [c][z][y][kx] passes
+    // only in the fft modes; the octant of the 2n lengths comes from those
+    // passes' setup where the sides are powers of two, else from plane_setup.
     auto p2 = [](int n) { return (n & (n - 1)) == 0; };
     if (rc == MM_OK) rc = plane_plan(ctx);
-    if (rc == MM_OK && (!ctx->plane.on || (p2(nx) && p2(ny)))) rc = classic_prepare(ctx);
+    if (rc == MM_OK && !ctx->plane.on) rc = classic_prepare(ctx);
+    if (rc == MM_OK && ctx->plane.on && p2(nx) && p2(ny)) rc = octant_prepare(ctx);
     if (rc == MM_OK && ctx->plane.on) rc = plane_setup(ctx);
     if (rc == MM_OK) rc = sync(ctx);
+    ctx->circles.clear();
     if (rc != MM_OK) {
         g_init_error = ctx->err;
         free_all(ctx);

@@ -1946,6 +1946,8 @@ __global__ void k_split_ff(const double* __restrict__ in, ff* __restrict__ out, 
 bool plane_ff_fits(const mm_ctx* ctx);
 int demag_prepare_ff(mm_ctx* ctx) {
     if (plane_ff_fits(ctx)) return plane_prepare_ff(ctx);
+    int rc = classic_prepare(ctx);
+    if (rc) return rc;
     if (ctx->kern_ff && ctx->tw.ff) return MM_OK;
     const long nk = 6L * ctx->Pz2 * ctx->Py2 * ctx->Hs;
     const long nt = 2L * ctx->tw.len;                         // doubles in the twiddle table
@@ -2051,16 +2053,23 @@ int demag_setup(mm_ctx* ctx) {
     return ctx->prec == MM_F64 ? setup<double>(ctx) : setup<float>(ctx);
 }
 
+int octant_prepare(mm_ctx* ctx) {
+    if (ctx->kern_ready) return MM_OK;
+    const size_t e = ctx->prec == MM_F64 ? sizeof(double) : sizeof(float);
+    int rc;
+    if (!ctx->kern && (rc = dev_alloc(ctx, &ctx->kern, 6 * (size_t)ctx->Pz2 * ctx->Py2 * ctx->Hs * e))) return rc;
+    if ((rc = blue_prepare(ctx)) || (rc = demag_setup(ctx))) return rc;
+    ctx->kern_ready = true;
+    return MM_OK;
+}
+
 int classic_prepare(mm_ctx* ctx) {
     if (ctx->classic_ready) return MM_OK;
     const size_t e = ctx->prec == MM_F64 ? sizeof(double) : sizeof(float);
     int rc;
-    if (!ctx->kern && (rc = dev_alloc(ctx, &ctx->kern, 6 * (size_t)ctx->Pz2 * ctx->Py2 * ctx->Hs * e))) return rc;
     if (!ctx->bufA && (rc = dev_alloc(ctx, &ctx->bufA, 3 * (size_t)ctx->nz * ctx->ny * ctx->Hs * 2 * e))) return rc;
     if (!ctx->bufB && (rc = dev_alloc(ctx, &ctx->bufB, 3 * (size_t)ctx->nz * ctx->Py * ctx->Hs * 2 * e))) return rc;
-    if ((rc = blue_prepare(ctx))) return rc;
-    if (!ctx->kern_ready && (rc = demag_setup(ctx))) return rc;
-    ctx->kern_ready = true;
+    if ((rc = blue_prepare(ctx)) || (rc = octant_prepare(ctx))) return rc;
     ctx->classic_ready = true;
     return MM_OK;
 }

@@ -166,6 +166,7 @@ struct mm_ctx {
     int xtma_grid;            // its persistent grid
 
     mm::PlanePlan plane;
+    std::vector<std::pair<int, std::vector<double>>> circles;   // unit_circle
     bool kern_ready;          // kern holds the octant (from mm_init_mesh on)
     bool classic_ready;       // bufA, bufB and the transform tables of the [c][z][y][kx] passes exist
 
@@ -293,9 +294,11 @@ int tc_prepare(mm_ctx* ctx);
 
 // ----- demag (mm_demag.cu)
 int demag_setup(mm_ctx* ctx);                          // K1: Newell tensor -> k-space octant
-// kern, bufA, bufB and tables of the [c][z][y][kx] passes: in mm_init_mesh for
-// power-of-two meshes and those that run them, else when an fft mode that
-// needs them is set (kern exists from mm_init_mesh on)
+// the octant of the [c][z][y][kx] passes (kern)
+int octant_prepare(mm_ctx* ctx);
+// kern, bufA, bufB and tables of those passes: in mm_init_mesh for contexts
+// that run them, else when an fft mode that needs them is set (kern exists
+// from mm_init_mesh on)
 int classic_prepare(mm_ctx* ctx);
 // plane layout (mm_plane.cu): chooses and allocates the plan, fills its octant
 int plane_plan(mm_ctx* ctx);
@@ -312,9 +315,14 @@ int plane_xfwd(mm_ctx* ctx, const void* m);
 int plane_yzy(mm_ctx* ctx);
 int plane_stage(mm_ctx* ctx, int method, int s, const void* m_in, const void* m0, void* m_out, void* hd, bool forward);
 int plane_field(mm_ctx* ctx, const void* m, void* H);
+// exp(-2 pi i m / len), m < len, re and im alternating, in long double and
+// rounded.  Kept on the context while it is created: on the host of a GB300
+// long double is software arithmetic, and the passes of one mesh share lengths
+// (a table of len 2^k gives len's, bit for bit).
+const std::vector<double>& unit_circle(mm_ctx* ctx, int len);
 // appends the four-step tables w^(t k1), [k1][t] and then [t][k1], of an x or
 // y length (or a z length) of mm_plane_launch.cuh; nothing for other lengths
-void four_step_table(int len, bool z, std::vector<double>& out);
+void four_step_table(mm_ctx* ctx, int len, bool z, std::vector<double>& out);
 int dev_alloc(mm_ctx* ctx, void** p, size_t bytes);
 int demag_apply(mm_ctx* ctx, const void* m, void* H);  // K2..K6
 int demag_apply_unit(mm_ctx* ctx, const void* g, void* H);  // same with Ms = 1 (adjoint)

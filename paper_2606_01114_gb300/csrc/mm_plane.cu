@@ -103,15 +103,6 @@ size_t elem(const mm_ctx* ctx) { return ctx->prec == MM_F64 ? 8 : 4; }
 long kern_count(const mm_ctx* ctx) { return (long)ctx->plane.K * 6 * ctx->Pz2 * ctx->plane.KQ; }
 long tw_count(const mm_ctx* ctx) { return 2 * ctx->plane.tw_len; }
 
-void table(int L, std::vector<double>& out) {
-    const long double pi = 3.141592653589793238462643383279502884L;
-    for (int m = 0; m < L; ++m) {
-        const long double a = 2.0L * pi * (long double)m / (long double)L;
-        out.push_back((double)cosl(a));
-        out.push_back((double)-sinl(a));
-    }
-}
-
 }  // namespace
 
 // Which contexts run in the plane layout: every mesh with nx, ny > 1 and a
@@ -159,15 +150,16 @@ int plane_plan(mm_ctx* ctx) {
     p.off_y = p.off_p + 2 * p.L;
     p.off_z = p.off_y + p.P;
     std::vector<double> t;
-    table(p.L, t);
-    table(2 * p.L, t);
-    table(p.P, t);
-    table(ctx->Pz, t);
+    unit_circle(ctx, 2 * p.L);       // before L, which it gives
+    for (int len : {p.L, 2 * p.L, p.P, ctx->Pz}) {
+        const std::vector<double>& c = unit_circle(ctx, len);
+        t.insert(t.end(), c.begin(), c.end());
+    }
     long* const off4[3] = {&p.off_x4, &p.off_y4, &p.off_z4};
     const int len4[3] = {p.L, p.P, ctx->Pz};
     for (int a = 0; a < 3; ++a) {
         *off4[a] = (long)t.size() / 2;
-        four_step_table(len4[a], a == 2, t);
+        four_step_table(ctx, len4[a], a == 2, t);
     }
     p.tw_len = (long)t.size() / 2;
     int rc;
@@ -222,8 +214,7 @@ int plane_setup(mm_ctx* ctx) {
     for (int q = 0; q < sets; ++q)
         for (int a = 0; a < 3; ++a) {
             off[q][a] = (long)t.size();
-            std::vector<double> e;
-            table(len[q][a], e);
+            const std::vector<double>& e = unit_circle(ctx, len[q][a]);
             for (int s = 0; s < 2; ++s)
                 for (int i = 0; i < len[q][a]; ++i) t.push_back(s ? -e[2 * i + 1] : e[2 * i]);   // cos, then sin
         }

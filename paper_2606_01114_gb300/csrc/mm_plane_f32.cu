@@ -8,15 +8,14 @@ int plane_yzy_f32(mm_ctx* ctx);
 
 int plane_line_len(int P) { return plane_line(P); }
 
-void four_step_table(int len, bool z, std::vector<double>& out) {
-    const long double pi = 3.141592653589793238462643383279502884L;
+void four_step_table(mm_ctx* ctx, int len, bool z, std::vector<double>& out) {
+    const std::vector<double>& c = unit_circle(ctx, len);
     auto put = [&](int L1, int L2) {
         for (int turn = 0; turn < 2; ++turn)
             for (int q = 0; q < len; ++q) {
-                const int t = turn ? q / L1 : q % L2, k1 = turn ? q % L1 : q / L2;
-                const long double a = 2.0L * pi * (long double)(t * k1) / (long double)len;
-                out.push_back((double)cosl(a));
-                out.push_back((double)-sinl(a));
+                const int t = turn ? q / L1 : q % L2, k1 = turn ? q % L1 : q / L2;   // t k1 < len
+                out.push_back(c[2 * (size_t)(t * k1)]);
+                out.push_back(c[2 * (size_t)(t * k1) + 1]);
             }
     };
     if (z) with_z_length(len, [&](auto A, auto B) { put(decltype(A)::value, decltype(B)::value); });

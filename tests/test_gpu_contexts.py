@@ -54,3 +54,41 @@ def test_first_kspace_product_can_be_captured(n, prec, tol):
     ref = micromag.Problem(n, D).demag_fft(m)
     assert np.linalg.norm(H.double().cpu().numpy() - ref) < tol * np.linalg.norm(ref)
     mm.mm_destroy(ctx)
+
+
+# a plain context of the plane layout holds its state arrays (11 vector fields,
+# Ms, A), the octant of the 2n lengths, and the planes, octant and line buffer
+# of its passes; not the arrays of passes it does not run
+@pytest.mark.parametrize("n", [(512, 512, 4), (256, 256, 4)], ids=lambda n: "x".join(map(str, n)))
+def test_device_memory_of_a_plain_context(n):
+    nx, ny, nz = n
+    N, P, K, Hs = nx * ny * nz, 2 * ny, nx + 1, (nx + 16) // 16 * 16
+    octants = 6 * (nz + 1) * (ny + 1) * Hs + K * 6 * (nz + 1) * ((P // 2 + 4) // 4 * 4)
+    want = 4 * (35 * N + octants + 2 * K * 3 * nz * ny)
+    warm = mm.mm_init_mesh(*n, *D, precision=mm.MM_F32)      # the library's own modules and streams
+    mm.mm_destroy(warm)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    ctx = mm.mm_init_mesh(*n, *D, precision=mm.MM_F32)
+    torch.cuda.synchronize()
+    used = free - torch.cuda.mem_get_info()[0]
+    mm.mm_destroy(ctx)
+    assert want < used < want + 20 * 2 ** 21      # allocations come in granules of 2 MB
+
+
+def test_modes_after_a_plain_context_allocate_what_they_need():
+    """Power-of-two meshes of the plane layout: the tensor-core mode and the
+    float-float mode of a mesh too large for its plane kernel run the passes
+    whose arrays a plain context does not hold; switching back restores it."""
+    for n, prec, mode, tol in (((64, 256, 2), "f32", mm.MM_TC_TF32, 1e-5), ((32, 256, 4), "f64", mm.MM_FFT_FF, 1e-12)):
+        m = wl.random_unit(n, seed=2)
+        ref = micromag.Problem(n, D).demag_fft(m)
+        ctx = mm.mm_init_mesh(*n, *D, precision=mm.MM_F64 if prec == "f64" else mm.MM_F32)
+        mm.mm_set_material(ctx, 8e5, 1.3e-11, 0.02, 0.0)
+        md = torch.tensor(m, dtype=torch.float64 if prec == "f64" else torch.float32, device="cuda")
+        H = torch.empty_like(md)
+        for k in (mode, 0, mode):
+            mm.mm_set_fft_mode(ctx, k)
+            mm.mm_demag_field(ctx, md, H)
+            assert np.linalg.norm(H.double().cpu().numpy() - ref) < tol * np.linalg.norm(ref)
+        mm.mm_destroy(ctx)
