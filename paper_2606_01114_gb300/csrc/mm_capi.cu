@@ -447,7 +447,7 @@ int mm_effective_field(mm_ctx* ctx, const void* m, void* H) {
     if (!ctx) return fail(nullptr, MM_ERR_INVALID_ARG, "ctx is NULL");
     MM_BIND(ctx);
     if (!m || !H) return fail(ctx, MM_ERR_INVALID_ARG, "m and H must be device pointers");
-    if (plane_fused(ctx)) return plane_field(ctx, m, H);
+    if (plane_fused(ctx, true)) return plane_field(ctx, m, H);
     int rc = demag_apply(ctx, m, ctx->Hd);
     if (rc) return rc;
     bool done = false;

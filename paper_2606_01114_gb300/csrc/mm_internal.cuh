@@ -87,6 +87,8 @@ struct Blue {
 // The plane-layout demag path (mm_plane.cu).  Lengths are padded to the next
 // of 8, 16, 32 and {4, 5, 6} 2^k (k >= 3) >= 2n, so they differ from ctx->Px,
 // Py when a side is not a power of two, or below 4.
+constexpr int kSMs = 152;   // of the one GPU this library is built for
+
 struct PlanePlan {
     int on = 0;          // the plain (fft_mode 0) and float-float passes run in the plane layout
     int lines = 0;       // y, z, y as three kernels: planes too large for one block, or too few (FP64)
@@ -310,7 +312,8 @@ int plane_prepare_ff(mm_ctx* ctx);
 // whether the context's current mode takes it.  plane_stage runs Runge-Kutta
 // stage s on the planes that plane_yzy left and, with `forward`, leaves the
 // planes of m_out for the next plane_yzy; hd (or NULL) receives the demag field.
-bool plane_fused(const mm_ctx* ctx);
+// (field: the effective field alone)
+bool plane_fused(const mm_ctx* ctx, bool field = false);
 int plane_xfwd(mm_ctx* ctx, const void* m);
 int plane_yzy(mm_ctx* ctx);
 int plane_stage(mm_ctx* ctx, int method, int s, const void* m_in, const void* m0, void* m_out, void* hd, bool forward);

@@ -732,7 +732,7 @@ __global__ void k_finite(long n3, const T* __restrict__ m, Control* ctl) {
 // kernels always do: a sub-partition issues one FP64 warp instruction per 64
 // cycles, and small blocks spread the warps evenly over the 608 of them.
 constexpr int kThreads = 256;
-inline int threads_for(long n, size_t elem) { return n < 152L * 2 * kThreads || elem == 8 ? 64 : kThreads; }
+inline int threads_for(long n, size_t elem) { return n < 2L * kSMs * kThreads || elem == 8 ? 64 : kThreads; }
 inline unsigned blocks_for(long n, int threads = kThreads) { return (unsigned)((n + threads - 1) / threads); }
 
 // ------------------------------------------------ Barzilai-Borwein minimiser
@@ -933,7 +933,7 @@ int energy_t(mm_ctx* ctx, const void* m, const void* Hd) {
     KernelTimer kt(ctx, MM_K_REDUCE);
     Params<T> p = make_params<T>(ctx);
     double V = ctx->dx * ctx->dy * ctx->dz;
-    const unsigned nb = std::min(blocks_for(p.N, kReduceThreads), 152u * 8);
+    const unsigned nb = std::min(blocks_for(p.N, kReduceThreads), 8u * kSMs);
     dep(k_energy<T>, nb, kReduceThreads, 0, ctx->stream)(p, (const T*)m, (const T*)Hd, V, kMu0, ctx->Ku, ctx->ctl);
     MM_LAUNCH_CHECK(ctx);
     return MM_OK;
@@ -1020,7 +1020,7 @@ int bb_iteration(mm_ctx* ctx, void* m, void* g, const void* g_prev, void* m_prev
 int check_finite_launch(mm_ctx* ctx, const void* m) {
     KernelTimer kt(ctx, MM_K_REDUCE);
     const long n3 = 3 * ctx->N;
-    const unsigned nb = std::min(blocks_for(n3, 4 * kThreads), 152u * 8);
+    const unsigned nb = std::min(blocks_for(n3, 4 * kThreads), 8u * kSMs);
     if (ctx->prec == MM_F64)
         dep(k_finite<double>, nb, kThreads, 0, ctx->stream)(n3, (const double*)m, ctx->ctl);
     else

@@ -110,11 +110,11 @@ long tw_count(const mm_ctx* ctx) { return 2 * ctx->plane.tw_len; }
 // lines of the padded y length) fits one block's shared memory with a z
 // transform that fits a thread's registers (nz <= 8; FP64 and float-float 4).
 // Power-of-two meshes also need two blocks per SM (113 KB a plane) or no more
-// planes than SMs; at one block per SM over several waves the five streaming
-// passes are the faster: 512x512x8 FP32 169 against 185 us, 512x512x4 FP64
-// 1804 against 1826 us.  On the near side of the line: 512x512x4 FP32 85
-// against 96 us, 64x512x8 (65 planes) 40 against 43 us, 256x256x8 44 against
-// 56 us.
+// than two planes an SM; at one block per SM over more waves the five streaming
+// passes are at least as fast: 512x512x8 FP32 153 against 157 us, 512x512x4 FP64
+// 1797 against 1795.  On the near side of the line: 256x512x8 FP32 (257 planes)
+// 69 against 83 us, 256x512x4 FP64 875 against 962, 64x512x8 29 against 43;
+// with two blocks per SM 512x512x4 FP32 61 against 94, 256x256x8 31 against 56.
 // The plane is a block's serial work, so few planes of many values leave most
 // SMs idle.  In FP64 (one warp instruction per sub-partition and 64 cycles) that
 // counts more than the two passes over memory it saves: up to 65 planes of nz P >= 256
@@ -138,7 +138,7 @@ int plane_plan(mm_ctx* ctx) {
     const bool regular = pow2(ctx->nx) && pow2(ctx->ny);
     const size_t smem = 3 * (size_t)ctx->nz * plane_line_len(p.P) * cs;
     const bool fits = ctx->nz <= (ctx->prec == MM_F32 ? 8 : 4) && smem <= 227 * 1024;
-    if (regular && (!fits || (smem > 113 * 1024 && p.L + 1 > 152))) return MM_OK;
+    if (regular && (!fits || (smem > 113 * 1024 && p.L + 1 > 2 * kSMs))) return MM_OK;
     const bool strip = (ctx->nx == 3 && pow2(ctx->ny)) || (ctx->ny == 3 && pow2(ctx->nx));
     if (strip && (ctx->prec == MM_F64 ? ctx->N >= 98304 : ctx->ny == 3 && ctx->N >= 196608)) return MM_OK;
     p.on = 1;

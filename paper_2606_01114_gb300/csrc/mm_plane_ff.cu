@@ -178,7 +178,7 @@ bool plane_ff_fits(const mm_ctx* ctx) {
     const PlanePlan& p = ctx->plane;
     const int work = 3 * ctx->nz * p.P;
     if (!p.on || ctx->nz > 4 || ctx->nx % 2 || work > 8 * kPlaneThreads) return false;
-    return ctx->nz < 4 || work <= 4 * kPlaneThreads || p.K <= 2 * 152;
+    return ctx->nz < 4 || work <= 4 * kPlaneThreads || p.K <= 2 * kSMs;
 }
 
 int plane_apply_ff(mm_ctx* ctx, const double* m, const double* Ms, double ms, double* H) {
@@ -189,7 +189,7 @@ int plane_apply_ff(mm_ctx* ctx, const double* m, const double* Ms, double ms, do
     const int lgL = ilog2(p.L);
     // 64-byte segments per plane (8 rows of short lines); 32-byte ones while the
     // larger blocks are too few to share the SMs evenly (256x256x1: 192 blocks)
-    const int lgB = lgL < 6 ? 3 : rows < 16 * 152 ? 1 : 2;
+    const int lgB = lgL < 6 ? 3 : rows < 16 * kSMs ? 1 : 2;
     const int nt = ((1 << (lgL + lgB - 3)) + 31) / 32 * 32;
     const size_t smem = sizeof(ffc) << (lgL + lgB);
     const unsigned nb = (unsigned)((rows + (1 << lgB) - 1) >> lgB);

@@ -106,18 +106,19 @@ int launch_plane(mm_ctx* ctx, PC<T>* buf, const T* kern, const PC<T>* tw) {
             // where that takes every plane into one wave.  Demag, 384 threads
             // -> rule: 256x256x4 20.9 -> 19.1 us, 512x512x4 64.9 -> 61.4,
             // 256x256x8 33.6 -> 30.6, 300x300x2 21.8 -> 19.0 (96 threads: 20.8);
-            // 64x512x8 (65 planes) 29.3 at 384, 35.9 at 192.
+            // 64x512x8 (65 planes) 29.3 at 384, 35.9 at 192; 350x350x4 (385
+            // planes, three blocks of 128 on an SM's 228 KB) 36.5 -> 34.9.
             auto even = [&](int cap) {
                 const int rounds = (tasks + cap - 1) / cap;
                 return ((tasks + rounds - 1) / rounds + 31) / 32 * 32;
             };
             int nt = even(sizeof(T) == 4 ? 512 : 256);
-            if (sizeof(T) == 4 && p.K > 152) {
+            if (sizeof(T) == 4 && p.K > kSMs) {
                 nt = even(256);
                 for (int cap : {256, 160, 128}) {
                     const int n = std::max(even(cap), std::min(128, nt));
-                    const long fit = std::min<long>(65536 / (128 * n), (227 * 1024) / (long)(smem + 1024));
-                    if (152 * fit >= p.K) {
+                    const long fit = std::min<long>(65536 / (128 * n), (228 * 1024) / (long)(smem + 1024));
+                    if (kSMs * fit >= p.K) {
                         nt = n;
                         break;
                     }
@@ -196,7 +197,7 @@ int launch_zline_t(mm_ctx* ctx, PC<T>* buf, const T* kern, const ZLine& g, int n
     if constexpr (zline_split<T>(PZ)) {
         // one column a block while four of them would leave SMs idle (5x2x512:
         // 264 us a field with four, 18 blocks; 97 with one)
-        if ((long)g.ncol * nrows <= 4 * 152) return launch_zline_b<T, L1, L2, COLY, 1, 96, 1>(ctx, buf, kern, g, nrows, tw);
+        if ((long)g.ncol * nrows <= 4 * kSMs) return launch_zline_b<T, L1, L2, COLY, 1, 96, 1>(ctx, buf, kern, g, nrows, tw);
         return launch_zline_b<T, L1, L2, COLY, 4, 384, 1>(ctx, buf, kern, g, nrows, tw);
     } else {
         constexpr int B = PZ <= 8 ? 32 : PZ <= 64 ? 128 / CS : PZ <= 512 ? 64 / CS : 32 / CS;

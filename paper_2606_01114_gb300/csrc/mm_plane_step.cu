@@ -5,6 +5,25 @@
 namespace mm {
 namespace {
 
+// four rows a block read and write whole 32-byte sectors of the planes; fewer
+// where that leaves SMs idle
+struct CellGrid {
+    int lgB;
+    long blocks;
+};
+CellGrid cell_grid(const mm_ctx* ctx) {
+    const long nrows = (long)ctx->ny * ctx->nz;
+    const int lgB = nrows >= 4 * kSMs ? 2 : nrows >= 2 * kSMs ? 1 : 0;
+    return {lgB, (nrows + (1 << lgB) - 1) >> lgB};
+}
+constexpr int cell_threads(int L1, int L2, CellGrid c) {
+    const int width = (3 << c.lgB) * (L1 > L2 ? L1 : L2);
+    return width > 256 ? (width + 31) / 32 * 32 : 256;
+}
+constexpr size_t cell_smem(int L1, int L2, CellGrid c) {
+    return (size_t)(3 << c.lgB) * (plane_pitch(L1, L2) + 4) * sizeof(float2);
+}
+
 template <bool STAGE>
 int launch_px_cell(mm_ctx* ctx, const float* m_in, float* H, const RkStage<float>& g) {
     const PlanePlan& p = ctx->plane;
@@ -19,22 +38,21 @@ int launch_px_cell(mm_ctx* ctx, const float* m_in, float* H, const RkStage<float
         par.cz = par.A * par.cz * inv;
         par.A = 1.f;
     }
-    const int nrows = ctx->ny * ctx->nz;
-    // four rows a block read and write whole 32-byte sectors of the planes;
-    // fewer where that leaves SMs idle
-    const int lgB = nrows >= 4 * 152 ? 2 : nrows >= 2 * 152 ? 1 : 0;
+    const CellGrid c = cell_grid(ctx);
     int rc = MM_OK;
     KernelTimer kt(ctx, STAGE ? MM_K_STAGE : MM_K_REDUCE);
     if (!with_length(p.L, [&](auto A, auto B) {
             constexpr int L1 = decltype(A)::value, L2 = decltype(B)::value;
             if constexpr (L1 * L2 <= 512) {
-                const int lines = 3 << lgB, width = lines * (L1 > L2 ? L1 : L2);
-                const int nt = width > 256 ? (width + 31) / 32 * 32 : 256;
-                const size_t smem = (size_t)lines * (plane_pitch(L1, L2) + 4) * sizeof(float2);
-                auto fn = k_px_cell<float, L1, L2, STAGE>;
+                const size_t smem = cell_smem(L1, L2, c);
+                auto fn = k_px_cell<float, L1, L2, STAGE, STAGE ? 512 : 384>;
+                // the longest rows lose 3 % to the bound while each block has an SM to itself
+                if constexpr (STAGE && L1 * L2 == 512) {
+                    if (c.blocks <= kSMs) fn = k_px_cell<float, L1, L2, STAGE, 384>;
+                }
                 if ((rc = smem_opt_in(ctx, (const void*)fn, smem))) return;
-                dep(fn, (unsigned)((nrows + (1 << lgB) - 1) >> lgB), nt, smem, ctx->stream)(
-                    (float2*)p.buf, p.R, par, folded, lgB, scale, tw + p.off_x4, tw + p.off_p, m_in, H, g, ctx->ctl);
+                dep(fn, (unsigned)c.blocks, cell_threads(L1, L2, c), smem, ctx->stream)(
+                    (float2*)p.buf, p.R, par, folded, c.lgB, scale, tw + p.off_x4, tw + p.off_p, m_in, H, g, ctx->ctl);
             }
         }))
         rc = fail(ctx, MM_ERR_INVALID_ARG, "x length %d", p.L);
@@ -47,15 +65,23 @@ int launch_px_cell(mm_ctx* ctx, const float* m_in, float* H, const RkStage<float
 
 // Small meshes: four kernels of a stage cost more in gaps, ramps and tails than
 // the fused kernel's lower occupancy in the cell part.  One RK4 stage, four
-// kernels -> two (uniform Ms / Ms per cell): 100x25x1 13.3 -> 9.2 / 16.0 -> 9.4
-// us, 64x64x4 14.0 -> 9.4 / 16.4 -> 10.0, 256x256x1 (66 k cells) 18.2 -> 14.9 /
-// 22.5 -> 15.7; 300x300x2 (180 k) 27.3 -> 27.8 / 31.8 -> 29.4, 256x256x4 (262 k)
-// 25.7 -> 29.4 / 32.2 -> 32.0.  The effective field alone: 11.5 -> 10.2, 12.0 ->
-// 9.9, 16.5 -> 15.0; 25.2 -> 26.3, 23.9 -> 27.6.
+// kernels -> two: 100x25x1 13.0 -> 9.2 us, 64x64x4 13.1 -> 8.4, 256x256x1 (66 k
+// cells) 17.4 -> 13.5, 300x300x1 18.3 -> 15.4, 512x175x1 18.9 -> 17.8, 350x350x1
+// (123 k) 20.1 -> 19.4, 200x200x4 (160 k) 22.6 -> 25.0; with Ms per cell 13.2 ->
+// 8.7, 17.7 -> 13.7, 18.7 -> 15.6, 19.5 -> 18.1, 20.7 -> 19.7, 23.9 -> 25.8.
+// An SM holds two blocks; a second wave of them pays on short rows only:
+// 64x351x4 (351 blocks) 19.3 -> 19.0, but 80x371x4 19.7 -> 21.7.
+// The effective field alone has one kernel fewer to save: 64x351x4 18.8 -> 17.0,
+// 96x309x4 19.0 -> 18.4, 160x140x4 (90 k) 18.2 -> 17.1, 128x468x1 14.7 -> 14.4, but
+// 256x351x1 (90 k) 16.7 -> 18.1, 160x185x4 (118 k) 20.3 -> 21.1, and no mesh of x
+// length 320 and more gains (300x100x1 16.1 -> 16.4, 512x29x1 15.1 -> 16.9).
 constexpr long kFusedCells = 120000;
 
-bool plane_fused(const mm_ctx* ctx) {
-    return ctx->prec == MM_F32 && ctx->plane.on && ctx->fft_mode == 0 && ctx->N <= kFusedCells;
+bool plane_fused(const mm_ctx* ctx, bool field) {
+    const PlanePlan& p = ctx->plane;
+    if (ctx->prec != MM_F32 || !p.on || ctx->fft_mode != 0 || ctx->N > kFusedCells) return false;
+    if (field) return p.L <= 96 || (p.L <= 256 && ctx->N <= (p.L & (p.L - 1) ? 100000 : 85000));
+    return p.L <= 64 || cell_grid(ctx).blocks <= 2 * kSMs;
 }
 
 int plane_stage(mm_ctx* ctx, int method, int s, const void* m_in, const void* m0, void* m_out, void* hd, bool forward) {

@@ -101,6 +101,25 @@ def test_demag_on_the_longest_z_lines_in_double(n):
     mm.mm_destroy(ctx)
 
 
+# both sides of the lines between the fused stage and field and the kernels
+# apart: one and two blocks an SM, one and two waves, x lengths of both kinds
+@pytest.mark.parametrize("n", [(512, 16, 1), (512, 175, 1), (300, 200, 1), (384, 39, 1), (80, 304, 4), (80, 305, 4), (64, 351, 4),
+                               (256, 83, 4), (256, 84, 4), (160, 156, 4), (160, 157, 4), (96, 234, 4), (256, 512, 8)],
+                         ids=lambda n: "x".join(map(str, n)))
+def test_field_and_steps_beside_the_lines(n):
+    out = []
+    for prec in ("f64", "f32"):
+        ctx = context(n, prec)
+        md = dev(wl.random_unit(n, seed=4), prec)
+        H = torch.empty_like(md)
+        mm.mm_effective_field(ctx, md, H)
+        mm.mm_rk4_trajectory(ctx, md, 1e-14, 2)
+        out.append((H.double().cpu().numpy(), md.double().cpu().numpy()))
+        mm.mm_destroy(ctx)
+    for a, b in zip(*out):
+        assert np.linalg.norm(b - a) < TOL["f32"] * np.linalg.norm(a)
+
+
 # FP64: three kernels in place of the plane kernel (few planes; z lengths 4 and
 # 8, every padded y length, up to 64 cells in x) and the sizes beside the line
 FEW = [(2, 100, 2), (4, 64, 2), (5, 61, 2), (8, 33, 4), (3, 32, 4), (16, 200, 2), (20, 160, 4), (33, 96, 4), (64, 256, 2),
