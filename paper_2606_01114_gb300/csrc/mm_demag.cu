@@ -302,7 +302,7 @@ __device__ __forceinline__ void zconv_one(C_t<T>* s, const T* kn, const FftGeom&
 }
 
 template <typename T>
-__global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512)
+__global__ void __launch_bounds__(512)
     k_zconv(C_t<T>* buf, const T* __restrict__ kern, int nz, int lgPz, int Py, int Hs, int Hx, int Py2, int Pz2,
             int lgB, const C_t<T>* __restrict__ twz) {
     dep_wait();
@@ -1272,12 +1272,10 @@ inline int x_rows_per_block(int L) { return clamp_pow2(2048 / L, 4, 64); }
 // columns per block of the y passes: at least 32 bytes of each row, at most
 // 512 active threads
 inline int col_tile(int L, int cs) { return clamp_pow2(4096 / L, 32 / cs, 32); }
-// columns per block of the z pass (three components each): at most 1024
-// (FP32) or 512 (FP64) active threads, at least 32 bytes of each row where
-// that limit allows
-inline int z_tile(int Pz, int cs) {
-    int cap = (cs == 8 ? 8192 : 4096) / (3 * Pz);       // nact = 3 B Pz / 8 <= 1024 or 512
-    int lo = 32 / cs;
+// columns per block of the z pass on 16-byte values (three components each): at
+// most 512 active threads, at least 32 bytes of each row where that limit allows
+inline int z_tile(int Pz) {
+    const int cap = 4096 / (3 * Pz), lo = 2;          // nact = 3 B Pz / 8 <= 512
     int b = Pz >= 8 ? 1024 / Pz : 32;
     if (b > cap) b = cap;
     if (b < lo && lo <= cap) b = lo;
@@ -1655,17 +1653,18 @@ int apply(mm_ctx* ctx, const T* m, T* H, bool unit = false) {
         if (rc) return rc;
     }
     // K4
-    if (sizeof(T) == 4 && ctx->Pz >= 64) {
-        rc = zline_f32(ctx, (float2*)Bf, (const float*)ctx->kern, (const float2*)table<T>(ctx, ctx->tw.off_z4));
-        if (rc) return rc;
-    } else if (sizeof(T) == 4) {
-        KernelTimer kt(ctx, MM_K_ZCONV);
-        rc = launch_zconv_reg(ctx, (float2*)Bf, (const float*)ctx->kern, 0, ctx->Hx);
+    if constexpr (sizeof(T) == 4) {
+        if (ctx->Pz >= 64) {
+            rc = zline_f32(ctx, (float2*)Bf, (const float*)ctx->kern, (const float2*)table<T>(ctx, ctx->tw.off_z4));
+        } else {
+            KernelTimer kt(ctx, MM_K_ZCONV);
+            rc = launch_zconv_reg(ctx, (float2*)Bf, (const float*)ctx->kern, 0, ctx->Hx);
+        }
         if (rc) return rc;
     } else {
         KernelTimer kt(ctx, MM_K_ZCONV);
         const int Pz = ctx->Pz;
-        const int B = z_tile(Pz, sizeof(C));
+        const int B = z_tile(Pz);
         size_t smem = (size_t)3 * Pz * B * sizeof(C) + (size_t)6 * ctx->Pz2 * B * sizeof(T);
         rc = smem_opt_in(ctx, (const void*)k_zconv<T>, smem);
         if (rc) return rc;
@@ -1861,7 +1860,7 @@ int apply_ff(mm_ctx* ctx, const double* m, double* H, bool unit) {
     } else {
         KernelTimer kt(ctx, MM_K_ZCONV);
         const int Pz = ctx->Pz;
-        const int B = z_tile(Pz, sizeof(C));
+        const int B = z_tile(Pz);
         const size_t smem = (size_t)3 * Pz * B * sizeof(C) + (size_t)6 * ctx->Pz2 * B * sizeof(ff);
         if ((rc = smem_opt_in(ctx, (const void*)k_zconv<ff>, smem))) return rc;
         dim3 grid((unsigned)((ctx->Hx + B - 1) / B), (unsigned)(ctx->Py / 2 + 1));

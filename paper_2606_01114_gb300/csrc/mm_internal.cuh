@@ -96,9 +96,9 @@ struct PlanePlan {
     int K = 0;           // planes: L + 1 kept x frequencies
     int KQ = 0;          // octant row stride (P / 2 + 1 rounded up to 4)
     long R = 0;          // plane stride of buf, complex (3 nz ny rounded up to 4)
-    // twiddle tables exp(-2 pi i m / len), natural order: L at 0, then 2L, P,
-    // Pz; behind them the four-step tables ([k1][t], [t][k1]) of L, P and Pz
-    long off_p = 0, off_y = 0, off_z = 0, off_x4 = 0, off_y4 = 0, off_z4 = 0, tw_len = 0;
+    // twiddle tables exp(-2 pi i m / len), natural order: L at 0, then 2L, P;
+    // behind them the four-step tables ([k1][t], [t][k1]) of L, P and Pz
+    long off_p = 0, off_y = 0, off_x4 = 0, off_y4 = 0, off_z4 = 0, tw_len = 0;
     void* buf = nullptr;     // complex [K][R]
     void* buf2 = nullptr;    // complex [K][3 nz][P] (lines)
     void* kern = nullptr;    // octant [K][6][Pz/2+1][KQ], path precision

@@ -148,10 +148,9 @@ int plane_plan(mm_ctx* ctx) {
     p.R = (3L * ctx->nz * ctx->ny + 3) / 4 * 4;
     p.off_p = p.L;
     p.off_y = p.off_p + 2 * p.L;
-    p.off_z = p.off_y + p.P;
     std::vector<double> t;
     unit_circle(ctx, 2 * p.L);       // before L, which it gives
-    for (int len : {p.L, 2 * p.L, p.P, ctx->Pz}) {
+    for (int len : {p.L, 2 * p.L, p.P}) {
         const std::vector<double>& c = unit_circle(ctx, len);
         t.insert(t.end(), c.begin(), c.end());
     }

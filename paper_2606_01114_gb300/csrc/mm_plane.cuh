@@ -8,8 +8,9 @@
 //   k_plane    one block per plane, everything on chip: y forward, z forward,
 //              the 3x3 tensor product, z inverse, y inverse, in place;
 //   k_px_inv   planes back to real rows of H.
-// Planes too large for one block's shared memory (or nz > 8) run y forward,
-// z product and y inverse as three kernels in the same layout (k_py, k_zline).
+// Planes too large for one block's shared memory (or nz > 8), and FP64 planes
+// too few to fill the SMs, run y forward, z product and y inverse as three
+// kernels in the same layout (k_py, k_zline).
 //
 // Lengths.  The convolution is linear, so the padded length P may be any
 // length >= 2n: it is the next of 8 (x: 2 L, L = 4), 16, 32 and {4, 5, 6} 2^k
@@ -39,25 +40,14 @@ template <typename T> using PC = typename cx<T>::type;
 
 constexpr int plane_pitch(int L1, int L2) { return L1 * (L2 + 1); }
 
-// real rows: S is the storage type of m, Ms and H (float, or double for the
-// double and float-float passes)
-template <typename T, typename S> __device__ __forceinline__ T pl_ld(S v) {
-    if constexpr (std::is_same<T, S>::value) return v;
-    else return from_real<T>(v);
-}
-template <typename S, typename T> __device__ __forceinline__ S pl_st(T v) {
-    if constexpr (std::is_same<T, S>::value) return v;
-    else return to_d(v);
-}
-
 // rows per block of the x passes
 template <typename T> constexpr int px_rows(int L) { return L <= 64 ? 8 : 4; }
 constexpr int px_threads(int B, int L1, int L2) { return (B * (L1 > L2 ? L1 : L2) + 31) / 32 * 32; }
 
 // ---------------------------------------------------------------- x forward
-template <typename T, typename S, int L1, int L2>
+template <typename T, int L1, int L2>
 __global__ void __launch_bounds__(px_threads(px_rows<T>(L1 * L2), L1, L2))
-    k_px_fwd(const S* __restrict__ in, int nx, const S* __restrict__ Ms, T ms, long ms_rows, PC<T>* __restrict__ out,
+    k_px_fwd(const T* __restrict__ in, int nx, const T* __restrict__ Ms, T ms, long ms_rows, PC<T>* __restrict__ out,
              long R, long rows, const PC<T>* __restrict__ twL, const PC<T>* __restrict__ twP) {
     dep_wait();
     using C = PC<T>;
@@ -69,11 +59,11 @@ __global__ void __launch_bounds__(px_threads(px_rows<T>(L1 * L2), L1, L2))
         const int t = tid % L2, b = tid / L2;
         const long r = r0 + b;
         const bool act = r < rows;
-        const S* row = in + (act ? r : 0) * nx;
-        const S* mrow = Ms ? Ms + (long)((unsigned)(act ? r : 0) % (unsigned)ms_rows) * nx : nullptr;
+        const T* row = in + (act ? r : 0) * nx;
+        const T* mrow = Ms ? Ms + (long)((unsigned)(act ? r : 0) % (unsigned)ms_rows) * nx : nullptr;
         // pairs in one access where every row starts on a pair boundary (the
         // library's own Ms array always does)
-        const bool even = nx % 2 == 0 && reinterpret_cast<uintptr_t>(in) % (2 * sizeof(S)) == 0;
+        const bool even = nx % 2 == 0 && reinterpret_cast<uintptr_t>(in) % (2 * sizeof(T)) == 0;
         C v[L1], w[L1 / 2];
 #pragma unroll
         for (int n1 = 0; n1 < L1 / 2; ++n1) {
@@ -82,16 +72,12 @@ __global__ void __launch_bounds__(px_threads(px_rows<T>(L1 * L2), L1, L2))
             w[n1] = cmk<C>(ms, ms);
             if (act && x < nx) {
                 if (even) {
-                    const PC<S> q = *reinterpret_cast<const PC<S>*>(row + x);
-                    v[n1] = cmk<C>(pl_ld<T>(q.x), pl_ld<T>(q.y));
-                    if (mrow) {
-                        const PC<S> u = *reinterpret_cast<const PC<S>*>(mrow + x);
-                        w[n1] = cmk<C>(pl_ld<T>(u.x), pl_ld<T>(u.y));
-                    }
+                    v[n1] = *reinterpret_cast<const C*>(row + x);
+                    if (mrow) w[n1] = *reinterpret_cast<const C*>(mrow + x);
                 } else {
                     const bool two = x + 1 < nx;
-                    v[n1] = cmk<C>(pl_ld<T>(row[x]), two ? pl_ld<T>(row[x + 1]) : (T)0);
-                    if (mrow) w[n1] = cmk<C>(pl_ld<T>(mrow[x]), two ? pl_ld<T>(mrow[x + 1]) : (T)0);
+                    v[n1] = cmk<C>(row[x], two ? row[x + 1] : (T)0);
+                    if (mrow) w[n1] = cmk<C>(mrow[x], two ? mrow[x + 1] : (T)0);
                 }
             }
         }
@@ -135,9 +121,9 @@ __global__ void __launch_bounds__(px_threads(px_rows<T>(L1 * L2), L1, L2))
 }
 
 // ---------------------------------------------------------------- x inverse
-template <typename T, typename S, int L1, int L2>
+template <typename T, int L1, int L2>
 __global__ void __launch_bounds__(px_threads(px_rows<T>(L1 * L2), L1, L2))
-    k_px_inv(const PC<T>* __restrict__ in, long R, S* __restrict__ out, int nx, long rows, T scale,
+    k_px_inv(const PC<T>* __restrict__ in, long R, T* __restrict__ out, int nx, long rows, T scale,
              const PC<T>* __restrict__ twL, const PC<T>* __restrict__ twP) {
     dep_wait();
     using C = PC<T>;
@@ -186,17 +172,16 @@ __global__ void __launch_bounds__(px_threads(px_rows<T>(L1 * L2), L1, L2))
         dif<L2, +1, false>(u);
         const long r = r0 + b;
         if (r < rows) {
-            S* row = out + r * nx;
-            const bool even = nx % 2 == 0 && reinterpret_cast<uintptr_t>(out) % (2 * sizeof(S)) == 0;
+            T* row = out + r * nx;
+            const bool even = nx % 2 == 0 && reinterpret_cast<uintptr_t>(out) % (2 * sizeof(T)) == 0;
 #pragma unroll
             for (int k2 = 0; k2 < L2 / 2; ++k2) {
                 const C z = u[dif_pos<L2>(k2)];
                 const int x = 2 * (k1 + L1 * k2);
-                const S a = pl_st<S>(z.x * scale), c = pl_st<S>(z.y * scale);
+                const T a = z.x * scale, c = z.y * scale;
                 if (x + 1 < nx) {
                     if (even) {
-                        using S2 = PC<S>;
-                        *reinterpret_cast<S2*>(row + x) = cmk<S2>(a, c);
+                        *reinterpret_cast<C*>(row + x) = cmk<C>(a, c);
                     } else {
                         row[x] = a;
                         row[x + 1] = c;

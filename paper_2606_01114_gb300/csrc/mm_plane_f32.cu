@@ -23,7 +23,7 @@ void four_step_table(mm_ctx* ctx, int len, bool z, std::vector<double>& out) {
 }
 
 int plane_xfwd_f32(mm_ctx* ctx, const float* m, const float* Ms, float ms) {
-    return launch_px_fwd<float, float>(ctx, m, Ms, ms, (long)ctx->nz * ctx->ny, (float2*)ctx->plane.buf,
+    return launch_px_fwd<float>(ctx, m, Ms, ms, (long)ctx->nz * ctx->ny, (float2*)ctx->plane.buf,
                                        3L * ctx->nz * ctx->ny, (const float2*)ctx->plane.tw);
 }
 
@@ -32,7 +32,7 @@ int plane_apply_f32(mm_ctx* ctx, const float* m, const float* Ms, float ms, floa
     int rc = plane_xfwd_f32(ctx, m, Ms, ms);
     if (rc || (rc = plane_yzy_f32(ctx))) return rc;
     const float scale = (float)(1.0 / ((double)p.L * p.P * ctx->Pz));
-    return launch_px_inv<float, float>(ctx, (const float2*)p.buf, H, 3L * ctx->nz * ctx->ny, scale, (const float2*)p.tw);
+    return launch_px_inv<float>(ctx, (const float2*)p.buf, H, 3L * ctx->nz * ctx->ny, scale, (const float2*)p.tw);
 }
 
 }  // namespace mm

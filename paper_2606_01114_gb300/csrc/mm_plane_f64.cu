@@ -27,10 +27,10 @@ int plane_apply_f64(mm_ctx* ctx, const double* m, const double* Ms, double ms, d
     const bool lite_x = rows * p.L <= kLiteX;
     const bool lite_yz = ctx->nz == 1 && !p.lines && 3L * p.K * p.P <= kLitePlane;
     int rc = lite_x ? lite_xfwd(ctx, m, Ms, ms)
-                    : launch_px_fwd<double, double>(ctx, m, Ms, ms, (long)ctx->nz * ctx->ny, buf, rows, tw);
+                    : launch_px_fwd<double>(ctx, m, Ms, ms, (long)ctx->nz * ctx->ny, buf, rows, tw);
     if (rc || (rc = lite_yz ? lite_plane(ctx) : plane_yzy_f64(ctx))) return rc;
     if (lite_x) return lite_xinv(ctx, H);
-    return launch_px_inv<double, double>(ctx, buf, H, rows, 1.0 / ((double)p.L * p.P * ctx->Pz), tw);
+    return launch_px_inv<double>(ctx, buf, H, rows, 1.0 / ((double)p.L * p.P * ctx->Pz), tw);
 }
 
 }  // namespace mm

@@ -48,8 +48,8 @@ inline int plane_line(int P) {
     return lp;
 }
 
-template <typename T, typename S>
-int launch_px_fwd(mm_ctx* ctx, const S* in, const S* Ms, T ms, long ms_rows, PC<T>* out, long rows, const PC<T>* tw) {
+template <typename T>
+int launch_px_fwd(mm_ctx* ctx, const T* in, const T* Ms, T ms, long ms_rows, PC<T>* out, long rows, const PC<T>* tw) {
     const PlanePlan& p = ctx->plane;
     int rc = MM_OK;
     KernelTimer kt(ctx, MM_K_XFWD);
@@ -57,7 +57,7 @@ int launch_px_fwd(mm_ctx* ctx, const S* in, const S* Ms, T ms, long ms_rows, PC<
             constexpr int L1 = decltype(A)::value, L2 = decltype(B)::value, L = L1 * L2;
             if constexpr (L <= 512) {
                 constexpr int BR = px_rows<T>(L);
-                dep(k_px_fwd<T, S, L1, L2>, (unsigned)((rows + BR - 1) / BR), px_threads(BR, L1, L2), 0, ctx->stream)(
+                dep(k_px_fwd<T, L1, L2>, (unsigned)((rows + BR - 1) / BR), px_threads(BR, L1, L2), 0, ctx->stream)(
                     in, ctx->nx, Ms, ms, ms_rows, out, p.R, rows, tw + p.off_x4, tw + p.off_p);
             }
         }))
@@ -67,8 +67,8 @@ int launch_px_fwd(mm_ctx* ctx, const S* in, const S* Ms, T ms, long ms_rows, PC<
     return MM_OK;
 }
 
-template <typename T, typename S>
-int launch_px_inv(mm_ctx* ctx, const PC<T>* in, S* out, long rows, T scale, const PC<T>* tw) {
+template <typename T>
+int launch_px_inv(mm_ctx* ctx, const PC<T>* in, T* out, long rows, T scale, const PC<T>* tw) {
     const PlanePlan& p = ctx->plane;
     int rc = MM_OK;
     KernelTimer kt(ctx, MM_K_XINV);
@@ -76,7 +76,7 @@ int launch_px_inv(mm_ctx* ctx, const PC<T>* in, S* out, long rows, T scale, cons
             constexpr int L1 = decltype(A)::value, L2 = decltype(B)::value, L = L1 * L2;
             if constexpr (L <= 512) {
                 constexpr int BR = px_rows<T>(L);
-                dep(k_px_inv<T, S, L1, L2>, (unsigned)((rows + BR - 1) / BR), px_threads(BR, L1, L2), 0, ctx->stream)(
+                dep(k_px_inv<T, L1, L2>, (unsigned)((rows + BR - 1) / BR), px_threads(BR, L1, L2), 0, ctx->stream)(
                     in, p.R, out, ctx->nx, rows, scale, tw + p.off_x4, tw + p.off_p);
             }
         }))
