@@ -110,13 +110,13 @@ def load_peaks():
 # the sources each timed kernel family is compiled from: stored ncu traffic
 # stays valid while these files are unchanged
 KERNEL_SOURCES = {
-    "demag": ("mm_demag.cu", "mm_fft.cuh", "mm_regfft.cuh", "mm_ff.cuh", "mm_tma.cuh", "mm_tcgen05.cuh",
-              "mm_internal.cuh"),
-    "stage": ("mm_llg.cu", "mm_fields.cuh", "mm_ff.cuh", "mm_internal.cuh"),
+    "demag": ("mm_demag.cu", "mm_zline.cu", "mm_plane_launch.cuh", "mm_plane.cuh", "mm_fft.cuh", "mm_regfft.cuh",
+              "mm_ff.cuh", "mm_tma.cuh", "mm_tcgen05.cuh", "mm_internal.cuh"),
+    "stage": ("mm_llg.cu", "mm_fields.cuh", "mm_rk.cuh", "mm_ff.cuh", "mm_internal.cuh"),
 }
 FAMILY = {"xfwd": "demag", "yfwd": "demag", "zconv": "demag", "yinv": "demag", "xinv": "demag", "stage": "stage"}
 # kernel-name prefixes of each timed class as ncu reports them
-NCU_NAMES = {"xfwd": "k_xfwd", "yfwd": "k_cols", "yinv": "k_cols", "zconv": "k_zconv", "xinv": "k_xinv",
+NCU_NAMES = {"xfwd": "k_xfwd", "yfwd": "k_cols", "yinv": "k_cols", "zconv": ("k_zconv", "k_zline"), "xinv": "k_xinv",
              "stage": "k_stage"}
 
 
