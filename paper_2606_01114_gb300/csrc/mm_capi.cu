@@ -539,13 +539,18 @@ int mm_relax(mm_ctx* ctx, void* m, double t_max, double torque_tol, long max_ste
         const long room = max_steps - (long)c->steps;
         const int batch = room < kCheck ? (int)room : kCheck;
         // The first trial's first stage is the state whose demag field the
-        // torque was taken with.  The host stays two trials ahead of the
-        // device and stops when the end time is reached: the batch used to
-        // run to its end, with every field evaluation of up to nine trials
-        // that change nothing (100x25x1 FP64 to 8 ps: 4.03 -> 3.23 ms).
+        // torque was taken with.  Where the end time may come inside the batch
+        // the host stays two trials ahead of the device and stops when it is
+        // reached: run to its end, the batch spent every field evaluation of up
+        // to nine trials that change nothing (100x25x1 FP64 to 8 ps: 4.03 ->
+        // 3.23 ms).  Steps grow at most five-fold each, in the first batch from
+        // the first step on and later by little: batches whose steps would have
+        // to be five times the next one are enqueued whole, so that a thread
+        // that is preempted does not leave the device idle.
+        const bool watch = c->steps < kCheck || c->t_max - c->t <= 5.0 * batch * c->dt;
         *ctx->mark = 0;
         for (int k = 0; k < batch; ++k, ++attempts) {
-            if (k >= 2 && trials_over(ctx, k - 1)) break;
+            if (watch && k >= 2 && trials_over(ctx, k - 1)) break;
             if ((rc = trial(ctx, m, MM_RKF45, k == 0, ctx->mark, k + 1))) return rc;
         }
     }
