@@ -130,6 +130,12 @@ def source_hash(kernel):
     return h.hexdigest()[:16]
 
 
+def traffic_key(precision, fft_mode):
+    """The name under which a mode's captures are stored: the plain passes
+    under the precision, any other mode (kernels of its own) under its name."""
+    return precision if fft_mode == "fp32" else fft_mode
+
+
 def ncu_traffic(kernel, precision):
     """DRAM bytes per launch of ``kernel`` from the committed ncu summary, or
     None when the kernel's sources changed since the counters were taken."""
@@ -565,7 +571,7 @@ def measure_f64(mm, w, stream, steps, warmup, peak, peak_src, alu, e2e_steps, cu
         r = run.timed(k_steps, stream)
         kt = r["kt"]
         dom = max(TIMED, key=lambda k: kt[k][0])
-        hbm = hbm_roofline(dom, kt, n, 8, peak, peak_src, "f64")
+        hbm = hbm_roofline(dom, kt, n, 8, peak, peak_src, traffic_key("f64", "ff" if mode else "fp32"))
         if name == "ff":
             fp32 = alu["fp32_fma_tflops"]
             roof = fp32 / 2.0 / FF_INSTR_PER_FLOP
@@ -832,7 +838,7 @@ def run_ours(args):
     rate = acc_all * N / (ms_max / 1e3) / 1e6
 
     peak, peak_src = load_peaks()
-    roofline = hbm_roofline(dom, kt_run, n, s, peak, peak_src, args.precision)
+    roofline = hbm_roofline(dom, kt_run, n, s, peak, peak_src, traffic_key(args.precision, args.fft_mode))
     extras = rank == 0 and world == 1 and not args.no_extras
     alu = measure_alu() if extras or prec == mm.MM_F64 else None
     if prec == mm.MM_F64 and algorithmic_flops(dom, n):
@@ -937,7 +943,7 @@ def run_ours(args):
 def main():
     args = parse()
     if args.ingest_ncu:
-        return ingest_ncu(args.ingest_ncu, args.precision, "film512 512x512x16 " + args.precision.upper())
+        return ingest_ncu(args.ingest_ncu, traffic_key(args.precision, args.fft_mode), "film512 512x512x16 " + args.precision.upper())
     if args.impl == "reference":
         return run_reference(args)
     return run_ours(args)

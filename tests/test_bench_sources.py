@@ -48,3 +48,11 @@ def test_the_register_z_pass_is_taken_for_the_z_pass(tmp_path, monkeypatch):
     assert bench.ingest_ncu(str(tmp_path / "raw.csv"), "ff", "film512 test") == 0
     t = json.load(open(tmp_path / "profiles" / "traffic.json"))
     assert t["zconv/ff"]["bytes_per_launch"] == 600 * 10 ** 6
+
+
+def test_a_mode_does_not_report_the_plain_passes_traffic(monkeypatch):
+    monkeypatch.setattr(bench, "source_hash", lambda k: "same")
+    monkeypatch.setattr(bench.json, "load", lambda f: {"zconv/f32": {"bytes_per_launch": 1, "source_sha": "same"}})
+    t = {m: bench.hbm_roofline("zconv", {"zconv": (1.0, 1)}, (512, 512, 16), 4, 1.0, "x", bench.traffic_key("f32", m))["traffic"]
+         for m in ("fp32", "tf32", "bf16", "f4")}
+    assert t == {"fp32": 1.0, "tf32": None, "bf16": None, "f4": None}
