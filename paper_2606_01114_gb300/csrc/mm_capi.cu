@@ -357,11 +357,10 @@ int mm_init_mesh(mm_ctx** out, int nx, int ny, int nz, double dx, double dy, dou
     }
     // Contexts of the plane layout need the arrays of the [c][z][y][kx] passes
     // only in the fft modes; the octant of the 2n lengths comes from those
-    // passes' setup where the sides are powers of two, else from plane_setup.
-    auto p2 = [](int n) { return (n & (n - 1)) == 0; };
+    // passes' setup where the plan has these lengths, else from plane_setup.
     if (rc == MM_OK) rc = plane_plan(ctx);
     if (rc == MM_OK && !ctx->plane.on) rc = classic_prepare(ctx);
-    if (rc == MM_OK && ctx->plane.on && p2(nx) && p2(ny)) rc = octant_prepare(ctx);
+    if (rc == MM_OK && ctx->plane.on && ctx->plane.L == nx && ctx->plane.P == ctx->Py) rc = octant_prepare(ctx);
     if (rc == MM_OK && ctx->plane.on) rc = plane_setup(ctx);
     if (rc == MM_OK) rc = sync(ctx);
     ctx->circles.clear();

@@ -186,13 +186,12 @@ void plane_free(mm_ctx* ctx) {
 // Fills the plan's octant.  Same padded lengths as the [c][z][y][kx] passes
 // (powers of two): their octant, turned.  Otherwise the Newell tensor
 // transformed axis by axis from its definition; that also fills
-// ctx->newell_host and, on meshes with a side that is not a power of two, the
-// octant of the 2n lengths (mm_kspace_product reads it and must neither
-// allocate nor wait).
+// ctx->newell_host and the octant of the 2n lengths (mm_kspace_product reads it
+// and must neither allocate nor wait).
 int plane_setup(mm_ctx* ctx) {
     PlanePlan& p = ctx->plane;
     const int Pz2 = ctx->Pz2, Py2 = p.P / 2 + 1;
-    if (ctx->kern_ready && p.L == ctx->nx && p.P == ctx->Py) {
+    if (ctx->kern_ready) {
         const long n = kern_count(ctx);
         if (ctx->prec == MM_F64)
             k_octant_turn<double><<<blocks(n), 256, 0, ctx->stream>>>((const double*)ctx->kern, (double*)p.kern, p.K, Pz2,
@@ -207,7 +206,7 @@ int plane_setup(mm_ctx* ctx) {
     // lengths and kept frequencies of the plan, and of the 2n octant
     const int len[2][3] = {{2 * p.L, p.P, ctx->Pz}, {ctx->Px, ctx->Py, ctx->Pz}};
     const int m[2][3] = {{p.K, Py2, Pz2}, {ctx->Hx, ctx->Py2, Pz2}};
-    const int sets = ctx->kern_ready ? 1 : 2;
+    constexpr int sets = 2;
     std::vector<double> t;
     long off[2][3];
     for (int q = 0; q < sets; ++q)
@@ -218,7 +217,7 @@ int plane_setup(mm_ctx* ctx) {
                 for (int i = 0; i < len[q][a]; ++i) t.push_back(s ? -e[2 * i + 1] : e[2 * i]);   // cos, then sin
         }
     const long fsize = (long)(ctx->nx + 1) * (ctx->ny + 1) * (ctx->nz + 1);
-    const size_t K = sets > 1 ? std::max(p.K, ctx->Hx) : p.K, Y = sets > 1 ? std::max(Py2, ctx->Py2) : Py2;
+    const size_t K = std::max(p.K, ctx->Hx), Y = std::max(Py2, ctx->Py2);
     void *oct = nullptr, *fg = nullptr, *a1 = nullptr, *a2 = nullptr, *a3 = nullptr, *tab = nullptr;
     auto cleanup = [&]() {
         for (void* q : {oct, fg, a1, a2, a3, tab}) cudaFree(q);
@@ -227,7 +226,7 @@ int plane_setup(mm_ctx* ctx) {
     auto A = [&](void** q, size_t b) {
         if (rc == MM_OK) rc = dev_alloc(ctx, q, b);
     };
-    if (sets > 1) A(&ctx->kern, 6 * (size_t)Pz2 * ctx->Py2 * ctx->Hs * elem(ctx));
+    A(&ctx->kern, 6 * (size_t)Pz2 * ctx->Py2 * ctx->Hs * elem(ctx));
     A(&oct, sizeof(double) * 6 * ctx->N);
     A(&fg, sizeof(double2) * fsize);
     A(&a1, sizeof(double) * (size_t)ctx->nz * ctx->ny * K);

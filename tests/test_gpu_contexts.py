@@ -23,9 +23,10 @@ def _built():
 
 
 # both sides ragged and above 32 (a chirp-z length each at 2n), one odd side,
-# narrow sides, a power of two beside a ragged side, powers of two
+# narrow sides, a power of two beside a ragged side, powers of two with and
+# without a side below the shortest padded length
 @pytest.mark.parametrize("prec,tol", [("f64", 1e-12), ("f32", 1e-5)])
-@pytest.mark.parametrize("n", [(50, 37, 4), (9, 64, 2), (3, 5, 1), (48, 33, 16), (32, 16, 2)],
+@pytest.mark.parametrize("n", [(50, 37, 4), (9, 64, 2), (3, 5, 1), (48, 33, 16), (32, 16, 2), (2, 2, 1), (2, 16, 4), (16, 2, 1)],
                          ids=lambda n: "x".join(map(str, n)))
 def test_first_kspace_product_can_be_captured(n, prec, tol):
     """The product on the spectrum of a library transform is the demag field,
