@@ -28,9 +28,11 @@
  *   - Work is enqueued on the stream given at mm_init_mesh (or mm_set_stream).
  *     Calls that return host scalars (energies, torque, step errors) wait for
  *     that stream.  Calls on one context must not overlap on the host.
- *   - Mesh sizes: nx, ny any of 1..512 (sides that are not powers of two are
- *     padded to the next of {4, 5, 6, 8} 2^k of at least twice their length);
- *     nz 1 or a power of two up to 512.
+ *   - Mesh sizes: nx, ny any of 1..512, nz 1 or a power of two up to 512.  The
+ *     demag convolution pads a side n to 2 n where nx, ny are powers of two (at
+ *     least 4) or one of them is 1, else to the next of 8, 16, 32 and 40, 48,
+ *     64, 80, 96, 128, ... ({4, 5, 6} 2^k) of at least 2 n; what a plan pads is
+ *     not visible in any result or array.
  *   - Every function returns MM_OK (0) or a negative MM_ERR_* code;
  *     mm_last_error() then describes the failure.  A failed call leaves the
  *     caller's buffers in an unspecified state but the context usable, except
@@ -57,14 +59,16 @@ enum {
     MM_ERR_DT_UNDERFLOW = -4, /* RKF45 shrank dt below the floor (1e-20 s) */
     MM_ERR_NOT_CONVERGED = -5,/* relax() hit max_steps before torque or t_max */
     MM_ERR_TIMEOUT = -6,      /* a bounded device wait gave up */
-    MM_ERR_NOMEM = -7         /* device allocation failed in mm_init_mesh */
+    MM_ERR_NOMEM = -7         /* device allocation failed (mm_init_mesh and the calls named there) */
 };
 
 /* Create a context for an nx x ny x nz mesh of dx x dy x dz cells.
  * Computes the Newell tensor on the device (double-double arithmetic),
  * transforms it and keeps its real k-space octant at the path precision;
- * allocates every scratch buffer the hot path needs (no allocation happens
- * after this call).  Material defaults: Ms = 8e5, A = 1.3e-11, alpha = 0.02,
+ * allocates every scratch buffer the hot path needs.  After this call only
+ * these allocate: mm_set_fft_mode (the first time a mode is set), the first
+ * mm_llg_step_host and the first adjoint call on the context, and
+ * mm_rk4_trajectory_vjp for the duration of the call.  Material defaults: Ms = 8e5, A = 1.3e-11, alpha = 0.02,
  * Ku = 0, u = z, no external field.
  *   out        receives the context (host pointer to a host pointer)
  *   precision  MM_F32 or MM_F64
@@ -121,8 +125,10 @@ int mm_set_dmi(mm_ctx* ctx, double D, int type);
 int mm_set_stt(mm_ctx* ctx, double J, double P, double Lambda, double eps_prime, const double p[3], double d);
 
 /* H = demagnetisation field of m (Eq. 4), both device [3][nz][ny][nx].
- * FP32 contexts with ny = 256 or 512, or nx = 512, run some passes fed by
- * the copy engine (TMA) with bounded waits; a wait that gives up raises
+ * FP32 contexts of power-of-two sides with ny = 256 or 512, or nx = 512, whose
+ * planes do not fit the plane layout (nz >= 16, or the largest with nz = 8), run
+ * some passes fed by the copy engine (TMA) with bounded waits; a wait that
+ * gives up raises
  * TIMEOUT in the device status, which mm_llg_step, mm_relax and
  * mm_minimize_bb report (no GPU fault is involved). */
 int mm_demag_field(mm_ctx* ctx, const void* m, void* H);
@@ -207,7 +213,10 @@ const char* mm_last_error(const mm_ctx* ctx);
  * points), for launch accounting. */
 long mm_kernel_launches(const mm_ctx* ctx);
 
-/* Kernel classes for per-kernel timing. */
+/* Kernel classes for per-kernel timing.  Where y forward, z and y inverse are
+ * one kernel (small and middling meshes) that kernel counts under ZCONV, and
+ * where the x passes are part of the stage or of the effective field (small
+ * FP32 meshes) they count under STAGE or REDUCE. */
 enum {
     MM_K_XFWD = 0,   /* demag pass 1: x real-to-complex, pruned          */
     MM_K_YFWD = 1,   /* demag pass 2: y forward, pruned input             */
@@ -337,16 +346,20 @@ int mm_dft32_tc(const void* in, void* out, long nlines, int mode, int direction,
  * for uniform Ms and A without DMI or STT, the LLG stage kernel as well
  * (its renormalisation finished in float64); m, Ms, H, the stage slopes and
  * everything else stay float64 arrays; the padded sizes Px, Py, Pz must be
- * powers of two.  Setting it allocates float-float
- * copies of the Newell octant and twiddle tables (6 (Pz/2+1)(Py/2+1) Hs x 8
- * bytes plus the tables), kept until mm_destroy.
+ * powers of two.  Setting it allocates float-float copies of the Newell octant
+ * the mode reads (8 bytes a value: 6 (Pz/2+1)(Py/2+1) Hs values, or as many in
+ * the plane layout) and of the twiddle tables.
  * MM_F32 context with ny = 512 and nz = 16: MM_FFT_F4 = the y forward pass,
  * the z transform with the tensor product and the y inverse pass fused into
  * one pass over kx planes, each held on chip by a cluster of four CTAs (the
  * 3-pass thin-film variant: the spectrum crosses HBM once between the x
  * passes instead of three times); setting it allocates a copy of the octant
  * laid out per kx plane (Hx x 4 x 6 x (Pz/2+1) x 256 floats) and a twiddle
- * table, kept until mm_destroy.
+ * table.
+ * A context whose plain passes run in the plane layout also allocates, the
+ * first time a mode needs them, the two spectrum buffers and the transform
+ * tables of the streaming passes.  What a mode allocates is kept until
+ * mm_destroy; setting a mode may wait for the stream.
  * Errors: INVALID_ARG (unknown mode, mode not valid for the context's
  * precision or mesh), NOMEM/CUDA (allocation or setup). */
 int mm_set_fft_mode(mm_ctx* ctx, int mode);

@@ -106,9 +106,10 @@ __device__ __forceinline__ V3<T> field_cell(const Params<T>& p, const T* __restr
 // 3 B lines a block: component c of row r0 + b is line c B + b.  STAGE: g and
 // ctl; otherwise the effective field to H.  folded: A / Ms is in the axis
 // constants of p already (uniform material: one rounding a bond fewer).
-// MAXT: the bound, not the block.  512 keeps the kernel at 128 registers, two
-// blocks of 256 threads to an SM; at 384 it took 130 to 132, one block, and more
-// rows than SMs went in two waves (300x300x1 21.3 us a stage, at 128 15.4).
+// MAXT: the bound, not the block.  512 keeps the stage within 128 registers (112
+// to 116 but for the longest rows), two blocks of 256 threads to an SM; at 384 it
+// took 130 to 132, one block, and more rows than SMs went in two waves
+// (300x300x1 21.3 us a stage, now 15.4).
 template <typename T, int L1, int L2, bool STAGE, int MAXT>
 __global__ void __launch_bounds__(MAXT)
     k_px_cell(PC<T>* __restrict__ buf, long R, Params<T> p, bool folded, int lgB, T scale, const PC<T>* __restrict__ twL,
